@@ -21,6 +21,9 @@
 // phase and gains its new one: over all translations the two exchanged
 // pixels cancel, over a sample of translations they need not.
 //
+// Segments of up to 255 pixels are evaluated from bit planes (lpf_swap.cu);
+// the walks here serve longer ones.
+//
 // Work split: blocks = (vector chunk) x (candidate stride); each block stages
 // the extended cell once (one bulk copy of a copy built per call in global
 // memory) and loops over its candidates.  Error changes are summed per
@@ -32,6 +35,7 @@
 
 #include "lpf_delta.cuh"
 #include "lpf_state.hpp"
+#include "lpf_swap.hpp"
 
 namespace lpf {
 
@@ -98,7 +102,7 @@ __global__ void __launch_bounds__(kDeltaThreads, 3) delta_kernel(const uint8_t* 
       if (partial) {
         float s = 0.0f;
         for (int w = 0; w < kDeltaWarps; ++w) s += warp_acc[w];
-        partial[(int64_t)k * g.n_chunks + ch] = s;
+        partial[(int64_t)ch * K + k] = s;
       }
       if (!skip) { delta_mark(sm, a, 1, g); delta_mark(sm, b, 0, g); }
     }
@@ -107,10 +111,8 @@ __global__ void __launch_bounds__(kDeltaThreads, 3) delta_kernel(const uint8_t* 
 }
 
 // Phase-0 count of S(v) + (x, y) for every canonical vector and translation,
-// from the extended cell (0/1 bytes), at delta_z_index in the sheared layout
-// (SHEARED, g.shear set) or the unsheared one.  Blocks stage the cell once
-// and take vectors at the grid stride; threads take translations.
-template <bool SHEARED>
+// from the extended cell (0/1 bytes), at delta_z_index.  Blocks stage the
+// cell once and take vectors at the grid stride; threads take translations.
 __global__ void __launch_bounds__(kDeltaThreads) z_init_kernel(const uint8_t* __restrict__ ext, DeltaArgs g,
                                                                uint8_t* __restrict__ z, int* __restrict__ status) {
   extern __shared__ __align__(16) uint8_t sm[];
@@ -125,7 +127,7 @@ __global__ void __launch_bounds__(kDeltaThreads) z_init_kernel(const uint8_t* __
     const int o0 = __ldg(g.dptr + v), L1 = __ldg(g.dptr + v + 1) - o0;
     int dx, dy;
     delta_vector(g, v, dx, dy);
-    const int m = SHEARED ? __ldg(g.shear + v) : 0;
+    const int m = __ldg(g.shear + v);
     uint8_t* zv = z + (int64_t)v * hw;
     for (int p = threadIdx.x; p < hw; p += blockDim.x) {
       // p runs over the vector's layout (delta_z_index)
@@ -139,51 +141,20 @@ __global__ void __launch_bounds__(kDeltaThreads) z_init_kernel(const uint8_t* __
   }
 }
 
-// Count changes (and error changes) of K candidates from the phase-0 counts
-// g.z: no staged cell, no block barriers -- a warp takes one candidate at a
-// time (candidates k = warp index over the grid's y extent, strided) and all
-// vectors of its block's chunk, in vector order, and writes that chunk's
-// partial error change.
-__global__ void __launch_bounds__(kDeltaThreads) delta_lookup_kernel(const uint8_t* __restrict__ img, DeltaArgs g,
-                                                                     const int32_t* __restrict__ pairs, int K,
-                                                                     int32_t* __restrict__ dcounts,
-                                                                     float* __restrict__ partial,
-                                                                     int* __restrict__ status) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int ch = blockIdx.x;
-  const int v0 = g.chunk[ch], v1 = g.chunk[ch + 1];
-  const int npix = g.H * g.W;
-  const int stride = gridDim.y * kDeltaWarps;
-  for (int k = blockIdx.y * kDeltaWarps + warp; k < K; k += stride) {
-    int a = pairs[2 * k], b = pairs[2 * k + 1];
-    int skip = 0;
-    if (a < 0 || b < 0 || a >= npix || b >= npix) {
-      skip = 1;
-      if (lane == 0) atomicOr(status, 2);
-    } else if ((img[a] != 0) == (img[b] != 0)) {
-      skip = 1;                                   // same phase (or a == b): identity
-    } else if (img[a] == 0) {
-      const int t = a; a = b; b = t;              // a holds phase 1
-    }
-    int32_t* dk = dcounts ? dcounts + (int64_t)k * 2 * g.n_canon : nullptr;
-    float acc = 0.0f;
-    if (skip) {
-      if (dk)
-        for (int v = v0 + lane; v < v1; v += 32) { dk[v] = 0; dk[g.n_canon + v] = 0; }
-    } else {
-      // the warp's own pass over the chunk: v0, v0 + 1, ... (one warp, so
-      // "warp 0 of 1" in the helper's striding)
-      acc = delta_lookup_vectors_warp(g, a, b, v0, v1, lane, dk, delta_terms_global(g));
-    }
-    if (lane == 0 && partial) partial[(int64_t)k * g.n_chunks + ch] = acc;
-  }
-}
-
-// de[k] = sum over chunks of partial[k][c], in chunk order.
+// de[k] = sum over chunks of partial[c][k], in chunk order; 32 loads in
+// flight per thread (a chain of adds behind single loads took 28 us for 4096
+// candidates and 456 chunks).
 __global__ void delta_reduce_kernel(const float* __restrict__ partial, int n_chunks, int K, float* __restrict__ de) {
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < K; k += gridDim.x * blockDim.x) {
     float s = 0.0f;
-    for (int c = 0; c < n_chunks; ++c) s += partial[(int64_t)k * n_chunks + c];
+    for (int c0 = 0; c0 < n_chunks; c0 += 32) {
+      float v[32];
+#pragma unroll
+      for (int u = 0; u < 32; ++u) v[u] = c0 + u < n_chunks ? partial[(int64_t)(c0 + u) * K + k] : 0.0f;
+#pragma unroll
+      for (int u = 0; u < 32; ++u)
+        if (c0 + u < n_chunks) s += v[u];
+    }
     de[k] = s;
   }
 }
@@ -315,11 +286,8 @@ int delta_prepare(lpf_paths* p, int H, int W, int K) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(delta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    optin - (int)fa.sharedSizeBytes);
     cudaFuncAttributes fz;
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fz, z_init_kernel<true>);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(z_init_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   optin - (int)fz.sharedSizeBytes);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fz, z_init_kernel<false>);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(z_init_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fz, z_init_kernel);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(z_init_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    optin - (int)fz.sharedSizeBytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sa_batch_kernel_entry(), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    optin - (int)fs.sharedSizeBytes);
@@ -327,7 +295,9 @@ int delta_prepare(lpf_paths* p, int H, int W, int K) {
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    optin - (int)fp.sharedSizeBytes);
     if (e != cudaSuccess) return set_cuda_error(e);
-    g_delta_max_smem = optin - (int)std::max(std::max(fa.sharedSizeBytes, fs.sharedSizeBytes), fp.sharedSizeBytes);
+    int max_static = (int)std::max(std::max(fa.sharedSizeBytes, fs.sharedSizeBytes), fp.sharedSizeBytes);
+    if (int rc = swap_planes_attributes(optin, &max_static)) return rc;
+    g_delta_max_smem = optin - max_static;
   }
   const size_t ext = (((size_t)delta_row_stride(W, p->host.rx) * (H + 2 * p->host.ry)) + 15) & ~size_t(15);
   if ((int64_t)ext > g_delta_max_smem) return LPF_EUNSUPPORTED;
@@ -398,21 +368,9 @@ size_t delta_z_bytes(const lpf_paths* p, int H, int W) {
   return b <= kZBudget ? b : 0;
 }
 
-int delta_z_prepare(lpf_paths* p, int H, int W) {
-  const size_t need = delta_z_bytes(p, H, W);
-  if (need > p->z_cap) {
-    if (p->d_z) { cudaDeviceSynchronize(); cudaFree(p->d_z); p->d_z = nullptr; p->z_cap = 0; }
-    cudaError_t e = cudaMalloc(&p->d_z, need);
-    if (e != cudaSuccess) return set_cuda_error(e);
-    p->z_cap = need;
-  }
-  return LPF_OK;
-}
-
 void z_init_launch(const uint8_t* ext, const DeltaArgs& g, uint8_t* z, int* status, cudaStream_t s) {
   const int blocks = (int)std::min<int64_t>(g.n_canon, 2 * (int64_t)(g_sms > 0 ? g_sms : 152));
-  if (g.shear) z_init_kernel<true><<<blocks, kDeltaThreads, g.ext_bytes, s>>>(ext, g, z, status);
-  else z_init_kernel<false><<<blocks, kDeltaThreads, g.ext_bytes, s>>>(ext, g, z, status);
+  z_init_kernel<<<blocks, kDeltaThreads, g.ext_bytes, s>>>(ext, g, z, status);
 }
 
 int delta_swap_run(const uint8_t* img_dev, int32_t H, int32_t W, lpf_paths* paths, const int32_t* pairs_dev,
@@ -435,40 +393,24 @@ int delta_swap_run(const uint8_t* img_dev, int32_t H, int32_t W, lpf_paths* path
   g.phase_mask = phase_mask;
   g.sel_ext = sel_ext;
   if (inv_norm > 0.0f) g.inv_norm = inv_norm;
-  {
+  float* partial = de_dev ? paths->d_partial : nullptr;
+  if (swap_planes_apply(paths)) {
+    rc = swap_planes_run(img_dev, paths, pairs_dev, K, dcounts_dev, partial, g, s);
+    if (rc) return rc;
+  } else {
+    // segments over 255 pixels: early-exit walks
     const int blocks = (int)std::min<int64_t>((g.ext_bytes + 255) / 256, 4096);
     build_ext_kernel<<<blocks, 256, 0, s>>>(img_dev, H, W, g.rx, g.ry, g.We, g.He, g.ext_bytes, paths->d_ext,
                                             paths->checked ? paths->d_status : nullptr);
-  }
-  dim3 grid(g.n_chunks, delta_stride(g.n_chunks, K));
-  // Phase-0 counts of every (vector, translation) when they fit the budget:
-  // count changes by lookups; otherwise by walks.
-  if (delta_z_bytes(paths, H, W) > 0) {
-    rc = delta_z_prepare(paths, H, W);
-    if (rc) return rc;
-    g.z = paths->d_z;
-    // unsheared counts: this call reads every candidate's lookups from an L2
-    // that holds z, and is bound by instruction issue, not by the sectors
-    // each warp touches (the annealer's sheared layout costs it 5 more
-    // instructions per lookup)
-    g.shear = nullptr;
-    z_init_launch(paths->d_ext, g, g.z, paths->d_status, s);
-    if (paths->ev_start) cudaEventRecord(paths->ev_start, s);
-    // a warp per candidate: enough candidate groups of 16 for a few warps per SM slot
-    grid.y = (unsigned)std::max(1, std::min((K + kDeltaWarps - 1) / kDeltaWarps,
-                                            (8 * (g_sms > 0 ? g_sms : 152) + g.n_chunks - 1) / g.n_chunks));
-    delta_lookup_kernel<<<grid, kDeltaThreads, 0, s>>>(img_dev, g, pairs_dev, K, dcounts_dev,
-                                                       de_dev ? paths->d_partial : nullptr, paths->d_status);
-    if (paths->ev_stop) cudaEventRecord(paths->ev_stop, s);
-  } else {
+    const dim3 grid(g.n_chunks, delta_stride(g.n_chunks, K));
     if (paths->ev_start) cudaEventRecord(paths->ev_start, s);
     delta_kernel<<<grid, kDeltaThreads, g.ext_bytes, s>>>(img_dev, paths->d_ext, g, pairs_dev, K, dcounts_dev,
-                                                          de_dev ? paths->d_partial : nullptr, paths->d_status);
+                                                          partial, paths->d_status);
     if (paths->ev_stop) cudaEventRecord(paths->ev_stop, s);
   }
   if (de_dev) {
-    const int blocks = std::min((K + 255) / 256, 1024);
-    delta_reduce_kernel<<<blocks, 256, 0, s>>>(paths->d_partial, g.n_chunks, K, de_dev);
+    const int blocks = std::min((K + 31) / 32, 4096);
+    delta_reduce_kernel<<<blocks, 32, 0, s>>>(paths->d_partial, g.n_chunks, K, de_dev);
   }
   return set_cuda_error(cudaGetLastError());
 }

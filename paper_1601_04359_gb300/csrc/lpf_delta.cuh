@@ -33,7 +33,7 @@ struct DeltaArgs {
   int max_chunk_entries;        // segment pixels of the largest chunk
   const uint8_t* sel_ext;       // selected start translations, extended layout (null: all)
   float inv_norm;               // descriptor = count * inv_norm (1/(H W), or 1/N selected)
-  // Phase-0 counts (see delta_lookup_vectors_strided): byte
+  // Phase-0 counts (see delta_chunk_lookup): byte
   // v H W + delta_z_index(v, x, y) of z = number of phase-0 pixels of
   // S(v) + (x, y), one byte per canonical vector and translation; null:
   // count changes by walks.  off16: the segments' pixel offsets
@@ -41,7 +41,7 @@ struct DeltaArgs {
   uint8_t* z;
   const int16_t* off16;
   const int16_t* vec16;         // canonical vectors (dx, dy) as int16 pairs
-  const int32_t* shear;         // their delta_shear, or null: z unsheared
+  const int32_t* shear;         // their delta_shear
 };
 
 // Where a walk finds the target and the current count of vector v for the
@@ -228,9 +228,8 @@ __device__ __forceinline__ int delta_wrap(const DeltaArgs& g, int t, int n) {
   return ((t % n) + n) % n;
 }
 
-// Index of translation (x, y) in z_v (m = delta_shear of v, or 0 for the
-// unsheared layout: rows of W bytes for x-major vectors, columns of H bytes
-// for y-major ones).
+// Index of translation (x, y) in z_v (m = delta_shear of v; 0 for vectors
+// along an axis: rows of W bytes, or columns of H bytes for y-major ones).
 __device__ __forceinline__ int delta_z_index(const DeltaArgs& g, int dx, int dy, int m, int x, int y) {
   const bool ymajor = dy > (dx < 0 ? -dx : dx);
   if (m == 0) return ymajor ? x * g.H + y : y * g.W + x;
@@ -279,95 +278,6 @@ __device__ __forceinline__ bool delta_on_segment(const DeltaArgs& g, int o0, int
     return g.off16[2 * (o0 + k) + 1] == uy;
   }
   return g.off16[2 * (o0 + uy)] == ux;      // y-major: pixel k at sy = k
-}
-
-// Same contract as delta_walk_vectors (a phase 1, b phase 0; the warp's
-// vectors v = v0, v0 + vstep, ...; lane 0 writes and returns), from the
-// phase-0 counts g.z in the unsheared layout (g.shear null).
-__device__ __forceinline__ float delta_lookup_vectors_strided(const DeltaArgs& g, int a, int b, int v0, int v1,
-                                                              int vstep, int lane, int32_t* dcounts_k,
-                                                              const DeltaTerms& dt);
-
-// One warp over all vectors v0 <= v < v1 (in order); lane 0 returns.
-__device__ __forceinline__ float delta_lookup_vectors_warp(const DeltaArgs& g, int a, int b, int v0, int v1,
-                                                           int lane, int32_t* dcounts_k, const DeltaTerms& dt) {
-  return delta_lookup_vectors_strided(g, a, b, v0, v1, 1, lane, dcounts_k, dt);
-}
-
-// Vectors v = v0, v0 + vstep, ... < v1.
-__device__ __forceinline__ float delta_lookup_vectors_strided(const DeltaArgs& g, int a, int b, int v0, int v1,
-                                                              int vstep, int lane, int32_t* dcounts_k,
-                                                              const DeltaTerms& dt) {
-  float acc = 0.0f;
-  const float invN = g.inv_norm;
-  const int W = g.W, H = g.H;
-  const int ay = a / W, ax = a - ay * W, by = b / W, bx = b - by * W;
-  const int64_t hw = (int64_t)H * W;
-  for (int v = v0; v < v1; v += vstep) {
-    const int o0 = __ldg(g.dptr + v);
-    const int L1 = __ldg(g.dptr + v + 1) - o0;
-    int dx, dy;
-    delta_vector(g, v, dx, dy);
-    const uint8_t* zv = g.z + (int64_t)v * hw;
-    int d0 = 0, d1 = 0;
-    // four lookups per lane in flight: offsets, then counts, then the tests
-    for (int t0 = 0; t0 < 2 * L1; t0 += 128) {
-      int xs[4], ys[4], zs[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int t = t0 + 32 * u + lane;
-        const int side = t >= L1;
-        const int i = t < 2 * L1 ? (side ? t - L1 : t) : 0;
-        const short2 s2 = reinterpret_cast<const short2*>(g.off16)[o0 + i];
-        int x = (side ? bx : ax) - s2.x, y = (side ? by : ay) - s2.y;
-        xs[u] = x < 0 ? x + W : (x >= W ? x - W : x);
-        ys[u] = y < 0 ? y + H : (y >= H ? y - H : y);
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)  // read at L2 (the annealer updates z in place)
-        zs[u] = t0 + 32 * u + lane < 2 * L1 ? __ldcg(zv + delta_z_index(g, dx, dy, 0, xs[u], ys[u])) : -1;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int t = t0 + 32 * u + lane;
-        if (t >= 2 * L1) continue;
-        const int x = xs[u], y = ys[u], z = zs[u];
-        if (g.sel_ext && !g.sel_ext[(y + g.ry) * g.We + (x + g.rx)]) continue;  // start not sampled
-        if (t < L1) {
-          if (z == 0) d1 -= 1;
-          if (z == L1 - 1 && !delta_on_segment(g, o0, dx, dy, x, y, bx, by)) d0 += 1;
-        } else {
-          if (z == L1) d0 -= 1;
-          if (z == 1 && !delta_on_segment(g, o0, dx, dy, x, y, ax, ay)) d1 += 1;
-        }
-      }
-    }
-    // one reduction for both phases: |d0|, |d1| <= 2 L1 < 2^15 per vector
-    int dp = d0 + d1 * 65536;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) dp += __shfl_xor_sync(0xffffffffu, dp, o);
-    d0 = (int)(short)(dp & 0xffff);
-    d1 = (dp - d0) / 65536;
-    if (lane == 0) {
-      if (dcounts_k) {
-        dcounts_k[v] = d0;
-        dcounts_k[g.n_canon + v] = d1;
-      }
-      if (g.target && (d0 | d1)) {
-        const int iv = v - dt.vbase;
-        if (d0 && (g.phase_mask & 1)) {
-          const float dd = dt.t[0][iv] - (float)dt.c[0][iv] * invN;
-          const float x = (float)d0 * invN;
-          acc += x * (x - 2.0f * dd);
-        }
-        if (d1 && (g.phase_mask & 2)) {
-          const float dd = dt.t[1][iv] - (float)dt.c[1][iv] * invN;
-          const float x = (float)d1 * invN;
-          acc += x * (x - 2.0f * dd);
-        }
-      }
-    }
-  }
-  return acc;
 }
 
 // A block's vector chunk for the block-wide lookups of the persistent
@@ -446,8 +356,7 @@ __device__ __forceinline__ void chunk_entry(const DeltaArgs& g, const ChunkTable
 // a (phase 1) and b (phase 0), from the phase-0 counts z, with the chunk's
 // 2 (L + 1) lookups per vector spread evenly over all threads of the block:
 // entry e < E looks at the translation through a of pixel e, entry E + e at
-// the one through b; kChunkUnroll lookups per thread in flight.  The tests
-// are those of delta_lookup_vectors_strided.  When the block has at most
+// the one through b; kChunkUnroll lookups per thread in flight.  When the block has at most
 // kChunkUnroll entries per thread, *held receives the thread's counts as
 // read (one byte each) and held_zi their offsets in z, for
 // delta_chunk_apply_held; else *held is 0.  Every thread calls it; thread 0

@@ -115,8 +115,8 @@ struct lpf_paths {
   size_t ext_cap = 0;
   uint32_t* d_sel = nullptr;     // work area: packed translation selection (Monte-Carlo variant)
   size_t sel_cap = 0;            // words
-  uint8_t* d_z = nullptr;        // work area: phase-0 counts per (vector, translation) of swap deltas
-  size_t z_cap = 0;              // bytes
+  uint32_t* d_swap = nullptr;    // work area of the bit-plane swap deltas: packed rows, selection, candidates
+  size_t swap_cap = 0;           // words
   int checked = 0;               // 1: kernels that read the image flag pixels other than 0 or 1
   int selftest = 0;              // 1: walks wait for bytes no copy delivers (failure-detection test)
 };
@@ -150,11 +150,10 @@ inline size_t persistent_smem_bytes(size_t ext_bytes, int mv, int me) {
          (size_t)me * (4 + 2) + 16;
 }
 int delta_max_smem();
-// Phase-0 counts for swap deltas by lookup: bytes for an H x W cell (0: not
-// used -- too long segments or too much memory), allocation in the handle,
-// and the kernel that fills them from an extended cell.
+// The annealer's phase-0 counts per translation: bytes for an H x W cell (0:
+// not used -- too long segments or too much memory), and the kernel that
+// fills them from an extended cell.
 size_t delta_z_bytes(const lpf_paths* p, int H, int W);
-int delta_z_prepare(lpf_paths* p, int H, int W);
 void z_init_launch(const uint8_t* ext, const DeltaArgs& g, uint8_t* z, int* status, cudaStream_t s);
 // The annealing batch kernel of the lineal-path objective (lpf_sa.cu), for
 // attribute and occupancy queries.
