@@ -141,21 +141,34 @@ __global__ void __launch_bounds__(kDeltaThreads) z_init_kernel(const uint8_t* __
   }
 }
 
-// de[k] = sum over chunks of partial[c][k], in chunk order; 32 loads in
-// flight per thread (a chain of adds behind single loads took 28 us for 4096
-// candidates and 456 chunks).
-__global__ void delta_reduce_kernel(const float* __restrict__ partial, int n_chunks, int K, float* __restrict__ de) {
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < K; k += gridDim.x * blockDim.x) {
+// de[k] = sum over chunks of partial[c][k], in chunk order.  A block's 8
+// warps load the chunks of 32 candidates into shared memory, one warp adds
+// them up: the loads of 256 chunks are in flight together (a chain of adds
+// behind one thread's own loads took 19 us for 64 candidates and 306 chunks).
+constexpr int kReduceChunks = 256;
+__global__ void __launch_bounds__(256) delta_reduce_kernel(const float* __restrict__ partial, int n_chunks, int K,
+                                                           float* __restrict__ de) {
+  __shared__ float s_p[kReduceChunks][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int k0 = blockIdx.x * 32; k0 < K; k0 += gridDim.x * 32) {
+    const int k = k0 + lane;
     float s = 0.0f;
-    for (int c0 = 0; c0 < n_chunks; c0 += 32) {
-      float v[32];
+    for (int c0 = 0; c0 < n_chunks; c0 += kReduceChunks) {
+      const int nc = min(kReduceChunks, n_chunks - c0);
+      float v[kReduceChunks / 8];
 #pragma unroll
-      for (int u = 0; u < 32; ++u) v[u] = c0 + u < n_chunks ? partial[(int64_t)(c0 + u) * K + k] : 0.0f;
+      for (int u = 0; u < kReduceChunks / 8; ++u)
+        v[u] = k < K && warp + 8 * u < nc ? partial[(int64_t)(c0 + warp + 8 * u) * K + k] : 0.0f;
 #pragma unroll
-      for (int u = 0; u < 32; ++u)
-        if (c0 + u < n_chunks) s += v[u];
+      for (int u = 0; u < kReduceChunks / 8; ++u) s_p[warp + 8 * u][lane] = v[u];
+      __syncthreads();
+      if (warp == 0) {
+#pragma unroll 8
+        for (int c = 0; c < nc; ++c) s += s_p[c][lane];
+      }
+      __syncthreads();
     }
-    de[k] = s;
+    if (warp == 0 && k < K) de[k] = s;
   }
 }
 
@@ -410,7 +423,7 @@ int delta_swap_run(const uint8_t* img_dev, int32_t H, int32_t W, lpf_paths* path
   }
   if (de_dev) {
     const int blocks = std::min((K + 31) / 32, 4096);
-    delta_reduce_kernel<<<blocks, 32, 0, s>>>(paths->d_partial, g.n_chunks, K, de_dev);
+    delta_reduce_kernel<<<blocks, 256, 0, s>>>(paths->d_partial, g.n_chunks, K, de_dev);
   }
   return set_cuda_error(cudaGetLastError());
 }

@@ -58,6 +58,7 @@ struct SwapArgs {
   int words;               // H * nw; word (y, j) of a plane is y + H j
   int tg, G;               // threads per vector, vectors side by side in a block
   int nmax;                // longest segment, rounded up to 8
+  uint32_t inv_H, inv_S;   // ceil(2^32 / H), ceil(2^32 / S): i / H = umulhi(i, inv_H) while i H < 2^32
   const uint32_t* img;     // packed rows: (H + ry) rows of S words, bit e = column (e - r32) mod W
   const uint32_t* sel;     // selected start translations by word, or null
   const int32_t* dptr;
@@ -72,12 +73,15 @@ struct SwapArgs {
   float inv_norm;
 };
 
+// i / n by the reciprocal inv = ceil(2^32 / n) (n > 1; n = 1 has inv = 0).
+__device__ __forceinline__ int fast_div(int i, uint32_t inv) { return inv ? (int)__umulhi((uint32_t)i, inv) : i; }
+
 static int swap_img_words(int H, int ry, int S) { return ((H + ry) * S + 3) & ~3; }
 
 // Bytes of dynamic shared memory.
 static size_t swap_smem(const SwapArgs& g, bool many) {
   const size_t img = (size_t)swap_img_words(g.H, g.ry, g.S) * 4;
-  const size_t group = many ? (size_t)g.words * 64 + 3 * img : (size_t)g.words * 12;
+  const size_t group = many ? (size_t)g.words * 64 + 4 * img : (size_t)((g.words * 3 + 3) & ~3) * 4;
   return img + (size_t)((g.S + 3) & ~3) * 4 + (size_t)g.G * (group + (size_t)2 * g.nmax * 4) + 64;
 }
 
@@ -172,19 +176,61 @@ __device__ __forceinline__ void to_bytes(BitCounter& q) {
   }
 }
 
-// 32 columns from column p0 (periodic) of row y of a plane without halo.
-__device__ __forceinline__ uint32_t plane_columns(const uint32_t* plane, int y, int p0, int H, int W, int nw) {
+// Columns p0 .. p0 + 31 (periodic) of row y of the three planes without
+// halo (plane_words apart).
+__device__ __forceinline__ uint4 plane_columns(const uint32_t* planes, int plane_words, int y, int p0, int H, int W,
+                                               int nw) {
+  uint32_t w[3];
   if (W >= 32) {
     const int j = p0 >> 5, have = W - p0;
-    const uint32_t hi = j + 1 < nw ? plane[y + H * (j + 1)] : 0u;
-    uint32_t w = __funnelshift_r(plane[y + H * j], hi, p0 & 31);
-    if (have < 32) w = (w & ((1u << have) - 1u)) | plane[y] << have;
-    return w;
+    const uint32_t* at = planes + y + H * j;
+    const bool more = j + 1 < nw;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) w[q] = __funnelshift_r(at[q * plane_words], more ? at[q * plane_words + H] : 0u, p0 & 31);
+    if (have < 32) {
+#pragma unroll
+      for (int q = 0; q < 3; ++q) w[q] = (w[q] & ((1u << have) - 1u)) | planes[q * plane_words + y] << have;
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const uint32_t row = planes[q * plane_words + y];  // W bits
+      w[q] = row >> p0;
+      for (int have = W - p0; have < 32; have += W) w[q] |= row << have;
+    }
   }
-  const uint32_t row = plane[y];  // W bits
-  uint32_t w = row >> p0;
-  for (int have = W - p0; have < 32; have += W) w |= row << have;
-  return w;
+  return make_uint4(w[0], w[1], w[2], 0u);
+}
+
+// Eight segment pixels (entries s[0..7], the last 8 - live of them absent)
+// added to the counters of 32 pixels; p: the word's planes with halo.
+template <bool FULL>
+__device__ __forceinline__ void add_pixels(BitCounter& cu, BitCounter& cn, const uint4* p, const uint32_t* s,
+                                           uint32_t chi, int live) {
+  uint32_t du[8], dn[8];
+  const uint4 s0 = *reinterpret_cast<const uint4*>(s), s1 = *reinterpret_cast<const uint4*>(s + 4);
+  const uint32_t e[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    du[t] = dn[t] = 0u;
+    if (FULL || t < live) {
+      const uint4* q = p + (e[t] >> 5);
+      const uint4 lo = q[0], hi = q[1];
+      du[t] = __funnelshift_r(lo.x, hi.x, e[t]);
+      const uint32_t x1 = __funnelshift_r(lo.y, hi.y, e[t]), x0 = __funnelshift_r(lo.z, hi.z, e[t]);
+      dn[t] = (chi & x1) | (~chi & x0);
+    }
+  }
+  add8(cu, du);
+  add8(cn, dn);
+}
+
+// One segment pixel of the walk: c = the image under 32 translations.
+__device__ __forceinline__ void walk_masks(uint32_t c, uint32_t& all1, uint32_t& all0, uint32_t& one1, uint32_t& one0) {
+  one1 = (all0 & c) | (one1 & ~c);
+  one0 = (all1 & ~c) | (one0 & c);
+  all0 &= ~c;
+  all1 &= c;
 }
 
 // Whether a segment of vector (dx, dy) can hold two pixels q and q + (ddx,
@@ -260,11 +306,11 @@ __global__ void __launch_bounds__(kSwapThreads, 3) swap_kernel(SwapArgs g, const
   uint32_t* s_img = smw;
   int* s_col = reinterpret_cast<int*>(s_img + img_words);  // column (32 k - r32) mod W
   uint32_t* s_groups = reinterpret_cast<uint32_t*>(s_col + ((S + 3) & ~3));
-  const int plane_words = MANY ? g.words * 16 : g.words * 3;  // planes; many: then the sum tables
-  const int group_words = plane_words + (MANY ? 3 * ext_words : 0) + 2 * g.nmax;
+  const int plane_words = MANY ? g.words * 16 : (g.words * 3 + 3) & ~3;  // planes; many: then the sum tables
+  const int group_words = plane_words + (MANY ? 4 * ext_words : 0) + 2 * g.nmax;
   const int gi = tid / g.tg, gt = tid - gi * g.tg;
   uint32_t* base = s_groups + gi * group_words;
-  uint32_t* ext = base + plane_words;
+  uint4* ext = reinterpret_cast<uint4*>(base + plane_words);  // {U, X1, X0, 0} by word of the packed rows
   uint32_t* segA = base + group_words - 2 * g.nmax;
   uint32_t* segB = segA + g.nmax;
 
@@ -304,7 +350,7 @@ __global__ void __launch_bounds__(kSwapThreads, 3) swap_kernel(SwapArgs g, const
         for (int h = 0; h < 2; ++h) {
           const int w = w0 + h * g.tg;
           const bool on = w < g.words;
-          const int j = on ? w / H : 0, y = on ? w - j * H : 0;
+          const int j = on ? fast_div(w, g.inv_H) : 0, y = on ? w - j * H : 0;
           const int rem = W - 32 * j;
           uint32_t m = on ? (rem >= 32 ? 0xffffffffu : (1u << rem) - 1u) : 0u;
           if (g.sel) m &= __ldg(g.sel + y + H * j);
@@ -312,22 +358,32 @@ __global__ void __launch_bounds__(kSwapThreads, 3) swap_kernel(SwapArgs g, const
           one1[h] = one0[h] = 0u;
           p[h] = s_img + y * S + j;
         }
-        for (int i = 0; i < n; ++i) {
+        int i = 0;
+        bool live = true;
+        for (; live && i + 8 <= n; i += 8) {  // eight pixels, their loads together, then one vote
+          const uint4 s0 = *reinterpret_cast<const uint4*>(segA + i), s1 = *reinterpret_cast<const uint4*>(segA + i + 4);
+          const uint32_t e[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
+          uint32_t any = 0;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            uint32_t c[8];
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+              const uint32_t* q = p[h] + (e[t] >> 5);
+              c[t] = __funnelshift_r(q[0], q[1], e[t]);
+            }
+#pragma unroll
+            for (int t = 0; t < 8; ++t) walk_masks(c[t], all1[h], all0[h], one1[h], one0[h]);
+            any |= all1[h] | all0[h] | one1[h] | one0[h];
+          }
+          live = __any_sync(0xffffffffu, any != 0);  // else nothing is left for the rest of the segment
+        }
+        for (; live && i < n; ++i) {
           const uint32_t s = segA[i];
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             const uint32_t* q = p[h] + (s >> 5);
-            const uint32_t c = __funnelshift_r(q[0], q[1], s);
-            one1[h] = (all0[h] & c) | (one1[h] & ~c);
-            one0[h] = (all1[h] & ~c) | (one0[h] & c);
-            all0[h] &= ~c;
-            all1[h] &= c;
-          }
-          if ((i & 7) == 7) {
-            uint32_t any = 0;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) any |= all1[h] | all0[h] | one1[h] | one0[h];
-            if (!__any_sync(0xffffffffu, any != 0)) break;  // nothing left for the rest of the segment
+            walk_masks(__funnelshift_r(q[0], q[1], s), all1[h], all0[h], one1[h], one0[h]);
           }
         }
         uint32_t any = 0;
@@ -349,37 +405,23 @@ __global__ void __launch_bounds__(kSwapThreads, 3) swap_kernel(SwapArgs g, const
       // ---- the planes with their periodic halo
       if (mine && s_any[gi])
         for (int e = gt; e < (H + g.ry) * S; e += g.tg) {
-          const int r = e / S, k = e - r * S;
-          const int y = r >= g.ry ? r - g.ry : r - g.ry + H, p0 = s_col[k];
-#pragma unroll
-          for (int q = 0; q < 3; ++q)
-            ext[q * ext_words + e] = plane_columns(base + q * g.words, y, p0, H, W, g.nw);
+          const int r = fast_div(e, g.inv_S), k = e - r * S;
+          const int y = r >= g.ry ? r - g.ry : r - g.ry + H;
+          ext[e] = plane_columns(base, g.words, y, s_col[k], H, W, g.nw);
         }
       __syncthreads();
       // ---- sums along the segment for every pixel, into byte tables (over the planes without halo)
       if (mine && s_any[gi])
         for (int w = gt; w < g.words; w += g.tg) {
-          const int j = w / H, y = w - j * H;
+          const int j = fast_div(w, g.inv_H), y = w - j * H;
           const uint32_t chi = s_img[y * S + j + (g.r32 >> 5)];
-          const uint32_t* p = ext + y * S + j;
+          const uint4* p = ext + y * S + j;
           BitCounter cu, cn;
 #pragma unroll
           for (int q = 0; q < 8; ++q) cu.c[q] = cn.c[q] = 0u;
-          for (int i0 = 0; i0 < n; i0 += 8) {
-            uint32_t du[8], dn[8];
-#pragma unroll
-            for (int t = 0; t < 8; ++t) {
-              const uint32_t s = i0 + t < n ? segB[i0 + t] : 0u;
-              const uint32_t* q = p + (s >> 5);
-              const uint32_t u = __funnelshift_r(q[0], q[1], s);
-              const uint32_t a = __funnelshift_r(q[ext_words], q[ext_words + 1], s);
-              const uint32_t b = __funnelshift_r(q[2 * ext_words], q[2 * ext_words + 1], s);
-              du[t] = i0 + t < n ? u : 0u;
-              dn[t] = i0 + t < n ? (chi & a) | (~chi & b) : 0u;
-            }
-            add8(cu, du);
-            add8(cn, dn);
-          }
+          int i = 0;
+          for (; i + 8 <= n; i += 8) add_pixels<true>(cu, cn, p, segB + i, chi, 8);
+          if (i < n) add_pixels<false>(cu, cn, p, segB + i, chi, n - i);
           to_bytes(cu);
           to_bytes(cn);
           uint4* tu = reinterpret_cast<uint4*>(base + 8 * w);
@@ -408,13 +450,16 @@ __global__ void __launch_bounds__(kSwapThreads, 3) swap_kernel(SwapArgs g, const
       if (MANY) {
         const uint8_t* tu = reinterpret_cast<const uint8_t*>(pl);
         const uint8_t* tn = tu + 32 * g.words;
-        const uint32_t* pext = pl + plane_words;
+        const uint4* pext = reinterpret_cast<const uint4*>(pl + plane_words);
+        uint4 next = make_uint4(0u, 0u, 0u, 0u);  // the next round's candidate, loaded a round ahead
+        if (tid < K) next = __ldg(reinterpret_cast<const uint4*>(cand) + tid);
         for (int k0 = warp * 32; k0 < K; k0 += nthr) {
           const int k = k0 + lane;
           int d0 = 0, d1 = 0;
+          const uint4 c = next;
+          next = make_uint4(0u, 0u, 0u, 0u);
+          if (k + nthr < K) next = __ldg(reinterpret_cast<const uint4*>(cand) + k + nthr);
           if (any) {
-            uint4 c = make_uint4(0u, 0u, 0u, 0u);
-            if (k < K) c = __ldg(reinterpret_cast<const uint4*>(cand) + k);
             const bool swap = c.z != c.w;
             bool share = false;
             int ax = 0, ay = 0, bx = 0, by = 0;
@@ -438,10 +483,10 @@ __global__ void __launch_bounds__(kSwapThreads, 3) swap_kernel(SwapArgs g, const
                 const short2 s = __ldg(sq + i);
                 int x, y;
                 swap_start(px, py, s, H, W, x, y);
-                if ((pext[ext_words + (y + g.ry) * S + ((x + g.r32) >> 5)] >> (x & 31)) & 1u)
+                if ((pext[(y + g.ry) * S + ((x + g.r32) >> 5)].y >> (x & 31)) & 1u)
                   both += swap_on_segment(sq, dv.x, dv.y, x, y, qx, qy, H, W);
                 swap_start(qx, qy, s, H, W, x, y);
-                if ((pext[2 * ext_words + (y + g.ry) * S + ((x + g.r32) >> 5)] >> (x & 31)) & 1u)
+                if ((pext[(y + g.ry) * S + ((x + g.r32) >> 5)].z >> (x & 31)) & 1u)
                   both += (int)swap_on_segment(sq, dv.x, dv.y, x, y, px, py, H, W) << 16;
               }
               both = __reduce_add_sync(0xffffffffu, both);
@@ -514,6 +559,8 @@ int swap_planes_run(const uint8_t* img_dev, lpf_paths* paths, const int32_t* pai
   g.S = (g.nw + ((g.r32 + d.rx) >> 5) + 1) | 1;  // odd: 32 rows in 32 banks
   g.words = g.H * g.nw;
   g.nmax = (std::max(d.rx, d.ry) + 1 + 7) & ~7;
+  g.inv_H = g.H > 1 ? (uint32_t)(((uint64_t(1) << 32) + g.H - 1) / g.H) : 0u;
+  g.inv_S = g.S > 1 ? (uint32_t)(((uint64_t(1) << 32) + g.S - 1) / g.S) : 0u;
   g.dptr = d.dptr;
   g.off16 = d.off16;
   g.vec16 = d.vec16;
