@@ -60,6 +60,7 @@ struct BatchDesc {
   int H, W, S, nw, G, BB, T, r32, rows, nbg, n_pieces, bg0;
   int rs, cs;               // the side's pixel (r, c) is img[r rs + c cs]
   int up;                   // packed row y holds the side's row (y - up) mod H
+  int gather;               // 1: the window is wide enough to re-deal masks (walk_unit)
   int primary;              // 1: side 0 (zeroes and mirrors the image's counts)
   uint32_t band_bytes;
 };
@@ -109,14 +110,14 @@ __global__ void batch_mirror_kernel(const BatchDesc* __restrict__ d) {
 }
 
 // One unit; returns the pixels the warp walked.
-template <int T>
+template <int T, bool GATHER>
 __device__ __forceinline__ uint32_t batch_unit(const BatchDesc& b, int bg, int tile, int pi, const uint32_t* sm,
-                                               int lane) {
+                                               uint2* deal, int lane) {
   const int bl = tile / b.G, grp = tile - (tile / b.G) * b.G;
   const int y = (bg * b.BB + bl) * 32 + lane;
   const uint32_t* lane_base = sm + (bl * 32 + lane) * b.S + grp * T;
-  return walk_unit<T, false>(b.prog, b.piece[pi], b.piece[pi + 1], lane_base, y, b.H, b.W, b.nw, grp * T, nullptr,
-                             lane, b.counts, b.n_full, b.base);
+  return walk_unit<T, GATHER, false>(b.prog, b.piece[pi], b.piece[pi + 1], lane_base, b.gather ? deal : nullptr, y, b.H, b.W, b.nw, grp * T,
+                             nullptr, lane, b.counts, b.n_full, b.base);
 }
 
 // The walk of the slots whose images take T words per thread (one kernel per
@@ -124,16 +125,18 @@ __device__ __forceinline__ uint32_t batch_unit(const BatchDesc& b, int bg, int t
 // allocation and spill).  slot_ctr is this kernel's slot counter in ctl.
 // T >= 4 keeps its masks and the image's fields in up to 80 registers (3
 // blocks per SM; with 64 it spills, measured 3 % slower on the 256 images).
-template <int T>
+template <int T, bool GATHER>
 __global__ void __launch_bounds__(kBatchThreads, (T >= 4 ? 3 : 4)) batch_walk_kernel(const BatchDesc* __restrict__ d,
                                                                    const BatchSlot* __restrict__ slots,
                                                                    int n_slots, int* __restrict__ ctl,
-                                                                   int slot_ctr,
+                                                                   int slot_ctr, uint32_t deal_at,
                                                                    unsigned long long* __restrict__ executed) {
   extern __shared__ __align__(16) uint32_t sm[];
   __shared__ __align__(8) uint64_t bar;
   __shared__ int s_abort, s_done, s_slot;
   __shared__ uint32_t s_walked[kBatchWarps];
+  // per warp, behind the staged rows: masks being re-dealt (deal_at = 0: no room, never)
+  uint2* deal = deal_at ? reinterpret_cast<uint2*>(reinterpret_cast<char*>(sm) + deal_at) + (threadIdx.x & ~31u) : nullptr;
   const int lane = threadIdx.x & 31;
   if (threadIdx.x == 0) { mbar_init(&bar, 1); s_abort = 0; }
   __syncthreads();
@@ -184,7 +187,7 @@ __global__ void __launch_bounds__(kBatchThreads, (T >= 4 ? 3 : 4)) batch_walk_ke
       u = __shfl_sync(0xffffffffu, u, 0);
       if (u >= units) break;
       const int tile = u % n_tiles, pi = u / n_tiles;
-      const uint32_t w = batch_unit<T>(b, sl.bg, tile, pi, sm, lane);
+      const uint32_t w = batch_unit<T, GATHER>(b, sl.bg, tile, pi, sm, deal, lane);
       if (lane == 0) s_walked[threadIdx.x >> 5] += w;
     }
     if (lane == 0 && s_walked[threadIdx.x >> 5])
@@ -200,23 +203,15 @@ __global__ void __launch_bounds__(kBatchThreads, (T >= 4 ? 3 : 4)) batch_walk_ke
 // T = 1 << k.
 static inline int t_index(int T) { return T == 1 ? 0 : T == 2 ? 1 : T == 4 ? 2 : 3; }
 
-static const void* batch_walk_fn(int k) {
-  switch (k) {
-    case 0: return (const void*)batch_walk_kernel<1>;
-    case 1: return (const void*)batch_walk_kernel<2>;
-    case 2: return (const void*)batch_walk_kernel<4>;
-    default: return (const void*)batch_walk_kernel<8>;
-  }
-}
+using BatchWalkFn = void (*)(const BatchDesc*, const BatchSlot*, int, int*, int, uint32_t, unsigned long long*);
 
-static void batch_walk_launch(int k, int blocks, uint32_t smem, cudaStream_t s, const BatchDesc* d,
-                              const BatchSlot* slots, int n_slots, int* ctl, int slot_ctr,
-                              unsigned long long* executed) {
+// gather: some image of the kernel has a window wide enough to re-deal masks.
+static BatchWalkFn batch_walk_fn(int k, bool gather) {
   switch (k) {
-    case 0: batch_walk_kernel<1><<<blocks, kBatchThreads, smem, s>>>(d, slots, n_slots, ctl, slot_ctr, executed); break;
-    case 1: batch_walk_kernel<2><<<blocks, kBatchThreads, smem, s>>>(d, slots, n_slots, ctl, slot_ctr, executed); break;
-    case 2: batch_walk_kernel<4><<<blocks, kBatchThreads, smem, s>>>(d, slots, n_slots, ctl, slot_ctr, executed); break;
-    default: batch_walk_kernel<8><<<blocks, kBatchThreads, smem, s>>>(d, slots, n_slots, ctl, slot_ctr, executed); break;
+    case 0: return batch_walk_kernel<1, false>;
+    case 1: return gather ? batch_walk_kernel<2, true> : batch_walk_kernel<2, false>;
+    case 2: return gather ? batch_walk_kernel<4, true> : batch_walk_kernel<4, false>;
+    default: return gather ? batch_walk_kernel<8, true> : batch_walk_kernel<8, false>;
   }
 }
 
@@ -280,6 +275,8 @@ struct lpf_batch {
   std::vector<lpf::Baked> baked;
   int desc_cap = 0;
   uint32_t max_band = 0;
+  uint32_t smem = 0, deal_at = 0;  // a walk block's dynamic shared memory, the re-deal entries in it (0: none)
+  bool gather_T[lpf::kBatchTs] = {false, false, false, false};  // per walk kernel: re-deals masks
   int max_pack = 0, max_full = 0;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
@@ -368,6 +365,7 @@ static int batch_build(lpf_batch* bt, const uint8_t* const* imgs, const int32_t*
       d.rs = side ? 1 : W[i];
       d.cs = side ? W[i] : 1;
       d.primary = side == 0;
+      d.gather = std::max(p->host.rx, p->host.ry) >= kGatherWindow;
       bt->desc.push_back(d);
       total_bg += g.nbg;
       bg_work.push_back((double)prog.n_pixel_words * g.G * g.BB * (g.T + 1));
@@ -416,9 +414,24 @@ static int batch_build(lpf_batch* bt, const uint8_t* const* imgs, const int32_t*
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   // each T's walk kernel: its shared-memory limit and resident blocks
+  bool gather = false;
+  for (bool& w : bt->gather_T) w = false;
+  for (const BatchDesc& d : bt->desc)
+    if (d.gather && d.T > 1) bt->gather_T[t_index(d.T)] = gather = true;
+  bt->smem = bt->max_band + (gather ? 8u * kBatchThreads : 0u);
+  for (int k = 0; k < kBatchTs && gather; ++k) {
+    cudaFuncAttributes fa;
+    if ((e = cudaFuncGetAttributes(&fa, batch_walk_fn(k, true))) != cudaSuccess) return set_cuda_error(e);
+    if ((int)bt->smem > optin - (int)fa.sharedSizeBytes) gather = false;
+  }
+  if (!gather) {  // no image wants it, or no room
+    bt->smem = bt->max_band;
+    for (bool& w : bt->gather_T) w = false;
+  }
+  bt->deal_at = bt->smem > bt->max_band ? bt->max_band : 0u;
   int resident_T[kBatchTs];
   for (int k = 0; k < kBatchTs; ++k) {
-    const void* fn = batch_walk_fn(k);
+    const BatchWalkFn fn = batch_walk_fn(k, bt->gather_T[k]);
     cudaFuncAttributes fa;
     if ((e = cudaFuncGetAttributes(&fa, fn)) != cudaSuccess) return set_cuda_error(e);
     const int max_dyn = optin - (int)fa.sharedSizeBytes;
@@ -426,7 +439,7 @@ static int batch_build(lpf_batch* bt, const uint8_t* const* imgs, const int32_t*
     if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dyn)) != cudaSuccess)
       return set_cuda_error(e);
     int per_sm = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBatchThreads, bt->max_band)) != cudaSuccess)
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBatchThreads, bt->smem)) != cudaSuccess)
       return set_cuda_error(e);
     resident_T[k] = std::max(1, per_sm) * sms;
   }
@@ -505,8 +518,8 @@ static void batch_enqueue(lpf_batch* bt, cudaStream_t s) {
       ks = bt->aux[n_fork];
       cudaStreamWaitEvent(ks, bt->ev_fork, 0);
     }
-    batch_walk_launch(k, bt->blocks_T[k], bt->max_band, ks, bt->d_desc, bt->d_slots + bt->slot_off[k], n,
-                      bt->d_ctl, kBatchCtlSlot + k, bt->d_exec);
+    batch_walk_fn(k, bt->gather_T[k])<<<bt->blocks_T[k], kBatchThreads, bt->smem, ks>>>(
+        bt->d_desc, bt->d_slots + bt->slot_off[k], n, bt->d_ctl, kBatchCtlSlot + k, bt->deal_at, bt->d_exec);
     if (!first) cudaEventRecord(bt->ev_join[n_fork++], ks);
     first = false;
   }

@@ -103,7 +103,12 @@ int make_sides(const Paths& paths, int H, int W, int T, int BB, Sides& s) {
     s.nbg += s.g[1].nbg;
     tiles = std::max(tiles, s.g[1].G * s.g[1].BB);
   }
-  s.threads = 32 * std::min(16, tiles);
+  // One warp per tile, at most 16; more (warps take units of any tile of the
+  // band group) where the staged rows let few blocks share an SM, up to the
+  // 32 warps that the registers allow.
+  const int fit = std::max(1, (228 * 1024) / (int)(s.band_bytes + 16 * 256 + 1024));
+  s.threads = 32 * std::min(16, std::max(tiles, 32 / fit));
+  s.gather = std::max(rx, ry) >= kGatherWindow;
   if (s.nbg > kMaxBandGroups) return LPF_EUNSUPPORTED;
   return LPF_OK;
 }
@@ -254,13 +259,17 @@ struct WalkSide {
   uint32_t band_bytes;
 };
 
+struct WalkSides {
+  WalkSide s[2];
+};
+
 // The units of band group lbg of side sd, pulled from its counter ctr until
 // none is left: unit u is the side's program piece u / n_tiles on tile
 // u % n_tiles (tile = one band and one group of T words, i.e. 32 rows x 32T
 // translations).  Returns the pixel words this warp ANDed.
-template <int T>
+template <int T, bool GATHER>
 __device__ __forceinline__ unsigned long long walk_band(const WalkSide& sd, int lbg, int* ctr, const uint32_t* sm,
-                                                        int lane, const uint4* __restrict__ prog,
+                                                        uint2* deal, int lane, const uint4* __restrict__ prog,
                                                         const uint32_t* __restrict__ piece,
                                                         unsigned long long* __restrict__ counts, int64_t n_full,
                                                         int64_t base) {
@@ -276,8 +285,8 @@ __device__ __forceinline__ unsigned long long walk_band(const WalkSide& sd, int 
     const int bl = tile / sd.G, grp = tile - bl * sd.G;
     const uint32_t* lane_base = sm + (bl * 32 + lane) * sd.S + grp * T;
     const int y = ((lbg % sd.nbg_s) * sd.BB + bl) * 32 + lane;  // translation row within the slice
-    executed += walk_unit<T>(prog, piece[pi], piece[pi + 1], lane_base, y, sd.H, sd.W, sd.nw, grp * T, sd.sel, lane,
-                             counts, n_full, base);
+    executed += walk_unit<T, GATHER>(prog, piece[pi], piece[pi + 1], lane_base, deal, y, sd.H, sd.W, sd.nw, grp * T, sd.sel,
+                             lane, counts, n_full, base);
   }
   return executed;
 }
@@ -293,17 +302,19 @@ __device__ __forceinline__ unsigned long long walk_band(const WalkSide& sd, int 
 // block barrier per move).  The launch bounds cap a thread at 64 registers
 // (two 512-thread blocks per SM), which keeps 32 warps resident per SM to
 // hide the latency of the shared-memory word loads.
-template <int T>
-__global__ void __launch_bounds__(512, 2) walk_kernel(WalkSide s0, WalkSide s1, const uint4* __restrict__ prog,
+template <int T, bool GATHER>
+__global__ void __launch_bounds__(512, 2) walk_kernel(const __grid_constant__ WalkSides ws, const uint4* __restrict__ prog,
                                                   const uint32_t* __restrict__ piece,
                                                   unsigned long long* __restrict__ counts, int64_t n_full,
-                                                  int64_t base, int* __restrict__ ctl, uint32_t extra_tx,
+                                                  int64_t base, int* __restrict__ ctl, uint32_t deal_at, uint32_t extra_tx,
                                                   uint32_t wait_rounds) {
   extern __shared__ __align__(16) uint32_t sm[];
   __shared__ __align__(8) uint64_t bar;
   __shared__ int s_abort, s_done;
+  // per warp, behind the staged rows: masks being re-dealt (deal_at = 0: no room, never)
+  uint2* deal = deal_at ? reinterpret_cast<uint2*>(reinterpret_cast<char*>(sm) + deal_at) + (threadIdx.x & ~31u) : nullptr;
   const int lane = threadIdx.x & 31;
-  const int n_bg = s0.nbg + s1.nbg;
+  const int n_bg = ws.s[0].nbg + ws.s[1].nbg;
   int* unit_ctr = ctl + kCtlUnits;
   if (threadIdx.x == 0) { mbar_init(&bar, 1); s_abort = 0; }
   __syncthreads();
@@ -313,12 +324,10 @@ __global__ void __launch_bounds__(512, 2) walk_kernel(WalkSide s0, WalkSide s1, 
 
   for (int k = 0; k < n_bg; ++k) {
     const int bg = (int)((blockIdx.x + (unsigned)k) % (unsigned)n_bg);
-    const bool side1 = bg >= s0.nbg;
-    const int lbg = side1 ? bg - s0.nbg : bg;
-    if (threadIdx.x == 0) {
-      const int units = side1 ? s1.G * s1.BB * s1.n_pieces : s0.G * s0.BB * s0.n_pieces;
-      s_done = *reinterpret_cast<volatile int*>(unit_ctr + bg) >= units;
-    }
+    const int side = bg >= ws.s[0].nbg;
+    const WalkSide& sd = ws.s[side];
+    const int lbg = side ? bg - ws.s[0].nbg : bg;
+    if (threadIdx.x == 0) s_done = *reinterpret_cast<volatile int*>(unit_ctr + bg) >= sd.G * sd.BB * sd.n_pieces;
     __syncthreads();
     if (s_done) {
       __syncthreads();  // s_done is rewritten next round
@@ -326,15 +335,11 @@ __global__ void __launch_bounds__(512, 2) walk_kernel(WalkSide s0, WalkSide s1, 
     }
     if (threadIdx.x == 0) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      const uint32_t bytes = side1 ? s1.band_bytes : s0.band_bytes;
       // (extra_tx > 0 only in the failure-detection self-test: bytes no copy delivers)
-      mbar_expect_tx(&bar, bytes + extra_tx);
+      mbar_expect_tx(&bar, sd.band_bytes + extra_tx);
       // band group lbg = slice lbg / nbg_s (volumes; images have one slice), band lbg % nbg_s
-      const int nbg_s = side1 ? s1.nbg_s : s0.nbg_s, BB = side1 ? s1.BB : s0.BB;
-      const size_t row0 = (size_t)(lbg / nbg_s) * (side1 ? s1.slice_rows : s0.slice_rows) +
-                          (size_t)(lbg % nbg_s) * 32 * BB;
-      const uint32_t* src = side1 ? s1.packed + row0 * s1.S : s0.packed + row0 * s0.S;
-      bulk_g2s(sm, src, bytes, &bar);
+      const size_t row0 = (size_t)(lbg / sd.nbg_s) * sd.slice_rows + (size_t)(lbg % sd.nbg_s) * 32 * sd.BB;
+      bulk_g2s(sm, sd.packed + row0 * sd.S, sd.band_bytes, &bar);
     }
     copy_pending = true;
     if (mbar_wait(&bar, parity, wait_rounds)) copy_pending = false;
@@ -342,8 +347,13 @@ __global__ void __launch_bounds__(512, 2) walk_kernel(WalkSide s0, WalkSide s1, 
     parity ^= 1u;
     __syncthreads();
     if (s_abort) break;
-    if (side1) executed += walk_band<T>(s1, lbg, unit_ctr + bg, sm, lane, prog, piece, counts, n_full, base);
-    else executed += walk_band<T>(s0, lbg, unit_ctr + bg, sm, lane, prog, piece, counts, n_full, base);
+    // One copy of the gathering walk serves both sides (two overflow the
+    // instruction cache: 270 instead of 205 us for the whole domain of
+    // 175x201); without it two copies, with the side's fields as constants,
+    // are the faster ones (18.4 and 18.9 us at 64x64, window 32).
+    if (GATHER) executed += walk_band<T, GATHER>(sd, lbg, unit_ctr + bg, sm, deal, lane, prog, piece, counts, n_full, base);
+    else if (side) executed += walk_band<T, GATHER>(ws.s[1], lbg, unit_ctr + bg, sm, deal, lane, prog, piece, counts, n_full, base);
+    else executed += walk_band<T, GATHER>(ws.s[0], lbg, unit_ctr + bg, sm, deal, lane, prog, piece, counts, n_full, base);
     __syncthreads();  // every warp is done with the staged band before it may be replaced
   }
   if (lane == 0) atomicAdd(reinterpret_cast<unsigned long long*>(ctl + kCtlExecuted), executed);
@@ -458,6 +468,18 @@ static int bake_sides(lpf_paths* p, const Sides& sd, bool standard, Baked& b) {
   return bake(p, prog0, sd.g[0], sd.n == 2 ? &prog1 : nullptr, sd.n == 2 ? &sd.g[1] : nullptr, b);
 }
 
+using WalkFn = void (*)(const WalkSides, const uint4*, const uint32_t*, unsigned long long*, int64_t, int64_t, int*,
+                        uint32_t, uint32_t, uint32_t);
+
+static WalkFn walk_fn(int T, bool gather) {
+  switch (T) {
+    case 1: return walk_kernel<1, false>;
+    case 2: return gather ? walk_kernel<2, true> : walk_kernel<2, false>;
+    case 4: return gather ? walk_kernel<4, true> : walk_kernel<4, false>;
+    default: return gather ? walk_kernel<8, true> : walk_kernel<8, false>;
+  }
+}
+
 static std::once_flag g_attr_once;
 static int g_attr_status = LPF_OK;
 static int g_max_dyn_smem = 0;  // dynamic shared memory a walk block may use
@@ -479,30 +501,29 @@ static void set_kernel_attributes() {
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) { g_attr_status = set_cuda_error(e); return; }
-  int rc = allow_smem(walk_kernel<1>, optin, g_max_dyn_smem);
-  if (!rc) rc = allow_smem(walk_kernel<2>, optin, g_max_dyn_smem);
-  if (!rc) rc = allow_smem(walk_kernel<4>, optin, g_max_dyn_smem);
-  if (!rc) rc = allow_smem(walk_kernel<8>, optin, g_max_dyn_smem);
+  int rc = LPF_OK;
+  for (int T : {1, 2, 4, 8})
+    for (bool gather : {false, true})
+      if (!rc) rc = allow_smem(walk_fn(T, gather), optin, g_max_dyn_smem);
   g_attr_status = rc;
 }
 
 static int g_num_sms = 0;
 
-template <int T>
-static int walk_blocks(const Sides& sd) {
-  int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, walk_kernel<T>, sd.threads, sd.band_bytes);
-  if (e != cudaSuccess) return -set_cuda_error(e);
-  return std::max(1, per_sm) * g_num_sms;
+// Dynamic shared memory of a walk block: the staged rows and, where masks
+// are re-dealt and it fits, 32 entries per warp for that.
+static uint32_t walk_smem(const Sides& sd) {
+  const uint32_t with = sd.band_bytes + 8u * (uint32_t)sd.threads;
+  return sd.gather && (int)with <= g_max_dyn_smem ? with : sd.band_bytes;
 }
 
 static int walk_blocks_for(const Sides& sd) {
-  switch (sd.g[0].T) {
-    case 1: return walk_blocks<1>(sd);
-    case 2: return walk_blocks<2>(sd);
-    case 4: return walk_blocks<4>(sd);
-    default: return walk_blocks<8>(sd);
-  }
+  int per_sm = 0;
+  const uint32_t smem = walk_smem(sd);
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, walk_fn(sd.g[0].T, smem > sd.band_bytes),
+                                                                sd.threads, smem);
+  if (e != cudaSuccess) return -set_cuda_error(e);
+  return std::max(1, per_sm) * g_num_sms;
 }
 
 static int num_sms() {
@@ -539,16 +560,13 @@ static void walk_sides(const Sides& sd, const Baked& b, const uint32_t* packed, 
 static void launch_walk(const Sides& sd, const Baked& b, const uint32_t* packed, const uint32_t* sel0,
                         const uint32_t* sel1, unsigned long long* c, int64_t n_full, int64_t base, int* ctl,
                         const lpf_paths* p, int blocks, cudaStream_t s) {
-  WalkSide w0, w1;
-  walk_sides(sd, b, packed, sel0, sel1, w0, w1);
+  WalkSides w;
+  walk_sides(sd, b, packed, sel0, sel1, w.s[0], w.s[1]);
   const uint4* prog = reinterpret_cast<const uint4*>(b.d_words);
+  const uint32_t smem = walk_smem(sd), deal_at = smem > sd.band_bytes ? sd.band_bytes : 0u;
   const uint32_t xt = selftest_extra_tx(p), wr = selftest_wait_rounds(p);
-  switch (sd.g[0].T) {
-    case 1: walk_kernel<1><<<blocks, sd.threads, sd.band_bytes, s>>>(w0, w1, prog, b.d_piece, c, n_full, base, ctl, xt, wr); break;
-    case 2: walk_kernel<2><<<blocks, sd.threads, sd.band_bytes, s>>>(w0, w1, prog, b.d_piece, c, n_full, base, ctl, xt, wr); break;
-    case 4: walk_kernel<4><<<blocks, sd.threads, sd.band_bytes, s>>>(w0, w1, prog, b.d_piece, c, n_full, base, ctl, xt, wr); break;
-    default: walk_kernel<8><<<blocks, sd.threads, sd.band_bytes, s>>>(w0, w1, prog, b.d_piece, c, n_full, base, ctl, xt, wr); break;
-  }
+  walk_fn(sd.g[0].T, deal_at != 0u)<<<blocks, sd.threads, smem, s>>>(w, prog, b.d_piece, c, n_full, base, ctl,
+                                                                     deal_at, xt, wr);
 }
 
 // Pack both sides of an image (one launch, one grid row per side), zeroing
@@ -714,6 +732,7 @@ static int run_full3(const uint8_t* vol, int D, int H, int W, lpf_paths* p, int6
   sd.packed_words = g.packed_words;
   sd.band_bytes = g.band_bytes;
   sd.nbg = g.nbg;
+  sd.gather = std::max(std::max(p->host.rx, p->host.ry), p->host.rz) >= kGatherWindow;
   // 16 warps per block whatever the band group's tile count: warps pull
   // units of any tile of the staged band group, and a volume's band group
   // (its slices with their rz halo) is large, so few blocks fit on an SM

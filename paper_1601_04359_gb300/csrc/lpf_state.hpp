@@ -56,7 +56,8 @@ struct Sides {
   size_t packed_words = 0;   // both sides
   uint32_t band_bytes = 0;   // the larger side's
   int nbg = 0;               // band groups of both sides
-  int threads = 0;           // walk block: one warp per tile of the larger side, at most 16
+  int threads = 0;           // walk block: at least one warp per tile of the larger side up to 16
+  bool gather = false;       // the walk re-deals masks (walk_unit)
 };
 int make_sides(const Paths& paths, int H, int W, int T, int BB, Sides& s);
 // The same for a D x H x W volume and window (rx, ry, rz).

@@ -30,8 +30,8 @@
 // one byte per vector and translation (136 MB at 128x128, window 64), filled
 // and read by 2n scattered lookups per candidate and vector.
 // Measured (error changes, a call): 4096 candidates on a 128x128 clustered
-// cell, window 64: 15.66 -> 0.94 ms; 64 candidates on a 50x50 cell, full
-// domain, with count changes: 0.300 -> 0.148 ms; the same bits.
+// cell, window 64: 15.66 -> 0.79 ms; 64 candidates on a 50x50 cell, full
+// domain, with count changes: 0.300 -> 0.113 ms; the same bits.
 //
 // Error changes are summed per (chunk, candidate) in vector order and then
 // over chunks in chunk order: bitwise reproducible.
