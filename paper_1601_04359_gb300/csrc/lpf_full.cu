@@ -113,6 +113,25 @@ int make_sides(const Paths& paths, int H, int W, int T, int BB, Sides& s) {
   return LPF_OK;
 }
 
+// The sides of n images of one size evaluated together: every side's packed
+// rows repeat per image, slice_rows apart (a 16-byte boundary: S is odd, so a
+// multiple of 4 rows), and its band groups are numbered image by image.
+static int stack_images(Sides& s, int n) {
+  int64_t nbg = 0;
+  for (int q = 0; q < s.n; ++q) {
+    Geometry& g = s.g[q];
+    g.slice_rows = (g.rows + 3) & ~3;
+    nbg += (int64_t)g.nbg_s * n;
+    g.nbg = g.nbg_s * n;
+    g.packed_words = (size_t)n * g.slice_rows * g.S + 4;
+  }
+  if (nbg > kMaxBandGroups) return LPF_EUNSUPPORTED;
+  s.off1 = (s.g[0].packed_words + 3) & ~size_t(3);
+  s.packed_words = s.n == 2 ? s.off1 + s.g[1].packed_words : s.g[0].packed_words;
+  s.nbg = (int)nbg;
+  return LPF_OK;
+}
+
 // Volume layout: packed row (z' * slice_rows + y'') holds image row
 // (y'' - ry) mod H of slice z' mod D, z' < D + rz; a block of band group
 // (z, b) stages rows z * slice_rows + 32 BB b onwards: its 32 BB
@@ -148,9 +167,10 @@ int make_geometry3(int D, int H, int W, int rx, int ry, int rz, int T, int BB, G
 struct PackSide {
   uint32_t* packed;
   int Ho, Wo, r32, S, rows, rs, cs, up;
+  int64_t slice_words;  // packed words from one image to the next (blockIdx.z)
 };
 
-// Packs side blockIdx.y.  Side 1 runs over its words column by column, so
+// Packs side blockIdx.y of image blockIdx.z.  Side 1 runs over its words column by column, so
 // that the threads of a warp read consecutive bytes of an image row.  Side
 // 0's blocks also zero the walk's n_zero64 counts and n_zero32 control words
 // (which would otherwise take two more launches).  pix_flag != null (checked
@@ -162,7 +182,9 @@ __global__ void pack_rows_kernel(const uint8_t* __restrict__ img, PackSide s0, P
   const PackSide ps = side1 ? s1 : s0;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (!side1) {
+  img += (int64_t)blockIdx.z * s0.Ho * s0.Wo;
+  uint32_t* packed = ps.packed + blockIdx.z * ps.slice_words;
+  if (!side1 && blockIdx.z == 0) {
     for (int64_t i = i0; i < n_zero64; i += stride) zero64[i] = 0ull;
     for (int64_t i = i0; i < n_zero32; i += stride) zero32[i] = 0;
   }
@@ -183,7 +205,7 @@ __global__ void pack_rows_kernel(const uint8_t* __restrict__ img, PackSide s0, P
       high |= v >> 1;
       if (++x == ps.Wo) x = 0;
     }
-    ps.packed[(int64_t)y * ps.S + k] = bits;
+    packed[(int64_t)y * ps.S + k] = bits;
   }
   if (pix_flag && high) atomicOr(pix_flag, kStatusPixel);
 }
@@ -257,6 +279,7 @@ struct WalkSide {
   int nbg, nbg_s, slice_rows;
   int piece0, n_pieces;
   uint32_t band_bytes;
+  int work_from;  // band groups whose work is reported (an ensemble: its last image's)
 };
 
 struct WalkSides {
@@ -306,11 +329,11 @@ template <int T, bool GATHER>
 __global__ void __launch_bounds__(512, 2) walk_kernel(const __grid_constant__ WalkSides ws, const uint4* __restrict__ prog,
                                                   const uint32_t* __restrict__ piece,
                                                   unsigned long long* __restrict__ counts, int64_t n_full,
-                                                  int64_t base, int* __restrict__ ctl, uint32_t deal_at, uint32_t extra_tx,
+                                                  int64_t base, int* __restrict__ ctl, uint32_t deal_at, int steal, uint32_t extra_tx,
                                                   uint32_t wait_rounds) {
   extern __shared__ __align__(16) uint32_t sm[];
   __shared__ __align__(8) uint64_t bar;
-  __shared__ int s_abort, s_done;
+  __shared__ int s_abort, s_next;
   // per warp, behind the staged rows: masks being re-dealt (deal_at = 0: no room, never)
   uint2* deal = deal_at ? reinterpret_cast<uint2*>(reinterpret_cast<char*>(sm) + deal_at) + (threadIdx.x & ~31u) : nullptr;
   const int lane = threadIdx.x & 31;
@@ -322,17 +345,34 @@ __global__ void __launch_bounds__(512, 2) walk_kernel(const __grid_constant__ Wa
   bool copy_pending = false;
   unsigned long long executed = 0;  // pixel words this warp ANDs
 
-  for (int k = 0; k < n_bg; ++k) {
+  for (int k = 0;; ++k) {
+    // The next band group with units left (the block's first one without
+    // asking): a warp looks at 32 counters at once -- one after the other,
+    // 128 band groups cost every block 0.1 ms at the end of a launch.
+    if (k > 0) {
+      if (!steal) break;  // (there are warps for every unit of every band group)
+      if (threadIdx.x < 32) {
+        int found = n_bg;
+        for (int k0 = k; k0 < n_bg && found == n_bg; k0 += 32) {
+          bool left = false;
+          if (k0 + lane < n_bg) {
+            const int bt = (int)((blockIdx.x + (unsigned)(k0 + lane)) % (unsigned)n_bg);
+            const WalkSide& st = ws.s[bt >= ws.s[0].nbg];
+            left = *reinterpret_cast<volatile int*>(unit_ctr + bt) < st.G * st.BB * st.n_pieces;
+          }
+          const uint32_t m = __ballot_sync(0xffffffffu, left);
+          if (m) found = k0 + __ffs(m) - 1;
+        }
+        if (lane == 0) s_next = found;
+      }
+      __syncthreads();
+      k = s_next;  // (rewritten only after the barrier at the end of the band group)
+      if (k >= n_bg) break;
+    }
     const int bg = (int)((blockIdx.x + (unsigned)k) % (unsigned)n_bg);
     const int side = bg >= ws.s[0].nbg;
     const WalkSide& sd = ws.s[side];
     const int lbg = side ? bg - ws.s[0].nbg : bg;
-    if (threadIdx.x == 0) s_done = *reinterpret_cast<volatile int*>(unit_ctr + bg) >= sd.G * sd.BB * sd.n_pieces;
-    __syncthreads();
-    if (s_done) {
-      __syncthreads();  // s_done is rewritten next round
-      continue;
-    }
     if (threadIdx.x == 0) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       // (extra_tx > 0 only in the failure-detection self-test: bytes no copy delivers)
@@ -351,9 +391,11 @@ __global__ void __launch_bounds__(512, 2) walk_kernel(const __grid_constant__ Wa
     // instruction cache: 270 instead of 205 us for the whole domain of
     // 175x201); without it two copies, with the side's fields as constants,
     // are the faster ones (18.4 and 18.9 us at 64x64, window 32).
-    if (GATHER) executed += walk_band<T, GATHER>(sd, lbg, unit_ctr + bg, sm, deal, lane, prog, piece, counts, n_full, base);
-    else if (side) executed += walk_band<T, GATHER>(ws.s[1], lbg, unit_ctr + bg, sm, deal, lane, prog, piece, counts, n_full, base);
-    else executed += walk_band<T, GATHER>(ws.s[0], lbg, unit_ctr + bg, sm, deal, lane, prog, piece, counts, n_full, base);
+    unsigned long long walked;
+    if (GATHER) walked = walk_band<T, GATHER>(sd, lbg, unit_ctr + bg, sm, deal, lane, prog, piece, counts, n_full, base);
+    else if (side) walked = walk_band<T, GATHER>(ws.s[1], lbg, unit_ctr + bg, sm, deal, lane, prog, piece, counts, n_full, base);
+    else walked = walk_band<T, GATHER>(ws.s[0], lbg, unit_ctr + bg, sm, deal, lane, prog, piece, counts, n_full, base);
+    if (lbg >= sd.work_from) executed += walked;
     __syncthreads();  // every warp is done with the staged band before it may be replaced
   }
   if (lane == 0) atomicAdd(reinterpret_cast<unsigned long long*>(ctl + kCtlExecuted), executed);
@@ -469,7 +511,7 @@ static int bake_sides(lpf_paths* p, const Sides& sd, bool standard, Baked& b) {
 }
 
 using WalkFn = void (*)(const WalkSides, const uint4*, const uint32_t*, unsigned long long*, int64_t, int64_t, int*,
-                        uint32_t, uint32_t, uint32_t);
+                        uint32_t, int, uint32_t, uint32_t);
 
 static WalkFn walk_fn(int T, bool gather) {
   switch (T) {
@@ -543,17 +585,18 @@ static uint32_t selftest_extra_tx(const lpf_paths* p) { return p->selftest ? 16u
 static uint32_t selftest_wait_rounds(const lpf_paths* p) { return p->selftest ? (1u << 16) : kWaitRounds; }
 
 // The walk's view of the sides: packed rows from `packed` (side 1 at
-// sd.off1), selections sel0/sel1 (or null), pieces from b.
+// sd.off1), selections sel0/sel1 (or null), pieces from b; work_from: report
+// the work of the last slice only (images; else all slices').
 static void walk_sides(const Sides& sd, const Baked& b, const uint32_t* packed, const uint32_t* sel0,
-                       const uint32_t* sel1, WalkSide& w0, WalkSide& w1) {
+                       const uint32_t* sel1, bool work_from, WalkSide& w0, WalkSide& w1) {
   const Geometry& g0 = sd.g[0];
   w0 = WalkSide{packed, sel0, g0.H, g0.W, g0.S, g0.nw, g0.G, g0.BB, g0.nbg, g0.nbg_s, g0.slice_rows,
-                0, b.n_pieces0, g0.band_bytes};
+                0, b.n_pieces0, g0.band_bytes, work_from ? g0.nbg - g0.nbg_s : 0};
   w1 = WalkSide{};
   if (sd.n == 2) {
     const Geometry& g1 = sd.g[1];
     w1 = WalkSide{packed + sd.off1, sel1, g1.H, g1.W, g1.S, g1.nw, g1.G, g1.BB, g1.nbg, g1.nbg_s, g1.slice_rows,
-                  b.n_pieces0, b.n_pieces - b.n_pieces0, g1.band_bytes};
+                  b.n_pieces0, b.n_pieces - b.n_pieces0, g1.band_bytes, work_from ? g1.nbg - g1.nbg_s : 0};
   }
 }
 
@@ -561,33 +604,44 @@ static void launch_walk(const Sides& sd, const Baked& b, const uint32_t* packed,
                         const uint32_t* sel1, unsigned long long* c, int64_t n_full, int64_t base, int* ctl,
                         const lpf_paths* p, int blocks, cudaStream_t s) {
   WalkSides w;
-  walk_sides(sd, b, packed, sel0, sel1, w.s[0], w.s[1]);
+  walk_sides(sd, b, packed, sel0, sel1, p->host.dims == 2, w.s[0], w.s[1]);
   const uint4* prog = reinterpret_cast<const uint4*>(b.d_words);
   const uint32_t smem = walk_smem(sd), deal_at = smem > sd.band_bytes ? sd.band_bytes : 0u;
   const uint32_t xt = selftest_extra_tx(p), wr = selftest_wait_rounds(p);
+  // Few units (small images): if the blocks that start on a band group have a
+  // warp for each of its units, no block has to look for another one.
+  int steal = 0;
+  for (const WalkSide& q : w.s)
+    if (q.nbg > 0 && (int64_t)(blocks / sd.nbg) * (sd.threads / 32) < (int64_t)q.G * q.BB * q.n_pieces) steal = 1;
   walk_fn(sd.g[0].T, deal_at != 0u)<<<blocks, sd.threads, smem, s>>>(w, prog, b.d_piece, c, n_full, base, ctl,
-                                                                     deal_at, xt, wr);
+                                                                     deal_at, steal, xt, wr);
 }
 
-// Pack both sides of an image (one launch, one grid row per side), zeroing
-// n_zero counts and the walk's control words 1.. of the sides' band groups.
+// Pack both sides of n_img images (one launch, one grid row per side and
+// image), zeroing n_zero counts and the walk's control words 1.. of the sides' band groups.
 static void launch_pack(const uint8_t* img, const Sides& sd, uint32_t* packed, int64_t* counts, int64_t n_zero,
-                        int* ctl, const lpf_paths* p, cudaStream_t s) {
+                        int* ctl, const lpf_paths* p, cudaStream_t s, int n_img = 1) {
   const Geometry& g0 = sd.g[0];
   const Geometry& g1 = sd.n == 2 ? sd.g[1] : sd.g[0];
-  const PackSide s0{packed, g0.H, g0.W, g0.r32, g0.S, g0.rows, g0.W, 1, 0};
-  const PackSide s1{packed + sd.off1, g1.H, g1.W, g1.r32, g1.S, g1.rows, 1, g0.W, g1.up};
+  const PackSide s0{packed, g0.H, g0.W, g0.r32, g0.S, g0.rows, g0.W, 1, 0,
+                    (int64_t)g0.slice_rows * g0.S};
+  const PackSide s1{packed + sd.off1, g1.H, g1.W, g1.r32, g1.S, g1.rows, 1, g0.W, g1.up,
+                    (int64_t)g1.slice_rows * g1.S};
   const int64_t total = std::max<int64_t>({(int64_t)g0.rows * g0.S, sd.n == 2 ? (int64_t)g1.rows * g1.S : 0, n_zero});
   const int pblocks = (int)std::min<int64_t>((total + 255) / 256, 4096);
-  pack_rows_kernel<<<dim3(pblocks, sd.n), 256, 0, s>>>(img, s0, s1, reinterpret_cast<unsigned long long*>(counts),
+  pack_rows_kernel<<<dim3(pblocks, sd.n, n_img), 256, 0, s>>>(img, s0, s1, reinterpret_cast<unsigned long long*>(counts),
                                                        n_zero, ctl + 1, kCtlUnits - 1 + sd.nbg,
                                                        p->checked ? ctl : nullptr);
 }
 
 // Enqueue one full evaluation with launch shape (T, BB) (<= 0: tuned or
 // default); `accumulate` adds to the counts instead of replacing them.
+// n_img > 1: n_img images one after another in memory, walked side by side as
+// the slices of one evaluation, their counts summed; mirror: fill the
+// non-canonical half.
 static int run_full(const uint8_t* img, int H, int W, lpf_paths* p, int64_t* counts, cudaStream_t s,
-                    bool standard, int T = 0, int BB = 0, const uint8_t* sel = nullptr, bool accumulate = false) {
+                    bool standard, int T = 0, int BB = 0, const uint8_t* sel = nullptr, bool accumulate = false,
+                    int n_img = 1, bool mirror = true) {
   if (!p || !img || !counts) return LPF_EINVAL;
   if (p->host.dims != 2) return LPF_EINVAL;  // a volume's handle: lpf_full_3d
   if (H < 1 || W < 1 || H > 8192 || W > 8192) return LPF_EINVAL;
@@ -604,10 +658,15 @@ static int run_full(const uint8_t* img, int H, int W, lpf_paths* p, int64_t* cou
   int rc = make_sides(p->host, H, W, T, BB, sd);
   if (rc) return rc;
   if ((int)sd.band_bytes > g_max_dyn_smem) return LPF_EUNSUPPORTED;
+  Sides one = sd;  // (the program is baked for the layout of a single image)
+  if (n_img > 1) {
+    rc = stack_images(sd, n_img);
+    if (rc) return rc;
+  }
   rc = ensure_device(p, sd.packed_words);
   if (rc) return rc;
   Baked& b = standard ? p->plain : p->tree;
-  rc = bake_sides(p, sd, standard, b);
+  rc = bake_sides(p, one, standard, b);
   if (rc) return rc;
   if ((rc = num_sms())) return rc;
   int blocks = walk_blocks_for(sd);
@@ -619,7 +678,7 @@ static int run_full(const uint8_t* img, int H, int W, lpf_paths* p, int64_t* cou
   cudaError_t e = cudaSuccess;
   // pack the rows; zero the counts (unless accumulating) and the work
   // counters (not the status flags)
-  launch_pack(img, sd, p->d_packed, counts, accumulate ? 0 : 2 * n_full, p->d_status, p, s);
+  launch_pack(img, sd, p->d_packed, counts, accumulate ? 0 : 2 * n_full, p->d_status, p, s, n_img);
   const uint32_t* sel0 = nullptr;
   const uint32_t* sel1 = nullptr;
   if (sel) {
@@ -644,17 +703,47 @@ static int run_full(const uint8_t* img, int H, int W, lpf_paths* p, int64_t* cou
   }
   unsigned long long* c = reinterpret_cast<unsigned long long*>(counts);
   // every warp walks every piece of its side
-  p->nominal_pixels = prog0.n_pixel_words * sd.g[0].nbg * sd.g[0].G * sd.g[0].BB;
-  if (sd.n == 2) p->nominal_pixels += prog1.n_pixel_words * sd.g[1].nbg * sd.g[1].G * sd.g[1].BB;
+  p->nominal_pixels = prog0.n_pixel_words * one.g[0].nbg * one.g[0].G * one.g[0].BB;
+  if (one.n == 2) p->nominal_pixels += prog1.n_pixel_words * one.g[1].nbg * one.g[1].G * one.g[1].BB;
   if (p->ev_start) cudaEventRecord(p->ev_start, s);
   launch_walk(sd, b, p->d_packed, sel0, sel1, c, n_full, base, p->d_status, p, blocks, s);
   if (p->ev_stop) cudaEventRecord(p->ev_stop, s);
-  if (n_full > 1) {
+  if (mirror && n_full > 1) {
     const int64_t n = 2 * (n_full - base - 1);
     const int mblocks = (int)std::min<int64_t>((n + 255) / 256, 4096);
     mirror_kernel<<<mblocks, 256, 0, s>>>(c, n_full, base);
   }
   return cuda_status(cudaGetLastError());
+}
+
+// Summed counts of n images: as many of them per set of launches as the work
+// area and the unit counters hold (one by one, 64 images of 100x128 take 64
+// times three launches that each leave most of the GPU idle: 2.55 ms).
+constexpr size_t kEnsembleWords = size_t(1) << 24;  // packed words (64 MiB)
+static int run_ensemble(const uint8_t* imgs, int n, int H, int W, lpf_paths* p, int64_t* counts, cudaStream_t s) {
+  int per = 1;
+  if (p && p->host.dims == 2 && H >= 1 && W >= 1 && H <= 8192 && W <= 8192 && p->host.rx < W && p->host.ry < H) {
+    int T = 0, BB = 0;
+    for (const Tuned& t : p->tuned)
+      if (t.H == H && t.W == W) { T = t.T; BB = t.BB; }
+    Sides sd;
+    if (make_sides(p->host, H, W, T, BB, sd) == LPF_OK)
+      per = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)n, kMaxBandGroups / sd.nbg, 65535,
+                                                         (int64_t)(kEnsembleWords / (sd.packed_words + 64))}));
+  }
+  for (int i = 0; i < n; i += per) {
+    const int m = std::min(per, n - i);
+    const uint8_t* img = imgs + (size_t)i * H * W;
+    const int rc = run_full(img, H, W, p, counts, s, false, 0, 0, nullptr, i > 0, m, i + m == n);
+    if (rc == LPF_ENOMEM && per > 1) {  // no room for the larger work area: one by one
+      (void)cudaGetLastError();
+      per = 1;
+      i -= 1;
+      continue;
+    }
+    if (rc) return rc;
+  }
+  return LPF_OK;
 }
 
 // Time every admissible (T, BB) for this image size and keep the fastest.
@@ -1023,14 +1112,7 @@ int lpf_full_mc(const uint8_t* img_dev, int32_t H, int32_t W, lpf_paths* paths, 
 int lpf_full_ensemble(const uint8_t* imgs_dev, int32_t n_img, int32_t H, int32_t W, lpf_paths* paths,
                       int64_t* counts_dev, lpf_stream_t stream) {
   if (!imgs_dev || n_img < 1) return LPF_EINVAL;
-  for (int32_t i = 0; i < n_img; ++i) {
-    // the non-canonical half is rewritten from the accumulated canonical
-    // half after every image, so the sum stays exact
-    const int rc = lpf::run_full(imgs_dev + (size_t)i * H * W, H, W, paths, counts_dev, (cudaStream_t)stream, false,
-                                 0, 0, nullptr, i > 0);
-    if (rc) return rc;
-  }
-  return LPF_OK;
+  return lpf::run_ensemble(imgs_dev, n_img, H, W, paths, counts_dev, (cudaStream_t)stream);
 }
 
 int lpf_full_standard(const uint8_t* img_dev, int32_t H, int32_t W, lpf_paths* paths, int64_t* counts_dev,
