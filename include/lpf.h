@@ -312,7 +312,8 @@ int lpf_delta_swap(const uint8_t *img_dev, int32_t H, int32_t W, lpf_paths *path
  * after another in imgs_dev (uint8 [n_img][H][W]), e.g. the parallel cuts of
  * a volume: the ensemble average over cuts of Sec. 6.3 is counts / (n_img *
  * H * W).  counts_dev: int64 [2][n_vec_full] as in lpf_full.  The images are
- * evaluated one after another on `stream` (each one pack and walk launch).
+ * evaluated side by side on `stream`, as many per pack and walk launch as the
+ * handle's work area holds (64 MiB of packed rows, or one image).
  * Errors: as lpf_full; n_img < 1 is LPF_EINVAL.
  */
 int lpf_full_ensemble(const uint8_t *imgs_dev, int32_t n_img, int32_t H, int32_t W, lpf_paths *paths,

@@ -503,11 +503,52 @@ static bool baked_for_sides(const Baked& b, const Sides& sd) {
          b.S1 == (sd.n == 2 ? sd.g[1].S : -1) && b.r32_1 == (sd.n == 2 ? sd.g[1].r32 : -1);
 }
 
-// Bake the image's programs (tree or plain) for the sides.
-static int bake_sides(lpf_paths* p, const Sides& sd, bool standard, Baked& b) {
-  const Program& prog0 = standard ? p->host.plain : p->host.tree;
-  const Program& prog1 = standard ? p->host.plain_t : p->host.tree_t;
-  return bake(p, prog0, sd.g[0], sd.n == 2 ? &prog1 : nullptr, sd.n == 2 ? &sd.g[1] : nullptr, b);
+static int g_num_sms = 0;
+
+static int num_sms() {
+  if (g_num_sms == 0) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaError_t e = cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return set_cuda_error(e);
+  }
+  return LPF_OK;
+}
+
+// Which of the handle's programs an evaluation walks.
+enum class Which { kTree, kFine, kPlain };
+
+static const Program& side_program(const lpf_paths* p, Which w, int side) {
+  const Paths& h = p->host;
+  if (w == Which::kPlain) return side ? h.plain_t : h.plain;
+  if (w == Which::kFine) return side ? h.fine_t : h.fine;
+  return side ? h.tree_t : h.tree;
+}
+
+static Baked& baked_program(lpf_paths* p, Which w) {
+  return w == Which::kPlain ? p->plain : w == Which::kFine ? p->fine : p->tree;
+}
+
+// The tree's pieces for n_img images of these sides: the short ones while
+// the long ones give the GPU's 32 warps per SM less than a unit each.  A
+// piece is a chain of dependent program loads (64x64, window 32: 328 units
+// of 64 nodes, 20.8 us a walk; 680 of 32 nodes, 14.5 us; 16 nodes gain one
+// more and take longer to lay out); with units for everyone the shorter
+// pieces only repeat more prologues (64 images of 100x128, window 40: 235 us
+// with 64 nodes, 279 with 32).
+static Which tree_pieces(const lpf_paths* p, const Sides& sd, int n_img) {
+  if (p->host.fine.piece_begin.size() < 2) return Which::kTree;
+  int64_t units = 0;
+  for (int q = 0; q < sd.n; ++q)
+    units += (int64_t)sd.g[q].nbg_s * n_img * sd.g[q].G * sd.g[q].BB *
+             ((int64_t)side_program(p, Which::kTree, q).piece_begin.size() - 1);
+  return units < 32 * (int64_t)g_num_sms ? Which::kFine : Which::kTree;
+}
+
+// Bake one of the image's programs for the sides.
+static int bake_sides(lpf_paths* p, const Sides& sd, Which w) {
+  return bake(p, side_program(p, w, 0), sd.g[0], sd.n == 2 ? &side_program(p, w, 1) : nullptr,
+              sd.n == 2 ? &sd.g[1] : nullptr, baked_program(p, w));
 }
 
 using WalkFn = void (*)(const WalkSides, const uint4*, const uint32_t*, unsigned long long*, int64_t, int64_t, int*,
@@ -550,8 +591,6 @@ static void set_kernel_attributes() {
   g_attr_status = rc;
 }
 
-static int g_num_sms = 0;
-
 // Dynamic shared memory of a walk block: the staged rows and, where masks
 // are re-dealt and it fits, 32 entries per warp for that.
 static uint32_t walk_smem(const Sides& sd) {
@@ -566,16 +605,6 @@ static int walk_blocks_for(const Sides& sd) {
                                                                 sd.threads, smem);
   if (e != cudaSuccess) return -set_cuda_error(e);
   return std::max(1, per_sm) * g_num_sms;
-}
-
-static int num_sms() {
-  if (g_num_sms == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaError_t e = cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return set_cuda_error(e);
-  }
-  return LPF_OK;
 }
 
 // Failure-detection self-test (lpf_paths_set_selftest): the staging wait
@@ -646,9 +675,7 @@ static int run_full(const uint8_t* img, int H, int W, lpf_paths* p, int64_t* cou
   if (p->host.dims != 2) return LPF_EINVAL;  // a volume's handle: lpf_full_3d
   if (H < 1 || W < 1 || H > 8192 || W > 8192) return LPF_EINVAL;
   if (p->host.rx >= W || p->host.ry >= H) return LPF_EINVAL;
-  const Program& prog0 = standard ? p->host.plain : p->host.tree;
-  const Program& prog1 = standard ? p->host.plain_t : p->host.tree_t;
-  if (std::max(prog0.stack_depth, prog1.stack_depth) > kDevStack) return LPF_EUNSUPPORTED;
+  if (std::max(p->host.tree.stack_depth, p->host.tree_t.stack_depth) > kDevStack && !standard) return LPF_EUNSUPPORTED;
   std::call_once(g_attr_once, set_kernel_attributes);
   if (g_attr_status) return g_attr_status;
   if (T <= 0)
@@ -665,10 +692,13 @@ static int run_full(const uint8_t* img, int H, int W, lpf_paths* p, int64_t* cou
   }
   rc = ensure_device(p, sd.packed_words);
   if (rc) return rc;
-  Baked& b = standard ? p->plain : p->tree;
-  rc = bake_sides(p, one, standard, b);
-  if (rc) return rc;
   if ((rc = num_sms())) return rc;
+  const Which which = standard ? Which::kPlain : tree_pieces(p, one, n_img);
+  const Program& prog0 = side_program(p, which, 0);
+  const Program& prog1 = side_program(p, which, 1);
+  Baked& b = baked_program(p, which);
+  rc = bake_sides(p, one, which);
+  if (rc) return rc;
   int blocks = walk_blocks_for(sd);
   if (blocks < 0) return -blocks;
   blocks = std::min(blocks, sd.nbg * b.n_pieces);
@@ -789,7 +819,7 @@ static int autotune_full(const uint8_t* img, int H, int W, lpf_paths* p, int64_t
     // trials re-baked it for each shape they ran)
     Sides sd;
     rc = make_sides(p->host, H, W, bt, bb, sd);
-    if (!rc) rc = bake_sides(p, sd, false, p->tree);
+    if (!rc) rc = bake_sides(p, sd, tree_pieces(p, sd, 1));
     if (rc) return rc;
   }
   for (Tuned& t : p->tuned)
@@ -930,22 +960,34 @@ static int run_full_noalloc(const uint8_t* img, int H, int W, lpf_paths* p, int6
   int dev = -1;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return set_cuda_error(e);
-  const Baked& b = p->tree;
+  if ((rc = num_sms())) return rc;
   // The programs for this size must already be on this device (an earlier
-  // lpf_full call put them there).  When the tuned shape needs other row
-  // layouts than the ones they were baked for (lpf_set_launch_shape after
-  // that call), the walk runs in the shape they were baked for instead.
-  if (b.d_words && b.W == W && !baked_for_sides(b, sd) && b.T > 0) {
-    rc = make_sides(p->host, H, W, b.T, b.BB, sd);
-    if (rc) return rc;
+  // lpf_full call put them there): the pieces this size walks, else the
+  // others.  When the tuned shape needs other row layouts than the ones they
+  // were baked for (lpf_set_launch_shape after that call), the walk runs in
+  // the shape they were baked for instead.
+  const Which first = tree_pieces(p, sd, 1);
+  const Baked* found = nullptr;
+  for (Which w : {first, first == Which::kFine ? Which::kTree : Which::kFine}) {
+    const Baked& c = baked_program(p, w);
+    Sides t = sd;
+    if (c.d_words && c.W == W && !baked_for_sides(c, t) && c.T > 0) {
+      rc = make_sides(p->host, H, W, c.T, c.BB, t);
+      if (rc) return rc;
+    }
+    if (baked_for_sides(c, t)) {
+      found = &c;
+      sd = t;
+      break;
+    }
   }
   if ((int)sd.band_bytes > g_max_dyn_smem) return LPF_EUNSUPPORTED;
   if (sd.packed_words > kNoAllocPackedWords) return LPF_EUNSUPPORTED;  // image too large for the fixed area
-  if (p->device != dev || !baked_for_sides(b, sd)) return LPF_EINVAL;
+  if (p->device != dev || !found) return LPF_EINVAL;
+  const Baked& b = *found;
   NoAllocSlot slot;
   rc = noalloc_slot(dev, slot);
   if (rc) return rc;
-  if ((rc = num_sms())) return rc;
   int blocks = walk_blocks_for(sd);
   if (blocks < 0) return -blocks;
   blocks = std::min(blocks, sd.nbg * b.n_pieces);
@@ -1079,6 +1121,8 @@ void lpf_paths_free(lpf_paths* p) {
     cudaDeviceSynchronize();
     cudaFree(p->tree.d_words);
     cudaFree(p->tree.d_piece);
+    cudaFree(p->fine.d_words);
+    cudaFree(p->fine.d_piece);
     cudaFree(p->plain.d_words);
     cudaFree(p->plain.d_piece);
     cudaFree(p->d_packed);

@@ -186,17 +186,23 @@ static void emit_records(const std::vector<Event>& ev, Program& prog,
   rec_pix.push_back(pix_total);
 }
 
-// The tree program of one prefix tree from its depth-first event list: cut
+// The records of a tree's depth-first event list (emit_records), and its
+// program from them: cut
 // into n_pieces pieces of similar pixel count, each with a prologue that
 // rebuilds its starting state from the tree's root (no emits).
-static void make_tree_program(const Trie& t, const std::vector<Event>& ev, int max_level, int n_pieces,
-                              Program& tree) {
-  std::vector<int64_t> rec_word, rec_pix;
-  std::vector<int32_t> rec_cur;
-  std::vector<std::vector<int32_t>> rec_stack;
-  std::vector<uint8_t> rec_restores;
+struct Records {
+  std::vector<int64_t> word, pix;
+  std::vector<int32_t> cur;
+  std::vector<std::vector<int32_t>> stack;
+  std::vector<uint8_t> restores;
   Program full;
-  emit_records(ev, full, rec_word, rec_pix, rec_cur, rec_stack, rec_restores);
+};
+
+static void make_tree_program(const Trie& t, const Records& rec, int max_level, int n_pieces, Program& tree) {
+  const std::vector<int64_t>&rec_word = rec.word, &rec_pix = rec.pix;
+  const std::vector<int32_t>& rec_cur = rec.cur;
+  const std::vector<std::vector<int32_t>>& rec_stack = rec.stack;
+  const Program& full = rec.full;
   const int64_t nrec = (int64_t)rec_word.size() - 1;
   const int64_t total = rec_pix.back();
   // Each cut sits near its share of the pixels, at the record (within a
@@ -429,12 +435,19 @@ int build_paths_nd(int32_t rx, int32_t ry, int32_t rz, int dims, int n_pieces, P
     wk.ev.reserve(sub[root] + 3 * p.n_canon / n_trees);
     wk.node(root, 0);
     if (wk.max_level > kMaxStack) { err = "prefix-tree stack deeper than supported"; return -2; }
-    make_tree_program(t, wk.ev, wk.max_level, pieces_for(sub[root]), o ? p.tree_t : p.tree);
+    Records rec;
+    emit_records(wk.ev, rec.full, rec.word, rec.pix, rec.cur, rec.stack, rec.restores);
+    make_tree_program(t, rec, wk.max_level, pieces_for(sub[root]), o ? p.tree_t : p.tree);
+    if (dims == 2 && nn <= kFineNodes) {
+      const int64_t piece_nodes = std::max<int64_t>(32, (int64_t)std::max(rx, ry) + 1);
+      make_tree_program(t, rec, wk.max_level, (int)std::max<int64_t>(1, sub[root] / piece_nodes),
+                        o ? p.fine_t : p.fine);
+    }
     // Plain program: every segment of the tree from scratch (Alg. 1 order).
     make_plain_program(t, cstart, clist, oseq, p.ptr, orient, (uint8_t)o, root, dims, o ? p.plain_t : p.plain);
     split_program(p, o ? p.plain_t : p.plain, pieces_for(sub[root]));
   }
-  for (Program* prog : {&p.tree, &p.tree_t, &p.plain, &p.plain_t}) {
+  for (Program* prog : {&p.tree, &p.tree_t, &p.fine, &p.fine_t, &p.plain, &p.plain_t}) {
     if (prog->piece_begin.empty()) prog->piece_begin.push_back(0);  // no tree: no pieces
     align_program(*prog);
     resolve_skips(*prog);
@@ -523,7 +536,7 @@ void bake_words(const Paths& p, const Program& prog, int S, int r32, std::vector
   out.reserve(w.size() + w.size() / 8);
   std::vector<int64_t> old_start, new_start;  // record starts (old: words, new: groups)
   std::vector<std::pair<uint32_t, uint32_t>> pix;  // (byte offset, shift)
-  std::vector<uint32_t> singles;
+  std::vector<uint32_t> pairs, singles;
   for (size_t i = 0; i < w.size();) {
     old_start.push_back((int64_t)i);
     new_start.push_back((int64_t)(out.size() / 4));
@@ -543,13 +556,32 @@ void bake_words(const Paths& p, const Program& prog, int S, int r32, std::vector
       pix.push_back({(uint32_t)(row * S + (sxp >> 5)) * 4u, (uint32_t)(sxp & 31)});
     }
     i += n;
-    std::stable_sort(pix.begin(), pix.end(),
-                     [](const std::pair<uint32_t, uint32_t>& a, const std::pair<uint32_t, uint32_t>& b) {
-                       return a.first < b.first;
-                     });
+    if (n <= 48) {  // (short records are most of a program, and nearly sorted or nearly reversed)
+      if (n > 1 && pix.front().first > pix.back().first) {
+        // reversed runs of one window keep their pixels' order
+        std::reverse(pix.begin(), pix.end());
+        for (size_t k = 0; k < pix.size();) {
+          size_t m = k + 1;
+          while (m < pix.size() && pix[m].first == pix[k].first) ++m;
+          std::reverse(pix.begin() + (std::ptrdiff_t)k, pix.begin() + (std::ptrdiff_t)m);
+          k = m;
+        }
+      }
+      for (size_t k = 1; k < pix.size(); ++k) {
+        const std::pair<uint32_t, uint32_t> v = pix[k];
+        size_t m = k;
+        for (; m > 0 && pix[m - 1].first > v.first; --m) pix[m] = pix[m - 1];
+        pix[m] = v;
+      }
+    } else {
+      std::stable_sort(pix.begin(), pix.end(),
+                       [](const std::pair<uint32_t, uint32_t>& a, const std::pair<uint32_t, uint32_t>& b) {
+                         return a.first < b.first;
+                       });
+    }
     // pairs of pixels in one word window, two pairs per group; a pair left
     // over and the unpaired pixels are singles
-    std::vector<uint32_t> pairs;
+    pairs.clear();
     singles.clear();
     for (size_t k = 0; k < pix.size();) {
       if (k + 1 < pix.size() && pix[k].first == pix[k + 1].first) {

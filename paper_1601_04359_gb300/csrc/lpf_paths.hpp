@@ -108,6 +108,10 @@ struct Paths {
   // scratch), for the image (tree, plain) and its transpose (tree_t, plain_t;
   // empty when root_t < 0).
   Program tree, tree_t;
+  // The same trees in pieces half as long, for images so small that the
+  // pieces of tree and tree_t leave warps without work (images; trees up to
+  // kFineNodes nodes, else empty).
+  Program fine, fine_t;
   Program plain, plain_t;
   int64_t n_nodes() const { return (int64_t)node_parent.size(); }
 };
@@ -129,6 +133,7 @@ void segment_canonical3(int dx, int dy, int dz, std::vector<int16_t>& out_xyz);
 // pieces let more warps share a small tree, whose walk is latency-bound.
 // Returns 0 or a negative status.
 constexpr int64_t kMaxPieces = 1024;
+constexpr int64_t kFineNodes = int64_t(1) << 17;  // (wider windows: even the smallest image has a unit per warp)
 int build_paths(int32_t rx, int32_t ry, int n_pieces, Paths& p, std::string& err);
 // The same for dims = 2 (rz ignored) or dims = 3 (vectors |dz| <= rz too).
 int build_paths_nd(int32_t rx, int32_t ry, int32_t rz, int dims, int n_pieces, Paths& p, std::string& err);

@@ -101,7 +101,7 @@ struct DeltaTables {
 struct lpf_paths {
   lpf::Paths host;
   int device = -1;
-  lpf::Baked tree, plain;
+  lpf::Baked tree, plain, fine;
   uint32_t* d_packed = nullptr;  // work area: packed image (one at a time)
   size_t packed_cap = 0;         // words
   int* d_status = nullptr;       // [0] status flags since the last check, [1] work counter,
