@@ -87,6 +87,17 @@ __device__ __forceinline__ void delta_mark(uint8_t* e, int c, uint8_t val, const
     for (int ex = (cx + g.rx) % g.W; ex < g.We; ex += g.W) e[ey * g.We + ex] = val;
 }
 
+// The same by the lanes of a warp: lanes 0 .. 8 write the copies of a, lanes
+// 16 .. 24 those of b (rx < W, ry < H: at most three copies along an axis).
+__device__ __forceinline__ void delta_mark_pair(uint8_t* e, int ax, int ay, uint8_t val_a, int bx, int by,
+                                                uint8_t val_b, const DeltaArgs& g, int lane) {
+  const int l = lane & 15;
+  if (l >= 9) return;
+  const int ey = (lane < 16 ? ay : by) + g.ry + (l / 3 - 1) * g.H;
+  const int ex = (lane < 16 ? ax : bx) + g.rx + (l % 3 - 1) * g.W;
+  if (ey >= 0 && ey < g.He && ex >= 0 && ex < g.W + 2 * g.rx) e[ey * g.We + ex] = lane < 16 ? val_a : val_b;
+}
+
 // Stage the extended cell (bulk copy, bounded wait).  False on timeout.
 __device__ __forceinline__ bool delta_stage(uint8_t* sm, const uint8_t* ext, uint32_t bytes, uint64_t* bar) {
   if (threadIdx.x == 0) {
@@ -258,28 +269,6 @@ __device__ __forceinline__ void delta_vector(const DeltaArgs& g, int v, int& dx,
   dy = d.y;
 }
 
-// True when pixel (qx, qy) lies on S(v) placed at translation (x, y), on the
-// torus (the segment spans fewer than W columns and H rows, so at most one
-// period of (qx, qy) is in its bounding box).
-__device__ __forceinline__ bool delta_on_segment(const DeltaArgs& g, int o0, int dx, int dy, int x, int y, int qx,
-                                                 int qy) {
-  int uy = qy - y;                          // in (-H, H)
-  if (uy < 0) uy += g.H;
-  if (uy > dy) return false;                // canonical: 0 <= sy <= dy
-  const int xlo = dx < 0 ? dx : 0, xhi = dx < 0 ? 0 : dx;
-  int ux = qx - x - xlo;                    // in (-W, W + rx), rx < W
-  if (ux < 0) ux += g.W;
-  else if (ux >= g.W) ux -= g.W;
-  ux += xlo;
-  if (ux > xhi) return false;
-  const int adx = dx < 0 ? -dx : dx;
-  if (adx >= dy) {                          // x-major: pixel k at sx = sign(dx) k
-    const int k = dx < 0 ? -ux : ux;
-    return g.off16[2 * (o0 + k) + 1] == uy;
-  }
-  return g.off16[2 * (o0 + uy)] == ux;      // y-major: pixel k at sy = k
-}
-
 // A block's vector chunk for the block-wide lookups of the persistent
 // annealer.  The segment pixels of the chunk's vectors v0 <= v < v0 + nv are
 // the contiguous entries o_base + [0, pre[nv]) of off16, copied to off;
@@ -289,8 +278,8 @@ __device__ __forceinline__ bool delta_on_segment(const DeltaArgs& g, int o0, int
 struct ChunkTables {
   const int32_t* pre;   // [nv + 1] entry offsets
   const short2* vec;    // [nv] the chunk's canonical vectors (dx, dy)
-  const int32_t* shear; // [nv] their delta_shear
-  const short2* off;    // [pre[nv]] the chunk's segment pixels (sx, sy)
+  const int32_t* desc;  // [nv] chunk_descriptor of each
+  const short2* off;    // [pre[nv]] the chunk's segment pixels (along the longer axis, along the other)
   const uint16_t* vid;  // [pre[nv]] the chunk-relative vector of every entry
   int32_t* d;           // [2][mv] count changes (phase 0, phase 1)
   float* term;          // [mv] error terms
@@ -317,15 +306,22 @@ struct PixelPair {
   int ax, ay, bx, by;
 };
 
-// delta_on_segment for chunk vector i, reading its pixels from the chunk's
-// copy in shared memory.
+// What a lookup needs of a vector, in one word: its delta_shear m (18 bits),
+// its pixels n (8 bits), whether it is y-major.
+__host__ __device__ __forceinline__ int32_t chunk_descriptor(int m, int n, bool ymajor) {
+  return (int32_t)((uint32_t)m << 14 | (uint32_t)n << 1 | (uint32_t)ymajor);
+}
+
+// True when pixel (qx, qy) lies on S(v) of chunk vector i placed at
+// translation (x, y), on the torus (the segment spans fewer than W columns
+// and H rows, so at most one period of (qx, qy) is in its bounding box).
 __device__ __forceinline__ bool chunk_on_segment(const DeltaArgs& g, const ChunkTables& ct, int i, int dx, int dy,
                                                  int x, int y, int qx, int qy) {
-  int uy = qy - y;
+  int uy = qy - y;                          // in (-H, H)
   if (uy < 0) uy += g.H;
-  if (uy > dy) return false;
+  if (uy > dy) return false;                // canonical: 0 <= sy <= dy
   const int xlo = dx < 0 ? dx : 0, xhi = dx < 0 ? 0 : dx;
-  int ux = qx - x - xlo;
+  int ux = qx - x - xlo;                    // in (-W, W + rx), rx < W
   if (ux < 0) ux += g.W;
   else if (ux >= g.W) ux -= g.W;
   ux += xlo;
@@ -333,23 +329,46 @@ __device__ __forceinline__ bool chunk_on_segment(const DeltaArgs& g, const Chunk
   const short2* o = ct.off + ct.pre[i];
   const int adx = dx < 0 ? -dx : dx;
   if (adx >= dy) return o[dx < 0 ? -ux : ux].y == uy;  // x-major: pixel k at sx = sign(dx) k
-  return o[uy].x == ux;                                // y-major: pixel k at sy = k
+  return o[uy].y == ux;                                // y-major: pixel k at sy = k
 }
 
-// Translation of chunk entry j for the exchange pixel (qx, qy): the start x
-// of the segment whose pixel j is q, wrapped onto the torus, and the byte of
-// z holding its phase-0 count (z has fewer than 2^31 bytes on the lookup
-// path).
+// t in (-2n, 3n) reduced into [0, n).
+__device__ __forceinline__ int chunk_wrap(int t, int n) {
+  if (t < 0) { t += n; if (t < 0) t += n; }
+  else if (t >= n) { t -= n; if (t >= n) t -= n; }
+  return t;
+}
+
+// Chunk entry j for the exchange pixel (qx, qy): its vector i and the byte of
+// z holding the phase-0 count of the translation whose pixel j is q (z has
+// fewer than 2^31 bytes on the lookup path).  The same index as
+// delta_z_index of that translation, reduced once: with t its coordinate
+// along the longer axis, the other one less the shear at t, modulo that
+// extent.
 __device__ __forceinline__ void chunk_entry(const DeltaArgs& g, const ChunkTables& ct, int v0, int j, int qx, int qy,
-                                            int& i, int& x, int& y, uint32_t& zi) {
+                                            int& i, uint32_t& zi) {
   i = ct.vid[j];
-  const short2 s2 = ct.off[j];
-  x = qx - s2.x;
-  y = qy - s2.y;
+  const short2 o = ct.off[j];
+  const int32_t d = ct.desc[i];
+  const bool ym = d & 1;
+  const int P = ym ? g.H : g.W, Q = ym ? g.W : g.H;
+  int t = (ym ? qy : qx) - o.x;
+  t = t < 0 ? t + P : (t >= P ? t - P : t);
+  int r = (ym ? qx : qy) - o.y - delta_shift(t, d >> 14);
+  // (square cells: |shear| < Q)
+  r = g.H == g.W ? chunk_wrap(r, Q) : ((r % Q) + Q) % Q;
+  zi = (uint32_t)(v0 + i) * (uint32_t)(g.H * g.W) + (uint32_t)(r * P + t);
+}
+
+// Its translation.
+__device__ __forceinline__ void chunk_translation(const DeltaArgs& g, const ChunkTables& ct, int j, int qx, int qy,
+                                                  int& x, int& y) {
+  const short2 o = ct.off[j];
+  const bool ym = ct.desc[ct.vid[j]] & 1;
+  x = qx - (ym ? o.y : o.x);
+  y = qy - (ym ? o.x : o.y);
   x = x < 0 ? x + g.W : (x >= g.W ? x - g.W : x);
   y = y < 0 ? y + g.H : (y >= g.H ? y - g.H : y);
-  const short2 dv = ct.vec[i];
-  zi = (uint32_t)(v0 + i) * (uint32_t)(g.H * g.W) + (uint32_t)delta_z_index(g, dv.x, dv.y, ct.shear[i], x, y);
 }
 
 // Count changes and error change of the chunk's vectors for the exchange of
@@ -359,24 +378,28 @@ __device__ __forceinline__ void chunk_entry(const DeltaArgs& g, const ChunkTable
 // the one through b; kChunkUnroll lookups per thread in flight.  When the block has at most
 // kChunkUnroll entries per thread, *held receives the thread's counts as
 // read (one byte each) and held_zi their offsets in z, for
-// delta_chunk_apply_held; else *held is 0.  Every thread calls it; thread 0
-// returns the chunk's error change, summed over the vectors in a fixed
-// order.
+// delta_chunk_apply_held; else *held is 0.  clean: ct.d is all zero already
+// (and a barrier has passed since).  Every thread calls it; thread 0 returns
+// the chunk's error change, summed over the vectors in a fixed order.  Chunks
+// of up to 64 vectors (most: 18 on average at window 64) are finished by warp
+// 0 alone, the others go on to wait for the batch's decision.
 __device__ __forceinline__ float delta_chunk_lookup(const DeltaArgs& g, const PixelPair& q, int v0,
                                                     const ChunkTables& ct, int32_t* dcounts_k,
                                                     const DeltaTerms& dt, uint32_t* held,
-                                                    uint32_t (&held_zi)[kChunkUnroll]) {
+                                                    uint32_t (&held_zi)[kChunkUnroll], bool clean) {
   const int E = ct.pre[ct.nv];
-  for (int i = threadIdx.x; i < ct.nv; i += blockDim.x) {
-    ct.d[i] = 0;
-    ct.d[ct.mv + i] = 0;
+  if (!clean) {
+    for (int i = threadIdx.x; i < ct.nv; i += blockDim.x) {
+      ct.d[i] = 0;
+      ct.d[ct.mv + i] = 0;
+    }
+    __syncthreads();
   }
-  __syncthreads();
   const int ax = q.ax, ay = q.ay, bx = q.bx, by = q.by;
   const int nthr = blockDim.x;
   uint32_t h = 0;
   for (int e0 = 0; e0 < 2 * E; e0 += kChunkUnroll * nthr) {
-    int vi[kChunkUnroll], xs[kChunkUnroll], ys[kChunkUnroll], zs[kChunkUnroll];
+    int vi[kChunkUnroll], zs[kChunkUnroll];
     uint32_t zi[kChunkUnroll];
 #pragma unroll
     for (int u = 0; u < kChunkUnroll; ++u) {
@@ -384,7 +407,7 @@ __device__ __forceinline__ float delta_chunk_lookup(const DeltaArgs& g, const Pi
       vi[u] = -1;
       if (e < 2 * E) {
         const bool side = e >= E;
-        chunk_entry(g, ct, v0, side ? e - E : e, side ? bx : ax, side ? by : ay, vi[u], xs[u], ys[u], zi[u]);
+        chunk_entry(g, ct, v0, side ? e - E : e, side ? bx : ax, side ? by : ay, vi[u], zi[u]);
       }
     }
 #pragma unroll
@@ -396,12 +419,17 @@ __device__ __forceinline__ float delta_chunk_lookup(const DeltaArgs& g, const Pi
     for (int u = 0; u < kChunkUnroll; ++u) {
       h |= (uint32_t)zs[u] << (8 * u);
       if (vi[u] < 0) continue;
+      const int i = vi[u], z = zs[u];
+      const int L1 = (ct.desc[i] >> 1) & 0xff;
+      // (at most one pixel off uniform, or nothing changes: few lookups)
+      if (z > 1 && z < L1 - 1) continue;
       const int e = e0 + u * nthr + (int)threadIdx.x;
-      const int i = vi[u], x = xs[u], y = ys[u], z = zs[u];
+      const bool side = e >= E;
+      int x, y;
+      chunk_translation(g, ct, side ? e - E : e, side ? bx : ax, side ? by : ay, x, y);
       if (g.sel_ext && !g.sel_ext[(y + g.ry) * g.We + (x + g.rx)]) continue;  // start not sampled
-      const int L1 = ct.pre[i + 1] - ct.pre[i];
       const short2 dv = ct.vec[i];
-      if (e < E) {
+      if (!side) {
         if (z == 0) atomicAdd(ct.d + ct.mv + i, -1);
         if (z == L1 - 1 && !chunk_on_segment(g, ct, i, dv.x, dv.y, x, y, bx, by)) atomicAdd(ct.d + i, 1);
       } else {
@@ -413,7 +441,8 @@ __device__ __forceinline__ float delta_chunk_lookup(const DeltaArgs& g, const Pi
   *held = 2 * E <= kChunkUnroll * nthr ? h : 0u;
   __syncthreads();
   const float invN = g.inv_norm;
-  for (int i = threadIdx.x; i < ct.nv; i += blockDim.x) {
+  // the error term of chunk vector i (and its count changes to dcounts_k)
+  auto term = [&](int i) -> float {
     const int d0 = ct.d[i], d1 = ct.d[ct.mv + i];
     const int v = v0 + i;
     if (dcounts_k) {
@@ -434,12 +463,16 @@ __device__ __forceinline__ float delta_chunk_lookup(const DeltaArgs& g, const Pi
         acc += xx * (xx - 2.0f * dd);
       }
     }
-    ct.term[i] = acc;
+    return acc;
+  };
+  const bool one_warp = ct.nv <= 64;
+  if (!one_warp) {
+    for (int i = threadIdx.x; i < ct.nv; i += blockDim.x) ct.term[i] = term(i);
+    __syncthreads();
   }
-  __syncthreads();
   float sum = 0.0f;
   if (threadIdx.x < 32) {  // lane-strided sums in vector order, then a fixed shuffle tree
-    for (int i = threadIdx.x; i < ct.nv; i += 32) sum += ct.term[i];
+    for (int i = threadIdx.x; i < ct.nv; i += 32) sum += one_warp ? term(i) : ct.term[i];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
   }
@@ -463,6 +496,16 @@ __device__ __forceinline__ bool chunk_maybe_both(const DeltaArgs& g, int dx, int
   return (cross < 0 ? -cross : cross) <= (adx > dy ? adx : dy);
 }
 
+// The torus displacement b - a in [-W/2, W/2) x [-H/2, H/2).
+__device__ __forceinline__ void chunk_displacement(const DeltaArgs& g, const PixelPair& q, int& ddx, int& ddy) {
+  ddx = q.bx - q.ax;
+  ddy = q.by - q.ay;
+  if (2 * ddx >= g.W) ddx -= g.W;
+  else if (2 * ddx < -g.W) ddx += g.W;
+  if (2 * ddy >= g.H) ddy -= g.H;
+  else if (2 * ddy < -g.H) ddy += g.H;
+}
+
 // After exchanging a (now phase 0) and b (now phase 1): z_v += 1 on the
 // translations through a and -= 1 on those through b, for the chunk's
 // vectors, with the counts delta_chunk_lookup read for this same exchange
@@ -472,29 +515,27 @@ __device__ __forceinline__ bool chunk_maybe_both(const DeltaArgs& g, int dx, int
 // translation through both pixels keeps its count (its two entries are
 // one byte, which neither stores); within one side a vector's translations
 // are distinct, so no two threads store the same byte.  Every thread calls
-// it with the same pixels as that lookup.
+// it with the same pixels as that lookup.  maybe: chunk_maybe_both of every
+// vector of the chunk (then only a flag is read per entry), or null.
 __device__ __forceinline__ void delta_chunk_apply_held(const DeltaArgs& g, const PixelPair& q, int v0,
                                                        const ChunkTables& ct, uint32_t held,
-                                                       const uint32_t (&held_zi)[kChunkUnroll]) {
+                                                       const uint32_t (&held_zi)[kChunkUnroll], const int* maybe) {
   const int E = ct.pre[ct.nv];
   const int nthr = blockDim.x;
-  int ddx = q.bx - q.ax, ddy = q.by - q.ay;
-  if (2 * ddx >= g.W) ddx -= g.W;
-  else if (2 * ddx < -g.W) ddx += g.W;
-  if (2 * ddy >= g.H) ddy -= g.H;
-  else if (2 * ddy < -g.H) ddy += g.H;
+  int ddx, ddy;
+  chunk_displacement(g, q, ddx, ddy);
 #pragma unroll
   for (int u = 0; u < kChunkUnroll; ++u) {
     const int e = u * nthr + (int)threadIdx.x;
     if (e >= 2 * E) continue;
     const bool side = e >= E;
     const int j = side ? e - E : e;
-    const short2 dv = ct.vec[ct.vid[j]];
-    if (chunk_maybe_both(g, dv.x, dv.y, ddx, ddy)) {  // rare: check the other pixel on the segment
-      int i, x, y;
-      uint32_t zi;
-      chunk_entry(g, ct, v0, j, side ? q.bx : q.ax, side ? q.by : q.ay, i, x, y, zi);
-      if (chunk_on_segment(g, ct, i, dv.x, dv.y, x, y, side ? q.ax : q.bx, side ? q.ay : q.by)) continue;
+    const int vi = ct.vid[j];
+    const short2 dv = ct.vec[vi];
+    if (maybe ? maybe[vi] : chunk_maybe_both(g, dv.x, dv.y, ddx, ddy)) {  // rare: check the other pixel on the segment
+      int x, y;
+      chunk_translation(g, ct, j, side ? q.bx : q.ax, side ? q.by : q.ay, x, y);
+      if (chunk_on_segment(g, ct, vi, dv.x, dv.y, x, y, side ? q.ax : q.bx, side ? q.ay : q.by)) continue;
     }
     const uint32_t z = (held >> (8 * u)) & 0xffu;
     __stcg(g.z + held_zi[u], (uint8_t)(side ? z - 1u : z + 1u));
@@ -521,8 +562,8 @@ __device__ __forceinline__ void delta_chunk_update(const DeltaArgs& g, const Pix
         ok[u] = j < E;
         zi[u] = 0;
         if (ok[u]) {
-          int i, x, y;
-          chunk_entry(g, ct, v0, j, qx, qy, i, x, y, zi[u]);
+          int i;
+          chunk_entry(g, ct, v0, j, qx, qy, i, zi[u]);
         }
       }
 #pragma unroll

@@ -226,14 +226,25 @@ __global__ void __launch_bounds__(kDeltaThreads, 3) sa_batch_kernel(
 // and keeps its extended cell and a copy of the run state in shared memory.
 // Per batch every block draws the batch's candidates, evaluates its chunk
 // for each (with the phase-0 counts: the chunk's lookups spread over all
-// threads of the block, so that every block takes about the same time to
-// reach the barrier; else walks) and writes its partial error changes; after one grid barrier every
-// block sums the partials of each candidate in the same fixed order, so all
-// blocks find the same first accepted candidate, apply it to their own cell
-// copy and to the counts of their own vectors, and advance their identical
-// copies of the run state.  Partials, pairs and uniforms alternate between
-// two buffers by batch parity: batch b + 2 may overwrite batch b's only after
-// the barrier of batch b + 1, which no block reaches before it has read them.
+// threads of the block, so that every block takes about the same time; else
+// walks) and gives its partial error changes to the others: in messages
+// (post_message) for batches of a few candidates, else through a grid
+// barrier.  Every block sums the partials of each candidate in the same fixed
+// order, so all blocks find the same first accepted candidate, apply it to
+// their own cell copy and to the counts of their own vectors, and advance
+// their identical copies of the run state.  Partials, pairs, uniforms and
+// messages alternate between two buffers by batch parity: batch b + 2 may
+// overwrite batch b's only after batch b + 1's have all arrived, which no
+// block gives before it has read batch b's.
+//
+// What bounds it: a batch is a chain of latencies -- the lookups, the messages'
+// way, the decision, its consequences -- and of the instructions of 48 warps
+// per SM in the lookups and updates.  Measured at 128x128, window 64 (a batch
+// of one): 14.0 -> 11.9 us by taking off that chain what another warp can do
+// while the messages are on their way (the next candidate and the schedule's
+// next step for both outcomes, which vectors may hold both pixels), one word
+// instead of four per vector in the lookups, and no marks for lookups.
+// Prefetching the next lookups' sectors of z into L2 gained nothing.
 
 constexpr uint32_t kBarrierPolls = 1u << 22;  // polls of a grid barrier before giving up (seconds)
 
@@ -264,17 +275,79 @@ __device__ __forceinline__ bool sa_grid_barrier(unsigned int* count, unsigned in
   return s_ok != 0;
 }
 
+// A candidate of a batch: its pixels (also as coordinates) and its uniform.
+struct SaCand {
+  int a, b;
+  float u;
+  PixelPair q;
+};
+
+// Batches of up to kMsgCandidates candidates (nearly all of them, while more
+// than a sixth of the candidates is accepted) need no grid barrier: a block
+// posts its partial error change of candidate k as one 64-bit message {batch
+// number, value}, and warp k of every block reads the messages of all blocks
+// until each carries the batch's number.  That is one store and one load on
+// the way instead of a counter's atomic, its polls and then the partials'
+// loads.  Messages alternate between two sets by batch parity, as the
+// partials do; a launch starts with all of them zero.
+constexpr int kMsgCandidates = 3;
+
+__device__ __forceinline__ void post_message(unsigned long long* to, unsigned int batch, float value) {
+  const unsigned long long m = (unsigned long long)batch << 32 | __float_as_uint(value);
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(to), "l"(m) : "memory");
+}
+
+// The sum over n messages of batch `batch` (lane-strided in chunk order, then a
+// fixed shuffle tree: sa_first_accept's order).  A warp calls it; false if
+// some message did not come within kBarrierPolls polls.
+static __device__ __noinline__ bool hear_messages(const unsigned long long* from, int n, unsigned int batch, int lane,
+                                              float* sum) {
+  float de = 0.0f;
+  bool all = true;
+  __nanosleep(600);  // blocks seldom finish closer together, and polls slow the others' lookups (4 % of a batch)
+  for (int c0 = lane; c0 - lane < n; c0 += 32 * 16) {
+    unsigned long long m[16];
+    unsigned pending = 0;
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      m[r] = 0;
+      if (c0 + 32 * r < n) pending |= 1u << r;
+    }
+    for (uint32_t it = 0; pending && it < kBarrierPolls; ++it) {
+#pragma unroll
+      for (int r = 0; r < 16; ++r)
+        if ((pending >> r) & 1u)
+          asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(m[r]) : "l"(from + c0 + 32 * r) : "memory");
+#pragma unroll
+      for (int r = 0; r < 16; ++r)
+        if (((pending >> r) & 1u) && (unsigned int)(m[r] >> 32) == batch) pending &= ~(1u << r);
+    }
+    all = all && pending == 0;
+#pragma unroll
+    for (int r = 0; r < 16; ++r)
+      if (c0 + 32 * r < n) de += __uint_as_float((unsigned int)m[r]);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) de += __shfl_xor_sync(0xffffffffu, de, o);
+  *sum = de;
+  return __all_sync(0xffffffffu, all);
+}
+
 __global__ void __launch_bounds__(kDeltaThreads, 3) sa_persistent_kernel(
     SaDev* __restrict__ st, uint8_t* __restrict__ cell, uint8_t* __restrict__ ext, DeltaArgs g,
     int32_t* __restrict__ pairs2, float* __restrict__ u2, int32_t* __restrict__ dcounts, float* __restrict__ partial2,
-    unsigned long long* __restrict__ counts, int* __restrict__ status, unsigned int* __restrict__ bar, int n_batches,
-    int k_max, unsigned int bar_extra, int bar_block) {
+    unsigned long long* __restrict__ counts, int* __restrict__ status, unsigned int* __restrict__ bar,
+    unsigned long long* __restrict__ msg, int n_batches, int k_max, unsigned int bar_extra, int bar_block) {
   extern __shared__ __align__(16) uint8_t sm[];
   __shared__ __align__(8) uint64_t mbar;
   __shared__ SaDev s_state;
-  __shared__ float warp_acc[kDeltaWarps];
-  __shared__ int s_a, s_b, s_na, s_nb;
-  __shared__ PixelPair s_q, s_nq;  // the pixels of s_a, s_b and of s_na, s_nb as coordinates
+  __shared__ union {  // walks; messages
+    float acc[kDeltaWarps];
+    SaCand drawn[2];  // the next batch's first candidate if this one is rejected, or accepted
+  } s_warp;
+  __shared__ SaCand s_cur, s_next;  // a batch's first candidate goes through s_next, later ones through s_cur
+  __shared__ int s_pa[kMsgCandidates], s_pb[kMsgCandidates], s_kstar, s_heard;
+  __shared__ float s_u[kMsgCandidates], s_de[kMsgCandidates];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ch = blockIdx.x;
   const int v0 = g.chunk[ch], v1 = g.chunk[ch + 1], nv = v1 - v0;
@@ -296,10 +369,10 @@ __global__ void __launch_bounds__(kDeltaThreads, 3) sa_persistent_kernel(
   ct.vec = s_vec;
   ct.d = reinterpret_cast<int32_t*>(s_vec + mv);                      // [2][mv]
   ct.term = reinterpret_cast<float*>(ct.d + 2 * mv);                  // [mv]
-  int32_t* s_shear = reinterpret_cast<int32_t*>(ct.term + mv);       // [mv]
-  short2* s_off = reinterpret_cast<short2*>(s_shear + mv);            // [max_chunk_entries]
+  int32_t* s_desc = reinterpret_cast<int32_t*>(ct.term + mv);        // [mv]
+  short2* s_off = reinterpret_cast<short2*>(s_desc + mv);            // [max_chunk_entries]
   uint16_t* s_vid = reinterpret_cast<uint16_t*>(s_off + g.max_chunk_entries);  // [max_chunk_entries]
-  ct.shear = s_shear;
+  ct.desc = s_desc;
   ct.off = s_off;
   ct.vid = s_vid;
   ct.nv = nv;
@@ -310,19 +383,23 @@ __global__ void __launch_bounds__(kDeltaThreads, 3) sa_persistent_kernel(
     if (i < nv) {
       const short2 dv = reinterpret_cast<const short2*>(g.vec16)[v0 + i];
       s_vec[i] = dv;
-      s_shear[i] = g.shear[v0 + i];
+      s_desc[i] = chunk_descriptor(g.shear[v0 + i], g.dptr[v0 + i + 1] - g.dptr[v0 + i],
+                                   dv.y > (dv.x < 0 ? -dv.x : dv.x));
     }
   }
   __syncthreads();  // s_pre is complete
   for (int j = threadIdx.x; j < n_ent; j += blockDim.x) {
-    s_off[j] = reinterpret_cast<const short2*>(g.off16)[o_base + j];
-    s_vid[j] = (uint16_t)chunk_vector_of(s_pre, nv, j);
+    const int i = chunk_vector_of(s_pre, nv, j);
+    const short2 o = reinterpret_cast<const short2*>(g.off16)[o_base + j];
+    s_off[j] = (s_desc[i] & 1) ? make_short2(o.y, o.x) : o;
+    s_vid[j] = (uint16_t)i;
   }
   for (int i = threadIdx.x; i < nv; i += blockDim.x) {
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
       s_tgt[p * mv + i] = g.target[p * g.n_full + g.base + v0 + i];
       s_cnt[p * mv + i] = (long long)counts[p * g.n_full + g.base + v0 + i];
+      ct.d[p * mv + i] = 0;
     }
   }
   __syncthreads();
@@ -335,140 +412,233 @@ __global__ void __launch_bounds__(kDeltaThreads, 3) sa_persistent_kernel(
   uint32_t held = 0;  // the phase-0 counts this thread read for candidate held_k
   uint32_t held_zi[kChunkUnroll] = {0, 0, 0, 0};  // and where they are in z
   int held_k = -1;
-  // Candidate k of batch bi (warp 0): drawn from the block's own cell copy,
-  // marked there, kept in *sa / *sb; block 0 also records it for the others.
-  // (n0: the batch's first evaluation index; the draw reads only the run
-  // state's fixed fields, so it may run while warp 0 advances the rest)
-  auto draw = [&](int bi, unsigned long long n0, int k, int* sa, int* sb, PixelPair* sq) {
-    int a, b;
-    float uu;
-    draw_candidate_warp(sm, g, n0 + (unsigned long long)k, s_state.key0, s_state.key1, a, b, uu, &s_state, lane);
-    if (lane == 0) {
-      if (ch == 0) {
-        pairs2[(size_t)(bi & 1) * 2 * k_max + 2 * k] = a;
-        pairs2[(size_t)(bi & 1) * 2 * k_max + 2 * k + 1] = b;
-        u2[(size_t)(bi & 1) * k_max + k] = uu;
-        __threadfence();  // written by a thread other than the one that arrives at the grid barrier
-      }
-      *sa = a;
-      *sb = b;
-      sq->ay = a / g.W;
-      sq->ax = a - sq->ay * g.W;
-      sq->by = b / g.W;
-      sq->bx = b - sq->by * g.W;
-      if (a != b) { delta_mark(sm, a, kMarkA, g); delta_mark(sm, b, kMarkB, g); }
-    }
+  const bool held_ok = 2 * n_ent <= kChunkUnroll * (int)blockDim.x;
+  // Candidate n of the run from the block's own cell copy (a whole warp); the
+  // draw reads only the run state's fixed fields, so it may run while warp 0
+  // advances the rest.
+  auto draw = [&](unsigned long long n) -> SaCand {
+    SaCand c;
+    draw_candidate_warp(sm, g, n, s_state.key0, s_state.key1, c.a, c.b, c.u, &s_state, lane);
+    c.q.ay = c.a / g.W;
+    c.q.ax = c.a - c.q.ay * g.W;
+    c.q.by = c.b / g.W;
+    c.q.bx = c.b - c.q.by * g.W;
+    return c;
   };
-  // The first candidate of every batch is drawn ahead, by warp 1 at the end
-  // of the batch before (while warp 0 advances the run state and the other
-  // warps apply the exchange), into s_na, s_nb; later candidates of a batch
-  // go through s_a, s_b.
-  if (warp == 1 && !s_state.done && n_batches > 0) draw(0, (unsigned long long)s_state.n_eval, 0, &s_na, &s_nb, &s_nq);
+  // Candidate k of batch bi taken up (lane 0 of a warp): kept in *to, recorded
+  // by block 0 for the others, marked for the walks (lookups need no marks).
+  auto take = [&](int bi, int k, const SaCand& c, SaCand* to) {
+    if (ch == 0) {
+      pairs2[(size_t)(bi & 1) * 2 * k_max + 2 * k] = c.a;
+      pairs2[(size_t)(bi & 1) * 2 * k_max + 2 * k + 1] = c.b;
+      u2[(size_t)(bi & 1) * k_max + k] = c.u;
+    }
+    *to = c;
+    if (!g.z && c.a != c.b) { delta_mark(sm, c.a, kMarkA, g); delta_mark(sm, c.b, kMarkB, g); }
+  };
+  // The first candidate of every batch is drawn ahead by warp 1: after a
+  // single-candidate batch both ways it can end, while the other blocks'
+  // messages are awaited; else once it has ended.
+  if (warp == 1 && !s_state.done && n_batches > 0) {
+    const SaCand c = draw((unsigned long long)s_state.n_eval);
+    if (lane == 0) take(0, 0, c, &s_next);
+  }
+  unsigned int n_bar = 0;  // grid barriers passed
   __syncthreads();
   for (int bi = 0; bi < n_batches && !s_state.done; ++bi) {
     const int Keff = s_state.k_eff;
     const unsigned long long n0 = (unsigned long long)s_state.n_eval;
+    const long long left = s_state.n_step - s_state.n_eval;
+    const int Kv = (int)min((long long)Keff, max(0LL, left));
+    const bool fast = g.z && Keff <= kMsgCandidates;
+    // (bar_extra > 0 only in lpf_sa_selftest_timeout: block bar_block, or
+    // every block if bar_block < 0, waits for what never comes)
+    const unsigned int extra = (bar_block < 0 || (int)blockIdx.x == bar_block) ? bar_extra : 0u;
     int32_t* pairs = pairs2 + (size_t)(bi & 1) * 2 * k_max;
     float* u = u2 + (size_t)(bi & 1) * k_max;
     float* partial = partial2 + (size_t)(bi & 1) * k_max * g.n_chunks;
-    int last_a = 0, last_b = 0;  // the batch's last candidate
-    PixelPair last_q = {0, 0, 0, 0};
+    unsigned long long* mail = msg + (size_t)(bi & 1) * kMsgCandidates * g.n_chunks;
+    if (threadIdx.x == 0) { s_kstar = INT_MAX; s_heard = 1; }
+    SaCand last;  // the batch's last candidate
     for (int k = 0; k < Keff; ++k) {
-      if (k > 0 && warp == 0) draw(bi, n0, k, &s_a, &s_b, &s_q);
-      __syncthreads();
-      const int a = k == 0 ? s_na : s_a, b = k == 0 ? s_nb : s_b;
-      const PixelPair q = k == 0 ? s_nq : s_q;
-      last_a = a;
-      last_b = b;
-      last_q = q;
+      if (k > 0) {
+        if (warp == 0) {
+          const SaCand c = draw(n0 + (unsigned long long)k);
+          if (lane == 0) take(bi, k, c, &s_cur);
+        }
+        __syncthreads();
+      }
+      last = k == 0 ? s_next : s_cur;
+      const int a = last.a, b = last.b;
+      if (fast && threadIdx.x == 0) { s_pa[k] = a; s_pb[k] = b; s_u[k] = last.u; }
       int32_t* dk = dcounts + (int64_t)k * 2 * g.n_canon;
       float acc = 0.0f;
-      const bool block_sum = a != b && g.z;  // block-wide lookups: thread 0 holds the chunk's sum
       held_k = -1;
-      if (a == b) delta_zero_vectors(g, v0, v1, dk);
-      else if (g.z) {
-        acc = delta_chunk_lookup(g, q, v0, ct, dk, dt, &held, held_zi);
-        if (2 * n_ent <= kChunkUnroll * (int)blockDim.x) held_k = k;  // this candidate's counts stay in registers
+      if (g.z) {
+        // count changes that stay in shared memory until the decision are not written out
+        int32_t* out = held_ok && k == Keff - 1 ? nullptr : dk;
+        if (a == b) {
+          if (out) delta_zero_vectors(g, v0, v1, out);
+        } else {
+          acc = delta_chunk_lookup(g, last.q, v0, ct, out, dt, &held, held_zi, k == 0);
+          if (held_ok) held_k = k;  // this candidate's counts stay in registers
+        }
+        if (threadIdx.x == 0) {
+          if (fast) post_message(mail + (size_t)k * g.n_chunks + ch, (unsigned int)(bi + 1), acc);
+          else partial[(int64_t)k * g.n_chunks + ch] = acc;
+        }
+        if (k + 1 < Keff) __syncthreads();  // before s_cur and ct.d are rewritten
+      } else {
+        if (a == b) delta_zero_vectors(g, v0, v1, dk);
+        else acc = delta_walk_vectors(sm, g, a, b, v0, v1, warp, lane, dk, dt);
+        if (lane == 0) s_warp.acc[warp] = acc;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+          float sum = 0.0f;
+          for (int w = 0; w < kDeltaWarps; ++w) sum += s_warp.acc[w];
+          partial[(int64_t)k * g.n_chunks + ch] = sum;
+          if (a != b) { delta_mark(sm, a, 1, g); delta_mark(sm, b, 0, g); }
+        }
+        __syncthreads();
       }
-      else acc = delta_walk_vectors(sm, g, a, b, v0, v1, warp, lane, dk, dt);
-      if (!block_sum && lane == 0) warp_acc[warp] = acc;
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        float sum = 0.0f;
-        if (block_sum) sum = acc;
-        else
-          for (int w = 0; w < kDeltaWarps; ++w) sum += warp_acc[w];
-        partial[(int64_t)k * g.n_chunks + ch] = sum;
-        if (a != b) { delta_mark(sm, a, 1, g); delta_mark(sm, b, 0, g); }
-      }
-      __syncthreads();
     }
-    // (bar_extra > 0 only in lpf_sa_selftest_timeout: a target that block
-    // bar_block, or every block if bar_block < 0, never reaches)
-    const unsigned int extra = (bar_block < 0 || (int)blockIdx.x == bar_block) ? bar_extra : 0u;
-    if (!sa_grid_barrier(bar, (unsigned int)(bi + 1) * gridDim.x + extra, status)) break;
 
-    const long long left = s_state.n_step - s_state.n_eval;
-    const int Kv = (int)min((long long)Keff, max(0LL, left));
+    // ---- the decision
     float de_star;
-    const int kstar = sa_first_accept(&s_state, Kv, partial, g.n_chunks, u, &de_star);
-    int acc_a = 0, acc_b = 0;
-    if (kstar >= 0) {
-      // every block drew the candidates itself and holds the last one
-      const int a = kstar == Keff - 1 ? last_a : __ldcg(pairs + 2 * kstar);
-      const int b = kstar == Keff - 1 ? last_b : __ldcg(pairs + 2 * kstar + 1);
-      acc_a = a;
-      acc_b = b;
-      if (a != b) {
-        // this block's vectors: apply the accepted candidate's changes
-        // (the block-wide lookups of the last candidate left its changes in ct.d)
-        const bool in_smem = held_k == kstar && held_k >= 0;
-        const int32_t* dk = dcounts + (int64_t)kstar * 2 * g.n_canon;
-        for (int i = threadIdx.x; i < nv; i += blockDim.x) {
-          const int v = v0 + i;
-          const int d0 = in_smem ? ct.d[i] : dk[v], d1 = in_smem ? ct.d[mv + i] : dk[(int64_t)g.n_canon + v];
-#pragma unroll
-          for (int p = 0; p < 2; ++p) {
-            const int d = p ? d1 : d0;
-            if (d == 0) continue;
-            const long long c = s_cnt[p * mv + i] + d;
-            s_cnt[p * mv + i] = c;
-            counts[p * g.n_full + g.base + v] = (unsigned long long)c;
-            if (v > 0) counts[p * g.n_full + (g.n_full - 1 - (g.base + v))] = (unsigned long long)c;
-          }
+    int kstar, acc_a = 0, acc_b = 0;
+    const bool ahead = fast && Keff == 1 && n0 + 1 < (unsigned long long)s_state.n_step && bi + 1 < n_batches;
+    // While the other blocks' messages are awaited, after a batch of one: warp
+    // 1 draws the next candidate for both ways the batch can end, warp 2 takes
+    // the schedule's step for both (lane 0: rejected, lane 1: accepted), and
+    // the others mark the vectors whose segments may hold both pixels.
+    SaStep step;
+    const bool flagged = fast && held_k >= 0 && nv <= 64;  // ct.term is free for the marks
+    int* s_maybe = reinterpret_cast<int*>(ct.term);
+    if (fast) {
+      if (ahead && warp == 1) {
+        SaCand c = draw(n0 + 1);
+        if (lane == 0) s_warp.drawn[0] = c;
+        if (last.a != last.b) {  // and on the cell after the exchange
+          delta_mark_pair(sm, last.q.ax, last.q.ay, 0, last.q.bx, last.q.by, 1, g, lane);
+          __syncwarp();
+          c = draw(n0 + 1);
+          __syncwarp();
+          delta_mark_pair(sm, last.q.ax, last.q.ay, 1, last.q.bx, last.q.by, 0, g, lane);
         }
-        // this block's vectors: the phase-0 counts follow the exchange
-        if (g.z) {
-          if (held_k == kstar) {
-            delta_chunk_apply_held(g, last_q, v0, ct, held, held_zi);
-          } else {
-            const PixelPair qk = {a % g.W, a / g.W, b % g.W, b / g.W};
-            delta_chunk_update(g, qk, v0, ct);
-          }
+        if (lane == 0) s_warp.drawn[1] = c;
+      } else if (ahead && warp == 2) {
+        if (lane < 2) step = sa_step(&s_state, Kv, lane - 1);
+      } else if (warp > 2) {
+        if (flagged) {
+          int ddx, ddy;
+          chunk_displacement(g, last.q, ddx, ddy);
+          const int i = (int)threadIdx.x - 96;
+          if (i < nv) s_maybe[i] = chunk_maybe_both(g, ct.vec[i].x, ct.vec[i].y, ddx, ddy);
         }
       }
+      // (s_pa, s_u of candidate k > 0 and s_kstar were written before a
+      // barrier of that candidate; candidate 0's by thread 0 of warp 0, whose
+      // own candidate it is)
+      if (warp < Kv) {
+        float de = 0.0f;
+        const bool ok = hear_messages(mail + (size_t)warp * g.n_chunks, g.n_chunks, (unsigned int)(bi + 1) + (extra << 30),
+                                      lane, &de);
+        if (!ok) {
+          if (lane == 0) { s_heard = 0; atomicOr(status, 4); }
+        } else if (lane == 0) {
+          const long long ck = s_state.c_stage + warp;
+          const long long wk = ck >= s_state.c_max ? ck / s_state.c_max : 0;  // stage ends before candidate k
+          const double Tk = wk ? s_state.T * pow(s_state.T_mult, (double)wk) : s_state.T;
+          s_de[warp] = de;
+          if (de <= 0.0f || s_u[warp] < expf(-de / (float)Tk)) atomicMin(&s_kstar, warp);
+        }
+      }
+      __syncthreads();
+      if (!s_heard) break;
+      kstar = s_kstar == INT_MAX ? -1 : s_kstar;
+      de_star = kstar >= 0 ? s_de[kstar] : 0.0f;
+      if (kstar >= 0) { acc_a = s_pa[kstar]; acc_b = s_pb[kstar]; }
+    } else {
+      if (ch == 0) __threadfence();  // the candidates, written by other threads than the one that arrives
+      ++n_bar;
+      if (!sa_grid_barrier(bar, n_bar * gridDim.x + extra, status)) break;
+      kstar = sa_first_accept(&s_state, Kv, partial, g.n_chunks, u, &de_star);
+      if (kstar >= 0) {
+        // every block drew the candidates itself and holds the last one
+        acc_a = kstar == Keff - 1 ? last.a : __ldcg(pairs + 2 * kstar);
+        acc_b = kstar == Keff - 1 ? last.b : __ldcg(pairs + 2 * kstar + 1);
+      }
     }
-    // warp 0 advances the run state (and block 0 writes the exchange to the
-    // cell); warp 1 makes the exchange on the block's cell copy and draws
-    // the next batch's first candidate on it
+    const bool swap = kstar >= 0 && acc_a != acc_b;
+
+    // ---- its consequences: warp 1 makes the exchange on the block's cell
+    // copy and settles the next batch's first candidate, warp 2 brings the run
+    // state up to date (block 0's warp 0 the cell), then all of them this
+    // block's counts
     if (warp == 0) {
-      if (lane == 0) {
-        if (ch == 0 && kstar >= 0 && acc_a != acc_b) {
+      if (ch == 0 && swap) {
+        const int ay = acc_a / g.W, by = acc_b / g.W;
+        if (lane == 0) {
           cell[acc_a] = 0;
           cell[acc_b] = 1;
-          delta_mark(ext, acc_a, 0, g);
-          delta_mark(ext, acc_b, 1, g);
         }
+        delta_mark_pair(ext, acc_a - ay * g.W, ay, 0, acc_b - by * g.W, by, 1, g, lane);
+        __syncwarp();
+      }
+    } else if (warp == 2) {
+      if (ahead) {
+        if (lane == (kstar >= 0 ? 1 : 0)) sa_settle(&s_state, step, Keff, kstar, de_star, acc_a, acc_b);
+      } else if (lane == 0) {
         sa_advance(&s_state, Keff, Kv, kstar, de_star, acc_a, acc_b);
       }
+      __syncwarp();
     } else if (warp == 1) {
-      if (lane == 0 && kstar >= 0 && acc_a != acc_b) {
-        delta_mark(sm, acc_a, 0, g);
-        delta_mark(sm, acc_b, 1, g);
+      if (swap) {
+        const int ay = acc_a / g.W, by = acc_b / g.W;
+        delta_mark_pair(sm, acc_a - ay * g.W, ay, 0, acc_b - by * g.W, by, 1, g, lane);
       }
       __syncwarp();
-      const unsigned long long n_next = n0 + (unsigned long long)(kstar >= 0 ? kstar + 1 : Kv);
-      if ((long long)n_next < s_state.n_step && bi + 1 < n_batches) draw(bi + 1, n_next, 0, &s_na, &s_nb, &s_nq);
+      if (ahead) {
+        if (lane == 0) take(bi + 1, 0, s_warp.drawn[swap ? 1 : 0], &s_next);
+      } else {
+        const unsigned long long n_next = n0 + (unsigned long long)(kstar >= 0 ? kstar + 1 : Kv);
+        if ((long long)n_next < s_state.n_step && bi + 1 < n_batches) {
+          const SaCand c = draw(n_next);
+          if (lane == 0) take(bi + 1, 0, c, &s_next);
+        }
+      }
+      __syncwarp();
+    }
+    // this block's vectors (the threads from warp 3 on first): the accepted
+    // candidate's changes, which the lookups of the last candidate left in
+    // ct.d; ct.d is zeroed for the next batch
+    const bool in_smem = held_k == kstar && held_k >= 0;
+    const int32_t* dk = dcounts + (int64_t)max(kstar, 0) * 2 * g.n_canon;
+    for (int i = ((int)threadIdx.x + (int)blockDim.x - 96) % (int)blockDim.x; i < nv; i += blockDim.x) {
+      const int v = v0 + i;
+      if (swap) {
+        const int d0 = in_smem ? ct.d[i] : dk[v], d1 = in_smem ? ct.d[mv + i] : dk[(int64_t)g.n_canon + v];
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+          const int d = p ? d1 : d0;
+          if (d == 0) continue;
+          const long long c = s_cnt[p * mv + i] + d;
+          s_cnt[p * mv + i] = c;
+          counts[p * g.n_full + g.base + v] = (unsigned long long)c;
+          if (v > 0) counts[p * g.n_full + (g.n_full - 1 - (g.base + v))] = (unsigned long long)c;
+        }
+      }
+      ct.d[i] = 0;
+      ct.d[mv + i] = 0;
+    }
+    // and the phase-0 counts follow the exchange
+    if (g.z && swap) {
+      if (held_k == kstar) {
+        delta_chunk_apply_held(g, last.q, v0, ct, held, held_zi, flagged ? s_maybe : nullptr);
+      } else {
+        const PixelPair qk = {acc_a % g.W, acc_a / g.W, acc_b % g.W, acc_b / g.W};
+        delta_chunk_update(g, qk, v0, ct);
+      }
     }
     __syncthreads();
   }
@@ -529,12 +699,13 @@ static size_t persistent_smem(const DeltaArgs& g) {
 // Launch the persistent annealer for nb batches (cooperative launch: every
 // block is resident, which its grid barrier relies on).
 static int launch_persistent(lpf_sa* sa, int nb, cudaStream_t s, unsigned int bar_extra = 0, int bar_block = -1) {
-  cudaError_t e = cudaMemsetAsync(sa->d_bar, 0, sizeof(unsigned int), s);
+  cudaError_t e = cudaMemsetAsync(sa->d_bar, 0, sa->bar_bytes, s);
   if (e != cudaSuccess) return set_cuda_error(e);
   unsigned long long* counts = reinterpret_cast<unsigned long long*>(sa->counts);
+  unsigned long long* msg = reinterpret_cast<unsigned long long*>(sa->d_bar + 4);
   int k_max = sa->prm.k_max;
   void* args[] = {&sa->d_st, &sa->cell, &sa->d_ext, &sa->g, &sa->d_pairs, &sa->d_u, &sa->d_dc, &sa->d_partial,
-                  &counts, &sa->d_status, &sa->d_bar, &nb, &k_max, &bar_extra, &bar_block};
+                  &counts, &sa->d_status, &sa->d_bar, &msg, &nb, &k_max, &bar_extra, &bar_block};
   e = cudaLaunchCooperativeKernel(sa_persistent_kernel_entry(), dim3(sa->g.n_chunks), dim3(kDeltaThreads), args,
                                   persistent_smem(sa->g), s);
   return set_cuda_error(e);
@@ -648,7 +819,8 @@ int sa_start(lpf_sa* sa, cudaStream_t s) {
   if (e == cudaSuccess) e = cudaMalloc(&sa->d_u, 2 * (size_t)prm->k_max * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&sa->d_de, (size_t)prm->k_max * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&sa->d_partial, 2 * (size_t)prm->k_max * nch * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc(&sa->d_bar, sizeof(unsigned int));
+  sa->bar_bytes = 16 + 2 * (size_t)kMsgCandidates * nch * sizeof(unsigned long long);
+  if (e == cudaSuccess) e = cudaMalloc(&sa->d_bar, sa->bar_bytes);
   if (e == cudaSuccess && sa->objective == kSaObjectiveLineal)
     e = cudaMalloc(&sa->d_dc, (size_t)prm->k_max * 2 * (size_t)sa->paths->host.n_canon * sizeof(int32_t));
   if (e == cudaSuccess) e = cudaMalloc(&sa->d_e, sizeof(double));

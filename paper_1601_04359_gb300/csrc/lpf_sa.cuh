@@ -150,7 +150,7 @@ __device__ __forceinline__ void draw_candidate_warp(const uint8_t* e, const Delt
 // block calls this.
 __device__ __forceinline__ int sa_first_accept(const SaDev* st, int Kv, const float* partial, int n_chunks,
                                                const float* u, float* de_star) {
-  __shared__ float s_de[32];
+  __shared__ float s_de[16];  // (blocks have at most 16 warps)
   __shared__ int s_kstar;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   if (threadIdx.x == 0) s_kstar = INT_MAX;
@@ -193,11 +193,17 @@ __device__ __forceinline__ int sa_first_accept(const SaDev* st, int Kv, const fl
   return kstar;
 }
 
-// Advance the run past a batch of Keff candidates of which Kv count (the
-// rest lie beyond n_step) and kstar (or -1) was accepted: stage counters,
-// temperature, error, statistics and the next batch size.  Thread 0 only.
-__device__ __forceinline__ void sa_advance(SaDev* st, int Keff, int Kv, int kstar, float de_star, int acc_a,
-                                           int acc_b) {
+// What a batch of Keff candidates, of which Kv count (the rest lie beyond
+// n_step) and kstar (or -1) is accepted, makes of the schedule: stage
+// counters, temperature, evaluations and the next batch size.
+struct SaStep {
+  double T, p_est;
+  long long c, s, n_eval;
+  int k_eff, done;
+};
+
+__device__ __forceinline__ SaStep sa_step(const SaDev* st, int Kv, int kstar) {
+  SaStep x;
   const long long c0 = st->c_stage, cmax = st->c_max;
   const double Tm = st->T_mult;
   const long long consumed = kstar >= 0 ? kstar + 1 : Kv;
@@ -214,6 +220,38 @@ __device__ __forceinline__ void sa_advance(SaDev* st, int Keff, int Kv, int ksta
     c += 1;
     s += 1;
     if (c >= cmax || s >= st->s_max) { c = 0; s = 0; T *= Tm; }
+  }
+  x.c = c;
+  x.s = s;
+  x.T = T;
+  x.n_eval = st->n_eval + consumed;
+  x.p_est = st->p_est;
+  if (consumed > 0) {
+    // (a double division only where it does something)
+    const double hit = kstar >= 0 ? 1.0 : 0.0;
+    const double obs = consumed == 1 ? hit : hit / (double)consumed;
+    x.p_est = 0.8 * st->p_est + 0.2 * obs;
+  }
+  // next batch size: a batch costs a fixed latency plus a share per
+  // candidate and yields (1 - (1-p)^K) / p evaluations; with the measured
+  // costs that ratio is best near K = 1/(2p)
+  const float want = ceilf(0.5f / fmaxf((float)x.p_est, 1e-9f));
+  x.k_eff = (int)fminf((float)st->k_max, fmaxf((float)st->k_min, want));
+  x.done = x.n_eval >= st->n_step ? 1 : st->done;
+  return x;
+}
+
+// The run state after that batch: the schedule, error and statistics.
+__device__ __forceinline__ void sa_settle(SaDev* st, const SaStep& x, int Keff, int kstar, float de_star, int acc_a,
+                                          int acc_b) {
+  st->c_stage = x.c;
+  st->s_stage = x.s;
+  st->T = x.T;
+  st->n_eval = x.n_eval;
+  st->p_est = x.p_est;
+  st->k_eff = x.k_eff;
+  st->done = x.done;
+  if (kstar >= 0) {
     st->acc_pair[0] = acc_a;
     st->acc_pair[1] = acc_b;
     st->acc_de = de_star;
@@ -224,23 +262,15 @@ __device__ __forceinline__ void sa_advance(SaDev* st, int Keff, int Kv, int ksta
     st->acc_pair[1] = 0;
     st->acc_de = 0.0f;
   }
-  st->c_stage = c;
-  st->s_stage = s;
-  st->T = T;
-  st->n_eval += consumed;
   st->n_cand += Keff;
   if (Keff > 0) st->n_batches += 1;
-  if (consumed > 0) {
-    const double obs = (kstar >= 0 ? 1.0 : 0.0) / (double)consumed;
-    st->p_est = 0.8 * st->p_est + 0.2 * obs;
-  }
-  // next batch size: a batch costs a fixed latency plus a share per
-  // candidate and yields (1 - (1-p)^K) / p evaluations; with the measured
-  // costs that ratio is best near K = 1/(2p)
-  const float want = ceilf(0.5f / fmaxf((float)st->p_est, 1e-9f));
-  st->k_eff = (int)fminf((float)st->k_max, fmaxf((float)st->k_min, want));
-  if (st->n_eval >= st->n_step) st->done = 1;
   st->ticket = 0u;
+}
+
+// Both at once.  One thread only.
+__device__ __forceinline__ void sa_advance(SaDev* st, int Keff, int Kv, int kstar, float de_star, int acc_a,
+                                           int acc_b) {
+  sa_settle(st, sa_step(st, Kv, kstar), Keff, kstar, de_star, acc_a, acc_b);
 }
 
 // The serial end of a batch works on a copy of the run state in shared
@@ -312,7 +342,8 @@ struct lpf_sa {
   int64_t err_n_full = 0, err_base = 0;  // error layout: [phase][err_n_full], summed from err_base
   int threads = 0;              // batch kernel block size
   int persistent = 0;           // batches run by the cooperative persistent kernel
-  unsigned int* d_bar = nullptr;  // its grid-barrier counter
+  unsigned int* d_bar = nullptr;  // its grid-barrier counter and, 16 bytes on, its messages
+  size_t bar_bytes = 0;
   uint8_t* d_sel_ext = nullptr; // Monte-Carlo runs: sampled translations, extended layout
   uint8_t* d_sel = nullptr;     // Monte-Carlo runs: the run's copy of the selection, H*W
   uint8_t* d_z = nullptr;       // phase-0 counts per (vector, translation), kept current by the run
