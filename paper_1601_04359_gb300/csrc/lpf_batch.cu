@@ -116,7 +116,7 @@ __device__ __forceinline__ uint32_t batch_unit(const BatchDesc& b, int bg, int t
   const int bl = tile / b.G, grp = tile - (tile / b.G) * b.G;
   const int y = (bg * b.BB + bl) * 32 + lane;
   const uint32_t* lane_base = sm + (bl * 32 + lane) * b.S + grp * T;
-  return walk_unit<T, GATHER, false>(b.prog, b.piece[pi], b.piece[pi + 1], lane_base, b.gather ? deal : nullptr, y, b.H, b.W, b.nw, grp * T,
+  return walk_unit<T, 1, GATHER, false>(b.prog, b.piece[pi], b.piece[pi + 1], lane_base, 0u, b.gather ? deal : nullptr, y, b.H, b.W, b.nw, grp * T,
                              nullptr, lane, b.counts, b.n_full, b.base);
 }
 

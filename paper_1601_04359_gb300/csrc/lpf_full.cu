@@ -48,16 +48,18 @@ constexpr int kCtlUnits = 4;
 constexpr int kMaxBandGroups = 8192;  // images: ceil(H / 32) <= 256; volumes: D * ceil(H / (32 BB))
 constexpr int kCtlWords = kCtlUnits + kMaxBandGroups;
 
-int layout_side(int H, int W, int rx, int ry, int T, int BB, Geometry& g, int up) {
+int layout_side(int H, int W, int rx, int ry, int T, int BB, Geometry& g, int up, int R) {
   g.H = H; g.W = W; g.rx = rx; g.ry = ry; g.up = up;
   g.nw = (W + 31) / 32;
+  const int TW = T / R;  // words of a row per thread
   g.T = T;
-  g.G = (g.nw + T - 1) / T;
+  g.R = R;
+  g.G = (g.nw + TW - 1) / TW;
   g.nbands = (H + 31) / 32;
   g.BB = std::max(1, std::min(BB, g.nbands));
   g.nbg = (g.nbands + g.BB - 1) / g.BB;
   g.r32 = ((rx + 31) / 32) * 32;
-  const int nwp = g.G * T;
+  const int nwp = g.G * TW;
   g.S = nwp + ((g.r32 + rx) >> 5) + 1;
   if ((g.S & 1) == 0) g.S += 1;
   g.rows = 32 * g.BB * g.nbg + ry + up;
@@ -70,6 +72,19 @@ int layout_side(int H, int W, int rx, int ry, int T, int BB, Geometry& g, int up
   g.nbg_s = g.nbg;
   if (band > (size_t)kMaxSmem - 64) return LPF_EUNSUPPORTED;
   return LPF_OK;
+}
+
+// Rows narrower than a thread's T = 8 words leave words without translations;
+// where BB bands can be folded R at a time, a tile takes R bands instead (the
+// decoding of records, most of the walk of short segments, then serves twice
+// the words: 128^3, window 16: 2.75 -> 1.98 ms).
+static int fold(int T, int W, int H, int BB) {
+  if (T != 8) return 1;
+  const int nw = (W + 31) / 32;
+  BB = std::max(1, std::min(BB, (H + 31) / 32));
+  int R = 1;
+  while (R < 4 && T / (2 * R) >= nw && BB % (2 * R) == 0) R *= 2;
+  return R;
 }
 
 int make_geometry(int H, int W, int rx, int ry, int T, int BB, Geometry& g) {
@@ -89,19 +104,23 @@ int make_sides(const Paths& paths, int H, int W, int T, int BB, Sides& s) {
   int rc = make_geometry(H, W, rx, std::min(rx, ry), T, BB, s.g[0]);
   if (rc) return rc;
   s.n = paths.root_t >= 0 ? 2 : 1;
+  // (one kernel walks both sides: both are folded alike)
+  int R = fold(s.g[0].T, W, H, s.g[0].BB);
+  if (s.n == 2) R = std::min(R, fold(s.g[0].T, H, W, s.g[0].BB));
+  if (R > 1 && (rc = layout_side(H, W, rx, std::min(rx, ry), s.g[0].T, s.g[0].BB, s.g[0], 0, R))) return rc;
   s.off1 = (s.g[0].packed_words + 3) & ~size_t(3);
   s.packed_words = s.g[0].packed_words;
   s.band_bytes = s.g[0].band_bytes;
   s.nbg = s.g[0].nbg;
-  int tiles = s.g[0].G * s.g[0].BB;
+  int tiles = tiles_of(s.g[0]);
   if (s.n == 2) {
     const int h = std::min(rx, ry - 1);  // transposed segments: row offsets -h .. h
-    rc = layout_side(W, H, ry, h, s.g[0].T, s.g[0].BB, s.g[1], h);
+    rc = layout_side(W, H, ry, h, s.g[0].T, s.g[0].BB, s.g[1], h, R);
     if (rc) return rc;
     s.packed_words = s.off1 + s.g[1].packed_words;
     s.band_bytes = std::max(s.band_bytes, s.g[1].band_bytes);
     s.nbg += s.g[1].nbg;
-    tiles = std::max(tiles, s.g[1].G * s.g[1].BB);
+    tiles = std::max(tiles, tiles_of(s.g[1]));
   }
   // One warp per tile, at most 16; more (warps take units of any tile of the
   // band group) where the staged rows let few blocks share an SM, up to the
@@ -137,8 +156,18 @@ static int stack_images(Sides& s, int n) {
 // (z, b) stages rows z * slice_rows + 32 BB b onwards: its 32 BB
 // translation rows, ry above and below them, and the rz following slices.
 int make_geometry3(int D, int H, int W, int rx, int ry, int rz, int T, int BB, Geometry& g) {
+  if (T <= 0 && W > 64 && W <= 128 && H > 32 && ((H + 31) / 32) % 2 == 0) {
+    // two bands per tile (a window this size stages few bands either way)
+    T = 8;
+    if (BB <= 0) BB = 4;
+    if (((H + 31) / 32) % 4 != 0) BB = 2;
+  }
   int rc = make_geometry(H, W, rx, ry, T, BB, g);
   if (rc && rc != LPF_EUNSUPPORTED) return rc;
+  if (const int R = fold(g.T, W, H, g.BB); R > 1) {
+    rc = layout_side(H, W, rx, ry, g.T, g.BB, g, 0, R);
+    if (rc && rc != LPF_EUNSUPPORTED) return rc;
+  }
   g.D = D;
   g.rz = rz;
   g.nbg_s = g.nbg;
@@ -275,7 +304,7 @@ __global__ void pack_sel_kernel(const uint8_t* __restrict__ sel, int Ho, int Wo,
 struct WalkSide {
   const uint32_t* packed;
   const uint32_t* sel;  // packed translation selection, or null
-  int H, W, S, nw, G, BB;
+  int H, W, S, nw, G, BB, tiles;
   int nbg, nbg_s, slice_rows;
   int piece0, n_pieces;
   uint32_t band_bytes;
@@ -288,15 +317,15 @@ struct WalkSides {
 
 // The units of band group lbg of side sd, pulled from its counter ctr until
 // none is left: unit u is the side's program piece u / n_tiles on tile
-// u % n_tiles (tile = one band and one group of T words, i.e. 32 rows x 32T
-// translations).  Returns the pixel words this warp ANDed.
-template <int T, bool GATHER>
+// u % n_tiles (tile = R bands and one group of T / R words, i.e. 32 R rows x
+// 32 T / R translations).  Returns the pixel words this warp ANDed.
+template <int T, int R, bool GATHER>
 __device__ __forceinline__ unsigned long long walk_band(const WalkSide& sd, int lbg, int* ctr, const uint32_t* sm,
                                                         uint2* deal, int lane, const uint4* __restrict__ prog,
                                                         const uint32_t* __restrict__ piece,
                                                         unsigned long long* __restrict__ counts, int64_t n_full,
                                                         int64_t base) {
-  const int n_tiles = sd.G * sd.BB;
+  const int n_tiles = sd.tiles;
   const int units = n_tiles * sd.n_pieces;
   unsigned long long executed = 0;
   for (;;) {
@@ -305,11 +334,11 @@ __device__ __forceinline__ unsigned long long walk_band(const WalkSide& sd, int 
     u = __shfl_sync(0xffffffffu, u, 0);
     if (u >= units) break;
     const int tile = u % n_tiles, pi = sd.piece0 + u / n_tiles;
-    const int bl = tile / sd.G, grp = tile - bl * sd.G;
-    const uint32_t* lane_base = sm + (bl * 32 + lane) * sd.S + grp * T;
+    const int row = tile / sd.G, grp = tile - row * sd.G, bl = row * R;
+    const uint32_t* lane_base = sm + (bl * 32 + lane) * sd.S + grp * (T / R);
     const int y = ((lbg % sd.nbg_s) * sd.BB + bl) * 32 + lane;  // translation row within the slice
-    executed += walk_unit<T, GATHER>(prog, piece[pi], piece[pi + 1], lane_base, deal, y, sd.H, sd.W, sd.nw, grp * T, sd.sel,
-                             lane, counts, n_full, base);
+    executed += walk_unit<T, R, GATHER>(prog, piece[pi], piece[pi + 1], lane_base, 128u * (uint32_t)sd.S, deal, y, sd.H,
+                                        sd.W, sd.nw, grp * (T / R), sd.sel, lane, counts, n_full, base);
   }
   return executed;
 }
@@ -325,7 +354,7 @@ __device__ __forceinline__ unsigned long long walk_band(const WalkSide& sd, int 
 // block barrier per move).  The launch bounds cap a thread at 64 registers
 // (two 512-thread blocks per SM), which keeps 32 warps resident per SM to
 // hide the latency of the shared-memory word loads.
-template <int T, bool GATHER>
+template <int T, int R, bool GATHER>
 __global__ void __launch_bounds__(512, 2) walk_kernel(const __grid_constant__ WalkSides ws, const uint4* __restrict__ prog,
                                                   const uint32_t* __restrict__ piece,
                                                   unsigned long long* __restrict__ counts, int64_t n_full,
@@ -358,7 +387,7 @@ __global__ void __launch_bounds__(512, 2) walk_kernel(const __grid_constant__ Wa
           if (k0 + lane < n_bg) {
             const int bt = (int)((blockIdx.x + (unsigned)(k0 + lane)) % (unsigned)n_bg);
             const WalkSide& st = ws.s[bt >= ws.s[0].nbg];
-            left = *reinterpret_cast<volatile int*>(unit_ctr + bt) < st.G * st.BB * st.n_pieces;
+            left = *reinterpret_cast<volatile int*>(unit_ctr + bt) < st.tiles * st.n_pieces;
           }
           const uint32_t m = __ballot_sync(0xffffffffu, left);
           if (m) found = k0 + __ffs(m) - 1;
@@ -392,9 +421,9 @@ __global__ void __launch_bounds__(512, 2) walk_kernel(const __grid_constant__ Wa
     // 175x201); without it two copies, with the side's fields as constants,
     // are the faster ones (18.4 and 18.9 us at 64x64, window 32).
     unsigned long long walked;
-    if (GATHER) walked = walk_band<T, GATHER>(sd, lbg, unit_ctr + bg, sm, deal, lane, prog, piece, counts, n_full, base);
-    else if (side) walked = walk_band<T, GATHER>(ws.s[1], lbg, unit_ctr + bg, sm, deal, lane, prog, piece, counts, n_full, base);
-    else walked = walk_band<T, GATHER>(ws.s[0], lbg, unit_ctr + bg, sm, deal, lane, prog, piece, counts, n_full, base);
+    if (GATHER) walked = walk_band<T, R, GATHER>(sd, lbg, unit_ctr + bg, sm, deal, lane, prog, piece, counts, n_full, base);
+    else if (side) walked = walk_band<T, R, GATHER>(ws.s[1], lbg, unit_ctr + bg, sm, deal, lane, prog, piece, counts, n_full, base);
+    else walked = walk_band<T, R, GATHER>(ws.s[0], lbg, unit_ctr + bg, sm, deal, lane, prog, piece, counts, n_full, base);
     if (lbg >= sd.work_from) executed += walked;
     __syncthreads();  // every warp is done with the staged band before it may be replaced
   }
@@ -540,7 +569,7 @@ static Which tree_pieces(const lpf_paths* p, const Sides& sd, int n_img) {
   if (p->host.fine.piece_begin.size() < 2) return Which::kTree;
   int64_t units = 0;
   for (int q = 0; q < sd.n; ++q)
-    units += (int64_t)sd.g[q].nbg_s * n_img * sd.g[q].G * sd.g[q].BB *
+    units += (int64_t)sd.g[q].nbg_s * n_img * tiles_of(sd.g[q]) *
              ((int64_t)side_program(p, Which::kTree, q).piece_begin.size() - 1);
   return units < 32 * (int64_t)g_num_sms ? Which::kFine : Which::kTree;
 }
@@ -554,12 +583,15 @@ static int bake_sides(lpf_paths* p, const Sides& sd, Which w) {
 using WalkFn = void (*)(const WalkSides, const uint4*, const uint32_t*, unsigned long long*, int64_t, int64_t, int*,
                         uint32_t, int, uint32_t, uint32_t);
 
-static WalkFn walk_fn(int T, bool gather) {
+static WalkFn walk_fn(int T, int R, bool gather) {
   switch (T) {
-    case 1: return walk_kernel<1, false>;
-    case 2: return gather ? walk_kernel<2, true> : walk_kernel<2, false>;
-    case 4: return gather ? walk_kernel<4, true> : walk_kernel<4, false>;
-    default: return gather ? walk_kernel<8, true> : walk_kernel<8, false>;
+    case 1: return walk_kernel<1, 1, false>;
+    case 2: return gather ? walk_kernel<2, 1, true> : walk_kernel<2, 1, false>;
+    case 4: return gather ? walk_kernel<4, 1, true> : walk_kernel<4, 1, false>;
+    default:
+      if (R == 4) return gather ? walk_kernel<8, 4, true> : walk_kernel<8, 4, false>;
+      if (R == 2) return gather ? walk_kernel<8, 2, true> : walk_kernel<8, 2, false>;
+      return gather ? walk_kernel<8, 1, true> : walk_kernel<8, 1, false>;
   }
 }
 
@@ -586,8 +618,9 @@ static void set_kernel_attributes() {
   if (e != cudaSuccess) { g_attr_status = set_cuda_error(e); return; }
   int rc = LPF_OK;
   for (int T : {1, 2, 4, 8})
-    for (bool gather : {false, true})
-      if (!rc) rc = allow_smem(walk_fn(T, gather), optin, g_max_dyn_smem);
+    for (int R : {1, 2, 4})
+      for (bool gather : {false, true})
+        if (!rc) rc = allow_smem(walk_fn(T, R, gather), optin, g_max_dyn_smem);
   g_attr_status = rc;
 }
 
@@ -601,7 +634,7 @@ static uint32_t walk_smem(const Sides& sd) {
 static int walk_blocks_for(const Sides& sd) {
   int per_sm = 0;
   const uint32_t smem = walk_smem(sd);
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, walk_fn(sd.g[0].T, smem > sd.band_bytes),
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, walk_fn(sd.g[0].T, sd.g[0].R, smem > sd.band_bytes),
                                                                 sd.threads, smem);
   if (e != cudaSuccess) return -set_cuda_error(e);
   return std::max(1, per_sm) * g_num_sms;
@@ -619,12 +652,12 @@ static uint32_t selftest_wait_rounds(const lpf_paths* p) { return p->selftest ? 
 static void walk_sides(const Sides& sd, const Baked& b, const uint32_t* packed, const uint32_t* sel0,
                        const uint32_t* sel1, bool work_from, WalkSide& w0, WalkSide& w1) {
   const Geometry& g0 = sd.g[0];
-  w0 = WalkSide{packed, sel0, g0.H, g0.W, g0.S, g0.nw, g0.G, g0.BB, g0.nbg, g0.nbg_s, g0.slice_rows,
+  w0 = WalkSide{packed, sel0, g0.H, g0.W, g0.S, g0.nw, g0.G, g0.BB, tiles_of(g0), g0.nbg, g0.nbg_s, g0.slice_rows,
                 0, b.n_pieces0, g0.band_bytes, work_from ? g0.nbg - g0.nbg_s : 0};
   w1 = WalkSide{};
   if (sd.n == 2) {
     const Geometry& g1 = sd.g[1];
-    w1 = WalkSide{packed + sd.off1, sel1, g1.H, g1.W, g1.S, g1.nw, g1.G, g1.BB, g1.nbg, g1.nbg_s, g1.slice_rows,
+    w1 = WalkSide{packed + sd.off1, sel1, g1.H, g1.W, g1.S, g1.nw, g1.G, g1.BB, tiles_of(g1), g1.nbg, g1.nbg_s, g1.slice_rows,
                   b.n_pieces0, b.n_pieces - b.n_pieces0, g1.band_bytes, work_from ? g1.nbg - g1.nbg_s : 0};
   }
 }
@@ -641,8 +674,8 @@ static void launch_walk(const Sides& sd, const Baked& b, const uint32_t* packed,
   // warp for each of its units, no block has to look for another one.
   int steal = 0;
   for (const WalkSide& q : w.s)
-    if (q.nbg > 0 && (int64_t)(blocks / sd.nbg) * (sd.threads / 32) < (int64_t)q.G * q.BB * q.n_pieces) steal = 1;
-  walk_fn(sd.g[0].T, deal_at != 0u)<<<blocks, sd.threads, smem, s>>>(w, prog, b.d_piece, c, n_full, base, ctl,
+    if (q.nbg > 0 && (int64_t)(blocks / sd.nbg) * (sd.threads / 32) < (int64_t)q.tiles * q.n_pieces) steal = 1;
+  walk_fn(sd.g[0].T, sd.g[0].R, deal_at != 0u)<<<blocks, sd.threads, smem, s>>>(w, prog, b.d_piece, c, n_full, base, ctl,
                                                                      deal_at, steal, xt, wr);
 }
 
@@ -733,8 +766,8 @@ static int run_full(const uint8_t* img, int H, int W, lpf_paths* p, int64_t* cou
   }
   unsigned long long* c = reinterpret_cast<unsigned long long*>(counts);
   // every warp walks every piece of its side
-  p->nominal_pixels = prog0.n_pixel_words * one.g[0].nbg * one.g[0].G * one.g[0].BB;
-  if (one.n == 2) p->nominal_pixels += prog1.n_pixel_words * one.g[1].nbg * one.g[1].G * one.g[1].BB;
+  p->nominal_pixels = prog0.n_pixel_words * one.g[0].nbg * tiles_of(one.g[0]);
+  if (one.n == 2) p->nominal_pixels += prog1.n_pixel_words * one.g[1].nbg * tiles_of(one.g[1]);
   if (p->ev_start) cudaEventRecord(p->ev_start, s);
   launch_walk(sd, b, p->d_packed, sel0, sel1, c, n_full, base, p->d_status, p, blocks, s);
   if (p->ev_stop) cudaEventRecord(p->ev_stop, s);
@@ -786,11 +819,11 @@ static int autotune_full(const uint8_t* img, int H, int W, lpf_paths* p, int64_t
   int bt = 0, bb = 0;
   int rc = LPF_OK;
   for (int T : {1, 2, 4, 8}) {
-    if (T > 1 && (T / 2) >= nw) continue;          // more words per thread than a row has
     for (int BB : {1, 2, 4, 8}) {
       Sides sd;
       if (make_sides(p->host, H, W, T, BB, sd) != LPF_OK) continue;
       if (sd.g[0].T != T || sd.g[0].BB != BB) continue;  // shape not admissible as asked
+      if (sd.g[0].R == 1 && T > 1 && (T / 2) >= nw) continue;  // more words per thread than a row has
       if ((int)sd.band_bytes > g_max_dyn_smem && g_max_dyn_smem > 0) continue;
       rc = run_full(img, H, W, p, counts, s, false, T, BB);  // warm-up (uploads tables)
       if (rc) break;
@@ -876,7 +909,7 @@ static int run_full3(const uint8_t* vol, int D, int H, int W, lpf_paths* p, int6
                                             p->checked ? p->d_status : nullptr);
   }
   unsigned long long* c = reinterpret_cast<unsigned long long*>(counts);
-  p->nominal_pixels = prog.n_pixel_words * g.nbg * g.G * g.BB;
+  p->nominal_pixels = prog.n_pixel_words * g.nbg * tiles_of(g);
   if (p->ev_start) cudaEventRecord(p->ev_start, s);
   launch_walk(sd, p->tree, p->d_packed, nullptr, nullptr, c, n_full, base, p->d_status, p, blocks, s);
   if (p->ev_stop) cudaEventRecord(p->ev_stop, s);

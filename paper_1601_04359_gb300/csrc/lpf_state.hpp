@@ -19,7 +19,8 @@ struct Geometry {
   int H = 0, W = 0, rx = 0, ry = 0;
   int nw = 0;      // words holding the W translations of a row
   int T = 0;       // words per thread
-  int G = 0;       // warps per band (word groups), G*T >= nw
+  int R = 1;       // bands per tile: a thread holds T / R words of each of R rows, 32 rows apart
+  int G = 0;       // word groups of a row, G*T/R >= nw
   int BB = 0;      // 32-row bands per block
   int nbg = 0;     // block-band groups = ceil(nbands / BB)
   int r32 = 0;     // rx rounded up to a multiple of 32
@@ -40,7 +41,9 @@ struct Geometry {
 int make_geometry(int H, int W, int rx, int ry, int T, int BB, Geometry& g);
 // The layout of one side for a fixed shape (T words per thread, BB bands per
 // block, clamped to the bands there are).
-int layout_side(int H, int W, int rx, int ry, int T, int BB, Geometry& g, int up = 0);
+int layout_side(int H, int W, int rx, int ry, int T, int BB, Geometry& g, int up = 0, int R = 1);
+// Tiles of a band group.
+inline int tiles_of(const Geometry& g) { return g.G * (g.BB / g.R); }
 
 // The sides of an image evaluation: side 0 walks the image's program (the
 // x-major vectors; column offsets up to rx, row offsets 0 .. min(rx, ry)),

@@ -38,50 +38,61 @@ namespace lpf {
 
 constexpr int kWalkStack = 24;
 
-// The T + 1 staged words of a pixel word's window.
-template <int T>
-__device__ __forceinline__ void load_window(const uint32_t* lane_base, uint32_t pix, uint32_t (&w)[T + 1]) {
-  const uint32_t* s = lane_word(lane_base, pix);
+// A lane's T words: T / R words of each of R rows 32 rows apart (R > 1 folds
+// the bands of narrow images into one tile, see layout_side); word t of the
+// window is w[win<T, R>(t)] and its successor.
+template <int T, int R>
+__device__ __forceinline__ constexpr int win(int t) { return t + t / (T / R); }
+
+// The R (T / R + 1) staged words of a pixel word's window; band: bytes from
+// one of the lane's rows to the next.
+template <int T, int R>
+__device__ __forceinline__ void load_window(const uint32_t* lane_base, uint32_t pix, uint32_t band,
+                                            uint32_t (&w)[T + R]) {
 #pragma unroll
-  for (int t = 0; t <= T; ++t) w[t] = s[t];
+  for (int r = 0; r < R; ++r) {
+    const uint32_t* s = reinterpret_cast<const uint32_t*>(reinterpret_cast<const char*>(lane_word(lane_base, pix)) + r * band);
+#pragma unroll
+    for (int t = 0; t <= T / R; ++t) w[r * (T / R + 1) + t] = s[t];
+  }
 }
 
 // Four single pixels (one group).
-template <int T>
-__device__ __forceinline__ void walk_singles4(const uint32_t* lane_base, uint4 P, uint32_t (&m1)[T],
+template <int T, int R>
+__device__ __forceinline__ void walk_singles4(const uint32_t* lane_base, uint32_t band, uint4 P, uint32_t (&m1)[T],
                                               uint32_t (&m0)[T]) {
   if (T <= 4) {
-    uint32_t wa[T + 1], wb[T + 1], wc[T + 1], wd[T + 1];
-    load_window<T>(lane_base, P.x, wa);
-    load_window<T>(lane_base, P.y, wb);
-    load_window<T>(lane_base, P.z, wc);
-    load_window<T>(lane_base, P.w, wd);
+    uint32_t wa[T + R], wb[T + R], wc[T + R], wd[T + R];
+    load_window<T, R>(lane_base, P.x, band, wa);
+    load_window<T, R>(lane_base, P.y, band, wb);
+    load_window<T, R>(lane_base, P.z, band, wc);
+    load_window<T, R>(lane_base, P.w, band, wd);
 #pragma unroll
     for (int t = 0; t < T; ++t) {
-      const uint32_t a = __funnelshift_r(wa[t], wa[t + 1], P.x);
-      const uint32_t b = __funnelshift_r(wb[t], wb[t + 1], P.y);
-      const uint32_t c = __funnelshift_r(wc[t], wc[t + 1], P.z);
-      const uint32_t d = __funnelshift_r(wd[t], wd[t + 1], P.w);
+      const uint32_t a = __funnelshift_r(wa[win<T, R>(t)], wa[win<T, R>(t) + 1], P.x);
+      const uint32_t b = __funnelshift_r(wb[win<T, R>(t)], wb[win<T, R>(t) + 1], P.y);
+      const uint32_t c = __funnelshift_r(wc[win<T, R>(t)], wc[win<T, R>(t) + 1], P.z);
+      const uint32_t d = __funnelshift_r(wd[win<T, R>(t)], wd[win<T, R>(t) + 1], P.w);
       m1[t] = (m1[t] & a & b) & c & d;
       m0[t] = (m0[t] & ~a & ~b) & ~c & ~d;
     }
   } else {  // two pixels at a time (registers)
-    uint32_t wa[T + 1], wb[T + 1];
-    load_window<T>(lane_base, P.x, wa);
-    load_window<T>(lane_base, P.y, wb);
+    uint32_t wa[T + R], wb[T + R];
+    load_window<T, R>(lane_base, P.x, band, wa);
+    load_window<T, R>(lane_base, P.y, band, wb);
 #pragma unroll
     for (int t = 0; t < T; ++t) {
-      const uint32_t a = __funnelshift_r(wa[t], wa[t + 1], P.x);
-      const uint32_t b = __funnelshift_r(wb[t], wb[t + 1], P.y);
+      const uint32_t a = __funnelshift_r(wa[win<T, R>(t)], wa[win<T, R>(t) + 1], P.x);
+      const uint32_t b = __funnelshift_r(wb[win<T, R>(t)], wb[win<T, R>(t) + 1], P.y);
       m1[t] = m1[t] & a & b;
       m0[t] = m0[t] & ~a & ~b;
     }
-    load_window<T>(lane_base, P.z, wa);
-    load_window<T>(lane_base, P.w, wb);
+    load_window<T, R>(lane_base, P.z, band, wa);
+    load_window<T, R>(lane_base, P.w, band, wb);
 #pragma unroll
     for (int t = 0; t < T; ++t) {
-      const uint32_t a = __funnelshift_r(wa[t], wa[t + 1], P.z);
-      const uint32_t b = __funnelshift_r(wb[t], wb[t + 1], P.w);
+      const uint32_t a = __funnelshift_r(wa[win<T, R>(t)], wa[win<T, R>(t) + 1], P.z);
+      const uint32_t b = __funnelshift_r(wb[win<T, R>(t)], wb[win<T, R>(t) + 1], P.w);
       m1[t] = m1[t] & a & b;
       m0[t] = m0[t] & ~a & ~b;
     }
@@ -89,31 +100,31 @@ __device__ __forceinline__ void walk_singles4(const uint32_t* lane_base, uint4 P
 }
 
 // Two single pixels.
-template <int T>
-__device__ __forceinline__ void walk_singles2(const uint32_t* lane_base, uint32_t p, uint32_t q, uint32_t (&m1)[T],
+template <int T, int R>
+__device__ __forceinline__ void walk_singles2(const uint32_t* lane_base, uint32_t band, uint32_t p, uint32_t q, uint32_t (&m1)[T],
                                               uint32_t (&m0)[T]) {
-  uint32_t wa[T + 1], wb[T + 1];
-  load_window<T>(lane_base, p, wa);
-  load_window<T>(lane_base, q, wb);
+  uint32_t wa[T + R], wb[T + R];
+  load_window<T, R>(lane_base, p, band, wa);
+  load_window<T, R>(lane_base, q, band, wb);
 #pragma unroll
   for (int t = 0; t < T; ++t) {
-    const uint32_t a = __funnelshift_r(wa[t], wa[t + 1], p);
-    const uint32_t b = __funnelshift_r(wb[t], wb[t + 1], q);
+    const uint32_t a = __funnelshift_r(wa[win<T, R>(t)], wa[win<T, R>(t) + 1], p);
+    const uint32_t b = __funnelshift_r(wb[win<T, R>(t)], wb[win<T, R>(t) + 1], q);
     m1[t] = m1[t] & a & b;
     m0[t] = m0[t] & ~a & ~b;
   }
 }
 
 // Two pairs {window|shift1, shift2} (one group): one window per pair.
-template <int T>
-__device__ __forceinline__ void walk_pairs2(const uint32_t* lane_base, uint4 P, uint32_t (&m1)[T], uint32_t (&m0)[T]) {
-  uint32_t wa[T + 1], wb[T + 1];
-  load_window<T>(lane_base, P.x, wa);
-  load_window<T>(lane_base, P.z, wb);
+template <int T, int R>
+__device__ __forceinline__ void walk_pairs2(const uint32_t* lane_base, uint32_t band, uint4 P, uint32_t (&m1)[T], uint32_t (&m0)[T]) {
+  uint32_t wa[T + R], wb[T + R];
+  load_window<T, R>(lane_base, P.x, band, wa);
+  load_window<T, R>(lane_base, P.z, band, wb);
 #pragma unroll
   for (int t = 0; t < T; ++t) {
-    const uint32_t a1 = __funnelshift_r(wa[t], wa[t + 1], P.x), a2 = __funnelshift_r(wa[t], wa[t + 1], P.y);
-    const uint32_t b1 = __funnelshift_r(wb[t], wb[t + 1], P.z), b2 = __funnelshift_r(wb[t], wb[t + 1], P.w);
+    const uint32_t a1 = __funnelshift_r(wa[win<T, R>(t)], wa[win<T, R>(t) + 1], P.x), a2 = __funnelshift_r(wa[win<T, R>(t)], wa[win<T, R>(t) + 1], P.y);
+    const uint32_t b1 = __funnelshift_r(wb[win<T, R>(t)], wb[win<T, R>(t) + 1], P.z), b2 = __funnelshift_r(wb[win<T, R>(t)], wb[win<T, R>(t) + 1], P.w);
     m1[t] = (m1[t] & a1 & a2) & b1 & b2;
     m0[t] = (m0[t] & ~a1 & ~a2) & ~b1 & ~b2;
   }
@@ -267,15 +278,15 @@ constexpr int kMaxLive = 32;  // one mask per lane (16: 2.18 instead of 1.97 ms 
 // 100x128, 6 %); at window 128 a third of the walk is gathered.
 constexpr int kGatherWindow = 64;
 
-// Valid translations of a tile: word t of the lane's row holds translations
-// x = 32 (j0 + t) + bit; those with x < W in a row y < H exist (and, with a
-// selection, only the selected ones).
-template <int T>
-__device__ __forceinline__ void tile_valid(int y, int H, int W, int nw, int j0, const uint32_t* __restrict__ sel,
+// Valid translations of a tile: word t of the lane (row y + 32 (t / (T / R)))
+// holds translations x = 32 (j0 + t mod T / R) + bit; those with x < W in a
+// row < H exist (and, with a selection, only the selected ones).
+template <int T, int R>
+__device__ __forceinline__ void tile_valid(int y0, int H, int W, int nw, int j0, const uint32_t* __restrict__ sel,
                                            uint32_t (&v)[T]) {
 #pragma unroll
   for (int t = 0; t < T; ++t) {
-    const int j = j0 + t;
+    const int j = j0 + t % (T / R), y = y0 + 32 * (t / (T / R));
     uint32_t m = 0;
     if (y < H && j < nw) {
       const int rem = W - 32 * j;
@@ -287,23 +298,24 @@ __device__ __forceinline__ void tile_valid(int y, int H, int W, int nw, int j0, 
 }
 
 // Walk program groups [pc, end) for this warp's tile.  lane_base: the lane's
-// first staged word (shared memory; row = the lane's translation row); deal:
+// first staged word (shared memory; row = the lane's first translation row),
+// band: bytes to its next row (R > 1); deal:
 // 32 entries of the warp's own for re-dealing its masks (GATHER), or null
 // (never re-deals).  Counts go to counts[base + vec] (phase 0) and counts[n_full +
 // base + vec] (phase 1).  Returns the pixels this warp walked (for the work
 // statistics).
 // UNROLL4: pair groups four per loop iteration (less loop control, more
 // code: the batched kernel keeps two).
-template <int T, bool GATHER, bool UNROLL4 = true>
+template <int T, int R, bool GATHER, bool UNROLL4 = true>
 __device__ __forceinline__ uint32_t walk_unit(const uint4* __restrict__ prog, uint32_t pc, uint32_t end,
-                                              const uint32_t* lane_base, uint2* deal, int y, int H, int W, int nw,
+                                              const uint32_t* lane_base, uint32_t band, uint2* deal, int y, int H, int W, int nw,
                                               int j0, const uint32_t* __restrict__ sel, int lane,
                                               unsigned long long* __restrict__ counts, int64_t n_full,
                                               int64_t base) {
   constexpr bool kGather = GATHER && T >= 2;  // (one word per lane already: nothing to win)
   uint32_t m1[T], m0[T];
   uint32_t st1[kWalkStack][T], st0[kWalkStack][T];
-  tile_valid<T>(y, H, W, nw, j0, sel, m1);
+  tile_valid<T, R>(y, H, W, nw, j0, sel, m1);
 #pragma unroll
   for (int t = 0; t < T; ++t) m0[t] = m1[t];
   uint32_t walked = 0;
@@ -326,8 +338,9 @@ __device__ __forceinline__ uint32_t walk_unit(const uint4* __restrict__ prog, ui
     const uint32_t word = smem_u32(lane_base);
 #pragma unroll
     for (int t = 0; t < T; ++t) {
-      if (m1[t]) deal[at++] = make_uint2(word + 4u * t, m1[t]);
-      if (m0[t]) deal[at++] = make_uint2((word + 4u * t) | 1u, m0[t]);
+      const uint32_t at_t = word + band * (t / (T / R)) + 4u * (t % (T / R));
+      if (m1[t]) deal[at++] = make_uint2(at_t, m1[t]);
+      if (m0[t]) deal[at++] = make_uint2(at_t | 1u, m0[t]);
     }
     __syncwarp();
     const uint2 d = lane < n ? deal[lane] : make_uint2(word, 0u);
@@ -346,7 +359,7 @@ __device__ __forceinline__ uint32_t walk_unit(const uint4* __restrict__ prog, ui
     const int vec = (int)hd.y;
     hd = next < end ? __ldg(prog + next) : make_uint4(0u, 0u, 0u, 0u);  // fetched while this record runs
     if (hdr & kReset) {
-      tile_valid<T>(y, H, W, nw, j0, sel, m1);
+      tile_valid<T, R>(y, H, W, nw, j0, sel, m1);
 #pragma unroll
       for (int t = 0; t < T; ++t) m0[t] = m1[t];
     }
@@ -365,15 +378,15 @@ __device__ __forceinline__ uint32_t walk_unit(const uint4* __restrict__ prog, ui
     uint32_t q = 0;
     for (; UNROLL4 && q + 4u <= n_pg; q += 4u) {
       const uint4 P0 = __ldg(g + q), P1 = __ldg(g + q + 1u), P2 = __ldg(g + q + 2u), P3 = __ldg(g + q + 3u);
-      walk_pairs2<T>(lane_base, P0, m1, m0);
-      walk_pairs2<T>(lane_base, P1, m1, m0);
+      walk_pairs2<T, R>(lane_base, band, P0, m1, m0);
+      walk_pairs2<T, R>(lane_base, band, P1, m1, m0);
       if (skip != 0u && !live_lanes<T, false>(m1, m0)) {
         dead = true;
         walked -= n - 4u * (q + 2u);  // pixels not walked (pair groups hold four pixels of the record)
         break;
       }
-      walk_pairs2<T>(lane_base, P2, m1, m0);
-      walk_pairs2<T>(lane_base, P3, m1, m0);
+      walk_pairs2<T, R>(lane_base, band, P2, m1, m0);
+      walk_pairs2<T, R>(lane_base, band, P3, m1, m0);
       if (skip != 0u) {
         const uint32_t lanes = live_lanes<T, kGather>(m1, m0);
         if (!lanes) {
@@ -389,21 +402,21 @@ __device__ __forceinline__ uint32_t walk_unit(const uint4* __restrict__ prog, ui
     }
     for (; !dead && !to && q + 2u <= n_pg; q += 2u) {
       const uint4 P0 = __ldg(g + q), P1 = __ldg(g + q + 1u);
-      walk_pairs2<T>(lane_base, P0, m1, m0);
-      walk_pairs2<T>(lane_base, P1, m1, m0);
+      walk_pairs2<T, R>(lane_base, band, P0, m1, m0);
+      walk_pairs2<T, R>(lane_base, band, P1, m1, m0);
       if (skip != 0u && !live_lanes<T, false>(m1, m0)) {
         dead = true;
         walked -= n - 4u * (q + 2u);
         break;
       }
     }
-    if (!dead && !to && q < n_pg) walk_pairs2<T>(lane_base, __ldg(g + q), m1, m0);
+    if (!dead && !to && q < n_pg) walk_pairs2<T, R>(lane_base, band, __ldg(g + q), m1, m0);
     if (!dead && !to) {
       g += n_pg;
       for (q = 0; q + 2u <= n_sg; q += 2u) {
         const uint4 P0 = __ldg(g + q), P1 = __ldg(g + q + 1u);
-        walk_singles4<T>(lane_base, P0, m1, m0);
-        walk_singles4<T>(lane_base, P1, m1, m0);
+        walk_singles4<T, R>(lane_base, band, P0, m1, m0);
+        walk_singles4<T, R>(lane_base, band, P1, m1, m0);
         if (skip != 0u && !live_lanes<T, false>(m1, m0)) {
           dead = true;
           const uint32_t done = 4u * (n_pg + q + 2u);
@@ -412,10 +425,10 @@ __device__ __forceinline__ uint32_t walk_unit(const uint4* __restrict__ prog, ui
         }
       }
       if (!dead) {
-        if (q < n_sg) walk_singles4<T>(lane_base, __ldg(g + q), m1, m0);
+        if (q < n_sg) walk_singles4<T, R>(lane_base, band, __ldg(g + q), m1, m0);
         if (half) {
           const uint4 P = __ldg(g + n_sg);
-          walk_singles2<T>(lane_base, P.x, P.y, m1, m0);
+          walk_singles2<T, R>(lane_base, band, P.x, P.y, m1, m0);
         }
       }
     }
