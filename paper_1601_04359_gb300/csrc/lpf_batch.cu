@@ -5,7 +5,7 @@
 // Every image brings its own window and program (its own paths handle).  A
 // batch is prepared once (programs uploaded, work area allocated, a device
 // table of per-image descriptors written); a run is then a few launches with
-// no host-device copies -- zero the counts, pack every image into bit rows,
+// no host-device copies -- pack every image into bit rows (zeroing the counts),
 // one persistent walk kernel per words-per-thread choice present, fill the
 // mirrored halves -- and can be replayed as a CUDA graph.  All blocks have 8
 // warps; each image side gets its own words per thread T (chosen by a
@@ -69,21 +69,24 @@ struct BatchSlot {
   int img, bg, g;  // image, its band group, global band-group index (counter)
 };
 
-__global__ void batch_zero_kernel(const BatchDesc* __restrict__ d) {
-  const BatchDesc& b = d[blockIdx.y];
-  if (!b.primary) return;
-  const int64_t n = 2 * b.n_full;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    b.counts[i] = 0ull;
-}
-
 // Packed rows of every side: bit b of word k of row y is the side's pixel at
 // row (y - up) mod H, column (32k + b - r32) mod W.  A transposed side runs over its
-// words column by column, so that a warp reads consecutive image bytes.
-__global__ void batch_pack_kernel(const BatchDesc* __restrict__ d) {
+// words column by column, so that a warp reads consecutive image bytes.  Also
+// zeroes the counts, the control words (the status of this run, the unit and
+// slot counters) and the work tallies: as launches of their own the three
+// took 10 us of a run.
+__global__ void batch_pack_kernel(const BatchDesc* __restrict__ d, int n_desc, int* __restrict__ ctl, int ctl_words,
+                                  unsigned long long* __restrict__ executed) {
   const BatchDesc& b = d[blockIdx.y];
+  const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+  if (blockIdx.y == 0) {
+    for (int64_t i = first; i < ctl_words; i += stride) ctl[i] = 0;
+    for (int64_t i = first; i < n_desc; i += stride) executed[i] = 0ull;
+  }
+  if (b.primary)
+    for (int64_t i = first; i < 2 * b.n_full; i += stride) b.counts[i] = 0ull;
   const int64_t total = (int64_t)b.rows * b.S;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+  for (int64_t i = first; i < total; i += stride) {
     int y, k;
     if (b.primary) { y = (int)(i / b.S); k = (int)(i % b.S); }
     else { k = (int)(i / b.rows); y = (int)(i % b.rows); }
@@ -365,7 +368,7 @@ static int batch_build(lpf_batch* bt, const uint8_t* const* imgs, const int32_t*
       d.rs = side ? 1 : W[i];
       d.cs = side ? W[i] : 1;
       d.primary = side == 0;
-      d.gather = std::max(p->host.rx, p->host.ry) >= kGatherWindow;
+      d.gather = std::max(p->host.rx, p->host.ry) >= kGatherWindowBatch;
       bt->desc.push_back(d);
       total_bg += g.nbg;
       bg_work.push_back((double)prog.n_pixel_words * g.G * g.BB * (g.T + 1));
@@ -414,10 +417,18 @@ static int batch_build(lpf_batch* bt, const uint8_t* const* imgs, const int32_t*
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   // each T's walk kernel: its shared-memory limit and resident blocks
+  // a kernel re-deals masks when most of its work is in images that want it
   bool gather = false;
-  for (bool& w : bt->gather_T) w = false;
-  for (const BatchDesc& d : bt->desc)
-    if (d.gather && d.T > 1) bt->gather_T[t_index(d.T)] = gather = true;
+  for (int k = 0; k < kBatchTs; ++k) {
+    double all = 0, wide = 0;
+    for (int i = 0; i < n_desc; ++i) {
+      if (t_index(bt->desc[i].T) != k) continue;
+      all += bg_work[i] * bt->desc[i].nbg;
+      if (bt->desc[i].gather) wide += bg_work[i] * bt->desc[i].nbg;
+    }
+    bt->gather_T[k] = k >= 2 && wide > 0.5 * all;
+    gather |= bt->gather_T[k];
+  }
   bt->smem = bt->max_band + (gather ? 8u * kBatchThreads : 0u);
   for (int k = 0; k < kBatchTs && gather; ++k) {
     cudaFuncAttributes fa;
@@ -496,11 +507,9 @@ static int batch_build(lpf_batch* bt, const uint8_t* const* imgs, const int32_t*
 }
 
 static void batch_enqueue(lpf_batch* bt, cudaStream_t s) {
-  cudaMemsetAsync(bt->d_ctl, 0, bt->ctl_words * sizeof(int), s);  // status of this run, unit counters
   const int n_desc = (int)bt->desc.size();
-  cudaMemsetAsync(bt->d_exec, 0, sizeof(unsigned long long) * n_desc, s);
-  batch_zero_kernel<<<dim3(bt->max_full, n_desc), 256, 0, s>>>(bt->d_desc);
-  batch_pack_kernel<<<dim3(bt->max_pack, n_desc), 256, 0, s>>>(bt->d_desc);
+  batch_pack_kernel<<<dim3(std::max(bt->max_pack, bt->max_full), n_desc), 256, 0, s>>>(
+      bt->d_desc, n_desc, bt->d_ctl, bt->ctl_words, bt->d_exec);
   // one walk kernel per T present, the one with the most work on the
   // caller's stream, the others on the batch's streams (their blocks take
   // the SMs the first one's blocks leave at its end); joined before the mirror

@@ -99,6 +99,9 @@ int make_geometry(int H, int W, int rx, int ry, int T, int BB, Geometry& g) {
   return layout_side(H, W, rx, ry, T, BB, g);
 }
 
+// Two units per warp slot of the GPU (152 SMs of 32): see kGatherWindow.
+constexpr int64_t kGatherUnits = 2 * 32 * 152;
+
 int make_sides(const Paths& paths, int H, int W, int T, int BB, Sides& s) {
   const int rx = paths.rx, ry = paths.ry;
   int rc = make_geometry(H, W, rx, std::min(rx, ry), T, BB, s.g[0]);
@@ -127,7 +130,11 @@ int make_sides(const Paths& paths, int H, int W, int T, int BB, Sides& s) {
   // 32 warps that the registers allow.
   const int fit = std::max(1, (228 * 1024) / (int)(s.band_bytes + 16 * 256 + 1024));
   s.threads = 32 * std::min(16, std::max(tiles, 32 / fit));
-  s.gather = std::max(rx, ry) >= kGatherWindow;
+  int64_t units = 0;
+  for (int q = 0; q < s.n; ++q)
+    units += (int64_t)s.g[q].nbg * tiles_of(s.g[q]) *
+             (int64_t)((q ? paths.tree_t : paths.tree).piece_begin.size() - 1);
+  s.gather = std::max(rx, ry) >= kGatherWindow && s.g[0].T >= 4 && units >= kGatherUnits;
   if (s.nbg > kMaxBandGroups) return LPF_EUNSUPPORTED;
   return LPF_OK;
 }

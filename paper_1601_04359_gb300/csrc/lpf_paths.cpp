@@ -438,7 +438,7 @@ int build_paths_nd(int32_t rx, int32_t ry, int32_t rz, int dims, int n_pieces, P
     Records rec;
     emit_records(wk.ev, rec.full, rec.word, rec.pix, rec.cur, rec.stack, rec.restores);
     make_tree_program(t, rec, wk.max_level, pieces_for(sub[root]), o ? p.tree_t : p.tree);
-    if (dims == 2 && nn <= kFineNodes) {
+    if (dims == 2 && nn <= kFineNodes && std::max(rx, ry) <= kFineWindow) {
       const int64_t piece_nodes = std::max<int64_t>(32, (int64_t)std::max(rx, ry) + 1);
       make_tree_program(t, rec, wk.max_level, (int)std::max<int64_t>(1, sub[root] / piece_nodes),
                         o ? p.fine_t : p.fine);

@@ -134,6 +134,7 @@ void segment_canonical3(int dx, int dy, int dz, std::vector<int16_t>& out_xyz);
 // Returns 0 or a negative status.
 constexpr int64_t kMaxPieces = 1024;
 constexpr int64_t kFineNodes = int64_t(1) << 17;  // (wider windows: even the smallest image has a unit per warp)
+constexpr int kFineWindow = 128;  // (a piece's prologue walks up to one segment: 31x215, whole domain, 76 -> 84 us)
 int build_paths(int32_t rx, int32_t ry, int n_pieces, Paths& p, std::string& err);
 // The same for dims = 2 (rz ignored) or dims = 3 (vectors |dz| <= rz too).
 int build_paths_nd(int32_t rx, int32_t ry, int32_t rz, int dims, int n_pieces, Paths& p, std::string& err);

@@ -154,6 +154,7 @@ inline size_t persistent_smem_bytes(size_t ext_bytes, int mv, int me) {
          (size_t)me * (4 + 2) + 16;
 }
 int delta_max_smem();
+int delta_num_sms();
 // The annealer's phase-0 counts per translation: bytes for an H x W cell (0:
 // not used -- too long segments or too much memory), and the kernel that
 // fills them from an extended cell.

@@ -82,7 +82,7 @@ static int swap_img_words(int H, int ry, int S) { return ((H + ry) * S + 3) & ~3
 static size_t swap_smem(const SwapArgs& g, bool many) {
   const size_t img = (size_t)swap_img_words(g.H, g.ry, g.S) * 4;
   const size_t group = many ? (size_t)g.words * 64 + 4 * img : (size_t)((g.words * 3 + 3) & ~3) * 4;
-  return img + (size_t)((g.S + 3) & ~3) * 4 + (size_t)g.G * (group + (size_t)2 * g.nmax * 4) + 64;
+  return img + (size_t)((g.S + 3) & ~3) * 4 + (size_t)g.G * (group + (size_t)3 * g.nmax * 4) + 64;
 }
 
 // Packed rows of the cell (img), selection words and candidates; flags as
@@ -251,7 +251,7 @@ __device__ __forceinline__ bool swap_maybe_both(int dx, int dy, int ddx, int ddy
 }
 
 // True when pixel (qx, qy) lies on S(v) placed at translation (x, y) (torus;
-// the segment spans fewer than W columns and H rows).
+// the segment spans fewer than W columns and H rows); seg in shared memory.
 __device__ __forceinline__ bool swap_on_segment(const short2* seg, int dx, int dy, int x, int y, int qx, int qy,
                                                 int H, int W) {
   int uy = qy - y;
@@ -264,8 +264,8 @@ __device__ __forceinline__ bool swap_on_segment(const short2* seg, int dx, int d
   ux += xlo;
   if (ux > xhi) return false;
   const int adx = dx < 0 ? -dx : dx;
-  if (adx >= dy) return __ldg(seg + (dx < 0 ? -ux : ux)).y == uy;  // x-major: pixel k at sx = sign(dx) k
-  return __ldg(seg + uy).x == ux;                                  // y-major: pixel k at sy = k
+  if (adx >= dy) return seg[dx < 0 ? -ux : ux].y == uy;  // x-major: pixel k at sx = sign(dx) k
+  return seg[uy].x == ux;                                  // y-major: pixel k at sy = k
 }
 
 // Translation of the segment whose pixel (sx, sy) is (qx, qy).
@@ -290,15 +290,20 @@ __device__ __forceinline__ float swap_add_error(float acc, int d0, int d1, float
   return acc;
 }
 
-// Block = one vector chunk; its threads form G groups of tg, which take the
-// chunk's vectors G at a time.  partial[chunk][K] (or null), dcounts
-// [K][2][n_canon] (or null).
+// Block = one vector chunk (x) and one share of the candidates (y); its threads
+// form G groups of tg, which take the chunk's vectors G at a time.
+// partial[chunk][K] (or null), dcounts [K][2][n_canon] (or null).
 template <bool MANY>
 __global__ void __launch_bounds__(kSwapThreads, 3) swap_kernel(SwapArgs g, const SwapCand* __restrict__ cand, int K,
                                                                int32_t* __restrict__ dcounts,
                                                                float* __restrict__ partial) {
   extern __shared__ __align__(16) uint32_t smw[];
-  __shared__ int s_any[kSwapWarps];  // per group: some translation is in one of the planes
+  // per group (at most one per warp): whether some translation is in one of
+  // the planes, and its vector (the candidates' loop reads no global memory
+  // but the candidates: its loads used to set the pace of small cells)
+  __shared__ int s_any[kSwapWarps], s_n[kSwapWarps];
+  __shared__ short2 s_vec[kSwapWarps];
+  __shared__ float s_dd[kSwapWarps][2];
   const int H = g.H, W = g.W, S = g.S;
   const int img_words = ((H + g.ry) * S + 3) & ~3;
   const int ext_words = img_words;  // words of a plane with halo (padded: groups start on 16 bytes)
@@ -307,12 +312,13 @@ __global__ void __launch_bounds__(kSwapThreads, 3) swap_kernel(SwapArgs g, const
   int* s_col = reinterpret_cast<int*>(s_img + img_words);  // column (32 k - r32) mod W
   uint32_t* s_groups = reinterpret_cast<uint32_t*>(s_col + ((S + 3) & ~3));
   const int plane_words = MANY ? g.words * 16 : (g.words * 3 + 3) & ~3;  // planes; many: then the sum tables
-  const int group_words = plane_words + (MANY ? 4 * ext_words : 0) + 2 * g.nmax;
+  const int group_words = plane_words + (MANY ? 4 * ext_words : 0) + 3 * g.nmax;
   const int gi = tid / g.tg, gt = tid - gi * g.tg;
   uint32_t* base = s_groups + gi * group_words;
   uint4* ext = reinterpret_cast<uint4*>(base + plane_words);  // {U, X1, X0, 0} by word of the packed rows
-  uint32_t* segA = base + group_words - 2 * g.nmax;
+  uint32_t* segA = base + group_words - 3 * g.nmax;
   uint32_t* segB = segA + g.nmax;
+  short2* segP = reinterpret_cast<short2*>(segB + g.nmax);
 
   for (int i = tid; i < (H + g.ry) * S; i += nthr) s_img[i] = __ldg(g.img + i);
   for (int k = tid; k < S; k += nthr) {
@@ -321,12 +327,13 @@ __global__ void __launch_bounds__(kSwapThreads, 3) swap_kernel(SwapArgs g, const
   }
   const int ch = blockIdx.x;
   const int v0 = g.chunk[ch], v1 = g.chunk[ch + 1];
+  const int k_lo = (int)((int64_t)K * blockIdx.y / gridDim.y), k_hi = (int)((int64_t)K * (blockIdx.y + 1) / gridDim.y);
   float* part = partial ? partial + (int64_t)ch * K : nullptr;
   if (part) {
     if (MANY)
-      for (int k = tid; k < K; k += nthr) part[k] = 0.0f;
+      for (int k = k_lo + tid; k < k_hi; k += nthr) part[k] = 0.0f;
     else if (lane == 0)
-      for (int k = warp; k < K; k += nwarps) part[k] = 0.0f;
+      for (int k = k_lo + warp; k < k_hi; k += nwarps) part[k] = 0.0f;
   }
 
   for (int vb = v0; vb < v1; vb += g.G) {
@@ -337,10 +344,21 @@ __global__ void __launch_bounds__(kSwapThreads, 3) swap_kernel(SwapArgs g, const
     const short2* seg = reinterpret_cast<const short2*>(g.off16) + o0;
     for (int i = gt; i < n; i += g.tg) {
       const short2 s = __ldg(seg + i);
+      segP[i] = s;
       segA[i] = (uint32_t)(s.y * S + ((s.x + g.r32) >> 5)) << 5 | (uint32_t)(s.x & 31);
       if (MANY) segB[i] = (uint32_t)((g.ry - s.y) * S + ((g.r32 - s.x) >> 5)) << 5 | (uint32_t)(-s.x & 31);
     }
-    if (gt == 0) s_any[gi] = 0;
+    if (gt == 0) {
+      s_any[gi] = 0;
+      s_n[gi] = n;
+      if (mine) {
+        s_vec[gi] = __ldg(reinterpret_cast<const short2*>(g.vec16) + v);
+        if (part) {
+          s_dd[gi][0] = g.target[v] - (float)g.counts[v] * g.inv_norm;
+          s_dd[gi][1] = g.target[g.n_full + v] - (float)g.counts[g.n_full + v] * g.inv_norm;
+        }
+      }
+    }
     __syncthreads();  // (also: the packed rows, and the last round's reads of the planes)
     if (mine) {
       for (int w0 = gt; w0 - lane < g.words; w0 += 2 * g.tg) {  // two words at a time (whole warps)
@@ -439,26 +457,22 @@ __global__ void __launch_bounds__(kSwapThreads, 3) swap_kernel(SwapArgs g, const
       const bool any = s_any[q] != 0;
       if (!any && !dcounts) continue;
       const uint32_t* pl = s_groups + q * group_words;
-      const int oq = __ldg(g.dptr + vq), nq = __ldg(g.dptr + vq + 1) - oq;
-      const short2* sq = reinterpret_cast<const short2*>(g.off16) + oq;
-      const short2 dv = __ldg(reinterpret_cast<const short2*>(g.vec16) + vq);
-      float dd0 = 0.0f, dd1 = 0.0f;
-      if (part) {
-        dd0 = g.target[vq] - (float)g.counts[vq] * g.inv_norm;
-        dd1 = g.target[g.n_full + vq] - (float)g.counts[g.n_full + vq] * g.inv_norm;
-      }
+      const int nq = s_n[q];
+      const short2* sq = reinterpret_cast<const short2*>(pl + group_words - g.nmax);
+      const short2 dv = s_vec[q];
+      const float dd0 = part ? s_dd[q][0] : 0.0f, dd1 = part ? s_dd[q][1] : 0.0f;
       if (MANY) {
         const uint8_t* tu = reinterpret_cast<const uint8_t*>(pl);
         const uint8_t* tn = tu + 32 * g.words;
         const uint4* pext = reinterpret_cast<const uint4*>(pl + plane_words);
         uint4 next = make_uint4(0u, 0u, 0u, 0u);  // the next round's candidate, loaded a round ahead
-        if (tid < K) next = __ldg(reinterpret_cast<const uint4*>(cand) + tid);
-        for (int k0 = warp * 32; k0 < K; k0 += nthr) {
+        if (k_lo + tid < k_hi) next = __ldg(reinterpret_cast<const uint4*>(cand) + k_lo + tid);
+        for (int k0 = k_lo + warp * 32; k0 < k_hi; k0 += nthr) {
           const int k = k0 + lane;
           int d0 = 0, d1 = 0;
           const uint4 c = next;
           next = make_uint4(0u, 0u, 0u, 0u);
-          if (k + nthr < K) next = __ldg(reinterpret_cast<const uint4*>(cand) + k + nthr);
+          if (k + nthr < k_hi) next = __ldg(reinterpret_cast<const uint4*>(cand) + k + nthr);
           if (any) {
             const bool swap = c.z != c.w;
             bool share = false;
@@ -480,7 +494,7 @@ __global__ void __launch_bounds__(kSwapThreads, 3) swap_kernel(SwapArgs g, const
               const int px = A & 0xffff, py = A >> 16, qx = B & 0xffff, qy = B >> 16;
               int both = 0;  // phase 0 | phase 1 << 16
               for (int i = lane; i < nq; i += 32) {
-                const short2 s = __ldg(sq + i);
+                const short2 s = sq[i];
                 int x, y;
                 swap_start(px, py, s, H, W, x, y);
                 if ((pext[(y + g.ry) * S + ((x + g.r32) >> 5)].y >> (x & 31)) & 1u)
@@ -496,7 +510,7 @@ __global__ void __launch_bounds__(kSwapThreads, 3) swap_kernel(SwapArgs g, const
               }
             }
           }
-          if (k < K) {
+          if (k < k_hi) {
             if (dcounts) {
               int32_t* dk = dcounts + (int64_t)k * 2 * g.n_canon + vq;
               dk[0] = d0;
@@ -506,14 +520,14 @@ __global__ void __launch_bounds__(kSwapThreads, 3) swap_kernel(SwapArgs g, const
           }
         }
       } else {
-        for (int k = warp; k < K; k += nwarps) {
+        for (int k = k_lo + warp; k < k_hi; k += nwarps) {
           int d0 = 0, d1 = 0;
           const uint4 c = __ldg(reinterpret_cast<const uint4*>(cand) + k);
           if (any && c.z != c.w) {
             const int ax = c.z & 0xffff, ay = c.z >> 16, bx = c.w & 0xffff, by = c.w >> 16;
             int e0 = 0, e1 = 0;
             for (int i = lane; i < nq; i += 32) {
-              const short2 s = __ldg(sq + i);
+              const short2 s = sq[i];
               int x, y;
               swap_start(ax, ay, s, H, W, x, y);
               int at = y + H * (x >> 5);
@@ -604,8 +618,13 @@ int swap_planes_run(const uint8_t* img_dev, lpf_paths* paths, const int32_t* pai
                                                                    pairs_dev, K, cand, paths->d_status,
                                                                    paths->checked);
   if (paths->ev_start) cudaEventRecord(paths->ev_start, s);
-  if (many) swap_kernel<true><<<d.n_chunks, g.G * g.tg, smem, s>>>(g, cand, K, dcounts_dev, partial_dev);
-  else swap_kernel<false><<<d.n_chunks, g.G * g.tg, smem, s>>>(g, cand, K, dcounts_dev, partial_dev);
+  // small windows have few chunks: shares of the candidates (at least one per
+  // warp, or a block's threads' worth) fill the SMs' three blocks, each share
+  // with its own walk (79x101, window 25x19, 28 candidates: 162 us without)
+  const int share = many ? kSwapThreads : kSwapWarps;
+  const dim3 grid(d.n_chunks, std::max(1, std::min(3 * delta_num_sms() / d.n_chunks, (K + share - 1) / share)));
+  if (many) swap_kernel<true><<<grid, g.G * g.tg, smem, s>>>(g, cand, K, dcounts_dev, partial_dev);
+  else swap_kernel<false><<<grid, g.G * g.tg, smem, s>>>(g, cand, K, dcounts_dev, partial_dev);
   if (paths->ev_stop) cudaEventRecord(paths->ev_stop, s);
   return LPF_OK;
 }

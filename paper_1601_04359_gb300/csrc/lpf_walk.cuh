@@ -274,9 +274,15 @@ static __device__ __noinline__ uint2 gathered_walk(const uint4* __restrict__ pro
 constexpr uint32_t kGatherGroups = 12;
 constexpr int kMaxLive = 32;  // one mask per lane (16: 2.18 instead of 1.97 ms at 512x512, window 256)
 // Windows from which tiles empty out enough to re-deal (kernels of their own:
-// at window 32, 64x64, the code alone costs 4 us of 19, at window 40,
-// 100x128, 6 %); at window 128 a third of the walk is gathered.
-constexpr int kGatherWindow = 64;
+// their code costs a launch 4 us and a walk that never re-deals 3 to 6 %); at
+// window 128 a third of the walk is gathered.  Images walked one at a time
+// also need four words per thread or more (with two, 334x50, window 25x167,
+// took 88 instead of 73 us) and two units per warp slot (112x93, whole
+// domain: 93 instead of 87 us); at window 119 (239x230) it is a loss of 2 %,
+// at 143 (210x286) a gain of a third; batches, whose images share a kernel, pay
+// from windows of 120 (96 and less: 3 to 5 % slower).
+constexpr int kGatherWindow = 128;
+constexpr int kGatherWindowBatch = 120;
 
 // Valid translations of a tile: word t of the lane (row y + 32 (t / (T / R)))
 // holds translations x = 32 (j0 + t mod T / R) + bit; those with x < W in a
@@ -432,27 +438,34 @@ __device__ __forceinline__ uint32_t walk_unit(const uint4* __restrict__ prog, ui
         }
       }
     }
-    if (!dead && !to && (hdr & (kEmit | kPush)) && skip != 0u) {
-      // Empty for the whole warp (one vote): so is every count below this node.
-      const uint32_t lanes = live_lanes<T, kGather>(m1, m0);
-      if (!lanes) dead = true;
-      else if (kGather && deal && next + kGatherGroups <= rec + skip && __popc(lanes) <= kMaxLive - 4)
-        to = gather(rec, n_pg + n_sg + 1u);
-    }
     if (dead || to) {
       pc = dead ? rec + skip : to;
       hd = pc < end ? __ldg(prog + pc) : make_uint4(0u, 0u, 0u, 0u);
       continue;
     }
-    if (hdr & kEmit) {
-      uint32_t c = 0;
+    if (hdr & (kEmit | kPush)) {
+      if (skip != 0u) {
+        // Empty for the whole warp (one vote): so is every count below this node.
+        const uint32_t lanes = live_lanes<T, kGather>(m1, m0);
+        if (!lanes) to = rec + skip;
+        else if (kGather && deal && next + kGatherGroups <= rec + skip && __popc(lanes) <= kMaxLive - 4)
+          to = gather(rec, n_pg + n_sg + 1u);
+        if (to) {
+          pc = to;
+          hd = pc < end ? __ldg(prog + pc) : make_uint4(0u, 0u, 0u, 0u);
+          continue;
+        }
+      }
+      if (hdr & kEmit) {
+        uint32_t c = 0;
 #pragma unroll
-      for (int t = 0; t < T; ++t) c += (uint32_t)__popc(m1[t]) + ((uint32_t)__popc(m0[t]) << 16);
-      c = __reduce_add_sync(0xffffffffu, c);  // one warp-reduce instruction
-      if (lane == 0) {
-        const uint32_t c1 = c & 0xffffu, c0 = c >> 16;
-        if (c0) atomicAdd(counts + base + vec, (unsigned long long)c0);
-        if (c1) atomicAdd(counts + n_full + base + vec, (unsigned long long)c1);
+        for (int t = 0; t < T; ++t) c += (uint32_t)__popc(m1[t]) + ((uint32_t)__popc(m0[t]) << 16);
+        c = __reduce_add_sync(0xffffffffu, c);  // one warp-reduce instruction
+        if (lane == 0) {
+          const uint32_t c1 = c & 0xffffu, c0 = c >> 16;
+          if (c0) atomicAdd(counts + base + vec, (unsigned long long)c0);
+          if (c1) atomicAdd(counts + n_full + base + vec, (unsigned long long)c1);
+        }
       }
     }
     if (hdr & kPush) {
