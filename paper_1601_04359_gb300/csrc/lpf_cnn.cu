@@ -123,10 +123,11 @@ __device__ __forceinline__ int wrap(int t, int n) {
 // = bf16(in[(y0+ly-1) % H][(x0+lx-1) % W][k]) for k < C, 0 up to KC.
 // With lo != null (split operand) also lo[...] = bf16(v - hi): the value as
 // two bfloat16 terms, hi + lo, about 16 significant bits.  Four channels per
-// load where there are that many (C is 2 or a multiple of 16).
+// load where there are that many (C is 2 or a multiple of 16).  live: the
+// channels there are from in on (C, or fewer for a share of them).
 template <int KC>
 __device__ __forceinline__ void stage_halo(const float* __restrict__ in, int H, int W, int C, int x0, int y0,
-                                           __nv_bfloat16* s, __nv_bfloat16* lo = nullptr) {
+                                           __nv_bfloat16* s, __nv_bfloat16* lo, int live) {
   constexpr int KS = KC + 8;
   constexpr int KQ = KC / 4;  // channel quads
   for (int i = threadIdx.x; i < kHalo * KQ; i += blockDim.x) {
@@ -135,8 +136,8 @@ __device__ __forceinline__ void stage_halo(const float* __restrict__ in, int H, 
     const int gy = wrap(y0 + ly - 1, H), gx = wrap(x0 + lx - 1, W);
     const float* src = in + ((int64_t)gy * W + gx) * C;
     float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    if (k + 3 < C) v = *reinterpret_cast<const float4*>(src + k);
-    else if (k < C) { v.x = src[0]; v.y = src[1]; }  // C = 2
+    if (k + 3 < live) v = *reinterpret_cast<const float4*>(src + k);
+    else if (k < live) { v.x = src[0]; v.y = src[1]; }  // C = 2
     const __nv_bfloat162 h0 = __floats2bfloat162_rn(v.x, v.y), h1 = __floats2bfloat162_rn(v.z, v.w);
     uint2 w;
     w.x = *reinterpret_cast<const uint32_t*>(&h0);
@@ -159,7 +160,8 @@ __device__ __forceinline__ void stage_halo(const float* __restrict__ in, int H, 
 // are).  So both stage whole rows in 16-byte asynchronous copies: gathered
 // one by one out of [9][K][N] they took most of a forward layer's time
 // (64 -> 48 channels at 128x128: 23.4 -> 10.2 us; all five layers and the
-// features 88 -> 55 us; a training step on 8 snapshots 1.11 -> 0.83 ms).  Optional ReLU; optional mask: out = 0 where
+// features 88 -> 55 us).  Starting a layer early to stage its weights behind
+// the one before gained nothing.  Optional ReLU; optional mask: out = 0 where
 // mask[p][n] <= 0 (the ReLU derivative of the layer input).  K <= KC, N <= NC.
 // A block stages the weights once and then takes output tiles t =
 // blockIdx.x, blockIdx.x + gridDim.x, ... of n_snap snapshots (tile t is
@@ -198,7 +200,7 @@ __global__ void __launch_bounds__(kConvThreads) cnn_conv_mma_kernel(const float*
     const int z = t / per_snap, tr = t - z * per_snap;
     const int x0 = (tr % tiles_x) * kTW, y0 = (tr / tiles_x) * kTH;
     __syncthreads();  // the previous tile's reads of s_in are done
-    stage_halo<KC>(in + z * in_stride, H, W, K, x0, y0, s_in, SPLIT ? s_lo : nullptr);
+    stage_halo<KC>(in + z * in_stride, H, W, K, x0, y0, s_in, SPLIT ? s_lo : nullptr, K);
     copies_wait();  // (the weights, first tile)
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -272,7 +274,11 @@ __global__ void __launch_bounds__(kConvThreads) cnn_conv_mma_kernel(const float*
 // N = co, K = the tile's pixels; warp t computes tap t.  Pixels outside the
 // image contribute nothing (their gradient rows are staged as zeros).
 // blockIdx.z selects a snapshot (in and g advance by in_stride, g_stride
-// floats); its tiles' partials follow those of the snapshots before it.
+// floats); its tiles' partials follow those of the snapshots before it.  A
+// block takes KC of the input channels, from KC times its share of blockIdx.x
+// on (the 64 of one layer in two shares: with all of them a thread holds 96
+// sums, one block of 9 warps fits on an SM, 124 us at 8 x 128x128; in two
+// shares 98 us).
 template <int KC, int NC>
 __global__ void __launch_bounds__(kDwThreads) cnn_dw_mma_kernel(const float* __restrict__ in,
                                                                 const float* __restrict__ g, int H, int W, int CIN,
@@ -286,9 +292,11 @@ __global__ void __launch_bounds__(kDwThreads) cnn_dw_mma_kernel(const float* __r
   __nv_bfloat16* s_in = csm;                          // [kHalo][KS]
   __nv_bfloat16* s_g = csm + kHalo * KS;              // [kTH * kTW][NS], gradient high terms
   __nv_bfloat16* s_gl = s_g + kTH * kTW * NS;         // and low terms (the gradient as hi + lo)
-  const int x0 = blockIdx.x * kTW, y0 = blockIdx.y * kTH;
-  const int blk = ((int)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-  stage_halo<KC>(in, H, W, CIN, x0, y0, s_in);
+  const int tiles_x = (W + kTW - 1) / kTW, share = blockIdx.x / tiles_x, tx = blockIdx.x - share * tiles_x;
+  const int c0 = share * KC;  // first input channel
+  const int x0 = tx * kTW, y0 = blockIdx.y * kTH;
+  const int blk = ((int)blockIdx.z * gridDim.y + blockIdx.y) * tiles_x + tx;
+  stage_halo<KC>(in + c0, H, W, CIN, x0, y0, s_in, nullptr, CIN - c0);
   for (int i = threadIdx.x; i < kTH * kTW * (NC / 4); i += blockDim.x) {
     const int q = i / (NC / 4), n = 4 * (i - q * (NC / 4));
     const int py = y0 + q / kTW, px = x0 + q % kTW;
@@ -310,7 +318,7 @@ __global__ void __launch_bounds__(kDwThreads) cnn_dw_mma_kernel(const float* __r
   }
   // bias partial: fixed order over the tile's pixels (float32, no rounding), a
   // row of loads in flight
-  if ((int)threadIdx.x < COUT) {
+  if (share == 0 && (int)threadIdx.x < COUT) {
     float sb = 0.0f;
     for (int r = 0; r < kTH && y0 + r < H; ++r) {
       float v[kTW];
@@ -376,31 +384,35 @@ __global__ void __launch_bounds__(kDwThreads) cnn_dw_mma_kernel(const float* __r
     for (int f = 0; f < NC / 8; ++f)
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const int ci = m * 16 + gid + (e >= 2 ? 8 : 0), co = f * 8 + tig * 2 + (e & 1);
+        const int ci = c0 + m * 16 + gid + (e >= 2 ? 8 : 0), co = f * 8 + tig * 2 + (e & 1);
         if (ci < CIN && co < COUT) dst[ci * COUT + co] = acc[m][f][e];
       }
 }
 
-// Reduction of the per-tile gradient partials, deterministic and with the
-// same additions as reducing the snapshots one by one:
+// Reduction of a layer's per-tile gradient partials, deterministic and with
+// the same additions as reducing the snapshots one by one; weights (n_w
+// values per tile, part) and biases (n_b, part_b) in one launch, a layer's
+// parameters being n_w + n_b values in a row:
 // s[z][i] = sum over the tiles b of snapshot z of part[z][b][i], tiles in
 // order (snapshot blockIdx.y; sixteen loads in flight, added in order) ...
-__global__ void cnn_reduce_tiles_kernel(const float* __restrict__ part, int n_blk, int n, float* __restrict__ s) {
+__global__ void cnn_reduce_tiles_kernel(const float* __restrict__ part, const float* __restrict__ part_b, int n_blk,
+                                        int n_w, int n_b, float* __restrict__ s) {
   const int z = blockIdx.y;
-  const float* pz = part + (int64_t)z * n_blk * n;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    float acc = 0.0f;
-    int b = 0;
-    for (; b + 16 <= n_blk; b += 16) {
-      float v[16];
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n_w + n_b) return;
+  const int n = i < n_w ? n_w : n_b;
+  const float* pz = i < n_w ? part + (int64_t)z * n_blk * n_w + i : part_b + (int64_t)z * n_blk * n_b + (i - n_w);
+  float acc = 0.0f;
+  int b = 0;
+  for (; b + 16 <= n_blk; b += 16) {
+    float v[16];
 #pragma unroll
-      for (int u = 0; u < 16; ++u) v[u] = pz[(int64_t)(b + u) * n + i];
+    for (int u = 0; u < 16; ++u) v[u] = pz[(int64_t)(b + u) * n];
 #pragma unroll
-      for (int u = 0; u < 16; ++u) acc += v[u];
-    }
-    for (; b < n_blk; ++b) acc += pz[(int64_t)b * n + i];
-    s[(int64_t)z * n + i] = acc;
+    for (int u = 0; u < 16; ++u) acc += v[u];
   }
+  for (; b < n_blk; ++b) acc += pz[(int64_t)b * n];
+  s[(int64_t)z * (n_w + n_b) + i] = acc;
 }
 
 // ... then dst[i] = s[0][i] (or dst[i] + s[0][i] when accumulating), then
@@ -609,7 +621,7 @@ static int cnn_reserve(lpf_cnn* c, int nb) {
   if (e == cudaSuccess) e = cudaMalloc(&c->d_part, b * c->n_blk * 9 * 64 * 64 * 4);
   if (e == cudaSuccess) e = cudaMalloc(&c->d_part_b, b * c->n_blk * 64 * 4);
   if (e == cudaSuccess) e = cudaMalloc(&c->d_loss, b * 4);
-  if (e == cudaSuccess) e = cudaMalloc(&c->d_snap, b * 9 * 64 * 64 * 4);
+  if (e == cudaSuccess) e = cudaMalloc(&c->d_snap, b * (9 * 64 * 64 + 64) * 4);
   if (e != cudaSuccess) return set_cuda_error(e);
   c->cap = nb;
   return LPF_OK;
@@ -643,11 +655,11 @@ static int cnn_alloc(lpf_cnn* c) {
   if (e != cudaSuccess) return set_cuda_error(e);
   std::vector<int2> isw(np, make_int2(-1, -1));
   for (int l = 0; l < kLayers; ++l) {
-    const int ci = kCh[l], co = kCh[l + 1];
-    for (int i = 0; i < layer_w_size(l); ++i) {
-      const int tap = i / (ci * co), r = i % (ci * co);
-      isw[c->w_off[l] + i] = make_int2((int)(c->wb_off[l] + i), (int)(c->wb_off[l] + (tap * co + r % co) * ci + r / co));
-    }
+    int2* to = isw.data() + c->w_off[l];
+    const int at = (int)c->wb_off[l], n_ci = kCh[l], n_co = kCh[l + 1];
+    for (int tap = 0, i = 0; tap < 9; ++tap)
+      for (int ci = 0; ci < n_ci; ++ci)
+        for (int co = 0; co < n_co; ++co, ++i) to[i] = make_int2(at + i, at + (tap * n_co + co) * n_ci + ci);
   }
   e = cudaMemcpy(c->d_isw, isw.data(), np * sizeof(int2), cudaMemcpyHostToDevice);
   return set_cuda_error(e);
@@ -735,7 +747,7 @@ static void dw_mma(const float* in, const float* g, int H, int W, int CIN, int C
     cudaFuncSetAttribute(cnn_dw_mma_kernel<KC, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     attr = true;
   }
-  const dim3 grid((W + kTW - 1) / kTW, (H + kTH - 1) / kTH, nb);
+  const dim3 grid((W + kTW - 1) / kTW * ((CIN + KC - 1) / KC), (H + kTH - 1) / kTH, nb);
   cnn_dw_mma_kernel<KC, NC><<<grid, kDwThreads, smem, s>>>(in, g, H, W, CIN, COUT, part, part_b,
                                                             (int64_t)H * W * CIN, (int64_t)H * W * COUT);
 }
@@ -745,7 +757,7 @@ static void dw_any(int CIN, int COUT, const float* in, const float* g, int H, in
   switch (CIN * 1000 + COUT) {
     case 2 * 1000 + 32: dw_mma<16, 32>(in, g, H, W, CIN, COUT, part, part_b, nb, s); break;
     case 32 * 1000 + 64: dw_mma<32, 64>(in, g, H, W, CIN, COUT, part, part_b, nb, s); break;
-    case 64 * 1000 + 48: dw_mma<64, 48>(in, g, H, W, CIN, COUT, part, part_b, nb, s); break;
+    case 64 * 1000 + 48: dw_mma<32, 48>(in, g, H, W, CIN, COUT, part, part_b, nb, s); break;
     case 48 * 1000 + 32: dw_mma<48, 32>(in, g, H, W, CIN, COUT, part, part_b, nb, s); break;
     default: dw_mma<32, 8>(in, g, H, W, CIN, COUT, part, part_b, nb, s); break;  // 32 -> 2
   }
@@ -787,10 +799,10 @@ static int cnn_fwd_bwd(lpf_cnn* c, const uint8_t* cells, int nb, const int32_t* 
     // g = dL/d(pre-activation output of layer l) here (ReLU mask already applied)
     dw_any(cin, cout, c->d_tact[l], g, H, W, c->d_part, c->d_part_b, nb, s);
     const int nw_l = 9 * cin * cout;
-    cnn_reduce_tiles_kernel<<<dim3((nw_l + 255) / 256, nb), 256, 0, s>>>(c->d_part, c->n_blk, nw_l, c->d_snap);
-    cnn_reduce_snaps_kernel<<<(nw_l + 255) / 256, 256, 0, s>>>(c->d_snap, nb, nw_l, c->d_g + c->w_off[l], accumulate);
-    cnn_reduce_tiles_kernel<<<dim3(1, nb), 64, 0, s>>>(c->d_part_b, c->n_blk, cout, c->d_snap);
-    cnn_reduce_snaps_kernel<<<1, 64, 0, s>>>(c->d_snap, nb, cout, c->d_g + c->b_off[l], accumulate);
+    const int np_l = nw_l + cout;  // (the layer's biases follow its weights in the parameter vector)
+    cnn_reduce_tiles_kernel<<<dim3((np_l + 255) / 256, nb), 256, 0, s>>>(c->d_part, c->d_part_b, c->n_blk, nw_l, cout,
+                                                                         c->d_snap);
+    cnn_reduce_snaps_kernel<<<(np_l + 255) / 256, 256, 0, s>>>(c->d_snap, nb, np_l, c->d_g + c->w_off[l], accumulate);
     if (l > 0) {
       // dL/d act[l] = transposed conv of g, then times the ReLU mask of act[l]
       conv_any(cout, cin, g, H, W, c->d_wbf + c->wb_off[l], 1, nullptr, 0, c->d_tact[l], g2, nb, s);
