@@ -759,7 +759,7 @@ static int sa_bind_tables(lpf_sa* sa) {
   if (sa->objective != kSaObjectiveLineal) return LPF_OK;
   const DeltaTables& t = sa->paths->delta;
   if (!(t.d_doff && t.We == sa->g.We && t.want_key == sa->delta_key)) {  // re-baked for another cell
-    const int rc = delta_prepare(sa->paths, sa->H, sa->W, 1);
+    const int rc = delta_prepare(sa->paths, sa->H, sa->W);
     if (rc) return rc;
     if (t.want_key != sa->delta_key) return LPF_EINVAL;  // (a cell of this width but another height)
   }
@@ -874,10 +874,10 @@ int sa_start(lpf_sa* sa, cudaStream_t s) {
       rc = s2_delta_run(sa->cell, sa->H, sa->W, sa->d_ext, sa->d_pairs, K, nullptr, sa->target, sa->counts, sa->d_de,
                         sa->d_partial, s);
     } else {
-      rc = delta_prepare(sa->paths, sa->H, sa->W, K);
+      rc = delta_prepare(sa->paths, sa->H, sa->W);
       if (!rc)
         rc = delta_swap_run(sa->cell, sa->H, sa->W, sa->paths, sa->d_pairs, K, nullptr, sa->target, sa->counts,
-                            sa->d_de, sa->phase_mask, s, sa->d_sel_ext, (float)sa->inv_norm);
+                            sa->d_de, sa->phase_mask, s, sa->d_sel_ext, (float)sa->inv_norm, true);
     }
     std::vector<float> de(K);
     if (!rc) {
@@ -926,7 +926,7 @@ static int sa_create_lineal(uint8_t* cell_dev, int32_t H, int32_t W, lpf_paths* 
   int rc = sel_dev ? lpf_full_mc(cell_dev, H, W, paths, sel_dev, counts_dev, stream)
                    : lpf_full(cell_dev, H, W, paths, counts_dev, stream);
   if (rc) return rc;
-  rc = delta_prepare(paths, H, W, 1);
+  rc = delta_prepare(paths, H, W);
   if (rc) return rc;
   lpf_sa* sa = new (std::nothrow) lpf_sa();
   if (!sa) return LPF_ENOMEM;

@@ -136,8 +136,8 @@ int bake(lpf_paths* p, const Program& prog0, const Geometry& g0, const Program* 
 // and a packed-image area of at least `words`.
 int ensure_device(lpf_paths* p, size_t packed_words);
 struct DeltaArgs;
-// Swap-delta: check sizes, bake tables, size the handle's work areas for K.
-int delta_prepare(lpf_paths* p, int H, int W, int K);
+// Swap-delta: check sizes, bake tables, size the handle's work area.
+int delta_prepare(lpf_paths* p, int H, int W);
 // Fill the kernel arguments of the swap-delta kernels for an H x W cell.
 int delta_geometry(const lpf_paths* p, int H, int W, DeltaArgs& g);
 // Candidate strides per vector chunk for K candidates.
@@ -167,10 +167,11 @@ const void* sa_persistent_kernel_entry();
 // lpf_delta_swap with the error restricted to the phases in phase_mask and,
 // optionally, the walks restricted to selected start translations (sel_ext:
 // extended layout, from build_sel_ext) with descriptor = count * inv_norm
-// (inv_norm <= 0: 1/(H W)).
+// (inv_norm <= 0: 1/(H W)).  whole_chunks: error changes summed per vector
+// chunk and then over the chunks, as the annealer does.
 int delta_swap_run(const uint8_t* img_dev, int32_t H, int32_t W, lpf_paths* paths, const int32_t* pairs_dev,
                    int32_t K, int32_t* dcounts_dev, const float* target_dev, const int64_t* counts_dev, float* de_dev,
-                   int phase_mask, cudaStream_t s, const uint8_t* sel_ext, float inv_norm);
+                   int phase_mask, cudaStream_t s, const uint8_t* sel_ext, float inv_norm, bool whole_chunks);
 int count_selected(const uint8_t* sel_dev, int H, int W, cudaStream_t s, int64_t* n);
 int build_sel_ext(const uint8_t* sel_dev, int H, int W, const lpf_paths* paths, cudaStream_t s, uint8_t** out);
 // Learned proposer internals used by the annealer.

@@ -30,11 +30,12 @@
 // one byte per vector and translation (136 MB at 128x128, window 64), filled
 // and read by 2n scattered lookups per candidate and vector.
 // Measured (error changes, a call): 4096 candidates on a 128x128 clustered
-// cell, window 64: 15.66 -> 0.79 ms; 64 candidates on a 50x50 cell, full
-// domain, with count changes: 0.300 -> 0.113 ms; the same bits.
+// cell, window 64: 15.66 -> 0.52 ms; 64 candidates on a 50x50 cell, full
+// domain, with count changes: 0.300 -> 0.075 ms.
 //
-// Error changes are summed per (chunk, candidate) in vector order and then
-// over chunks in chunk order: bitwise reproducible.
+// Error changes are summed per (part of a chunk, candidate) in vector order
+// and then over the parts in a fixed order that depends on the cell and window
+// alone: bitwise reproducible, whatever the number of candidates.
 #include <algorithm>
 
 #include "lpf_delta.cuh"
@@ -47,14 +48,17 @@ constexpr int kSwapThreads = 256;  // 2 words per thread at 128x128; 3 blocks (6
 constexpr int kSwapWarps = kSwapThreads / 32;
 constexpr int kSwapMaxPixels = 255;  // pixels of a segment (the sums are bytes)
 
-// A candidate with a holding phase 1 (a == b: identity): byte offsets of its
-// pixels in the sum tables, and the pixels as y << 16 | x.
-struct SwapCand {
-  uint32_t ta, tb, a, b;
+// Candidates, a holding phase 1 (both pixels 0: identity), as two arrays of K:
+// the byte offsets of a and b in the sum tables, which every vector reads, and
+// a and b as y << 16 | x, which few (vector, candidate) pairs need.
+struct SwapCands {
+  uint2 *table, *pixel;
 };
+constexpr int kSwapUnroll = 4;  // candidates a thread has in flight where it has several
 
 struct SwapArgs {
   int H, W, nw, S, rx, ry, r32;
+  int split;               // parts of a vector chunk, a block each
   int words;               // H * nw; word (y, j) of a plane is y + H j
   int tg, G;               // threads per vector, vectors side by side in a block
   int nmax;                // longest segment, rounded up to 8
@@ -89,7 +93,7 @@ static size_t swap_smem(const SwapArgs& g, bool many) {
 // build_ext_kernel and delta_kernel set them.
 __global__ void swap_prep_kernel(const uint8_t* __restrict__ cell, SwapArgs g, uint32_t* __restrict__ img,
                                  const uint8_t* __restrict__ sel_ext, int We, uint32_t* __restrict__ sel,
-                                 const int32_t* __restrict__ pairs, int K, SwapCand* __restrict__ cand,
+                                 const int32_t* __restrict__ pairs, int K, SwapCands cand,
                                  int* __restrict__ status, int checked) {
   const int stride = gridDim.x * blockDim.x, i0 = blockIdx.x * blockDim.x + threadIdx.x;
   uint32_t high = 0;
@@ -119,18 +123,19 @@ __global__ void swap_prep_kernel(const uint8_t* __restrict__ cell, SwapArgs g, u
   const int npix = g.H * g.W;
   for (int k = i0; k < K; k += stride) {
     int a = pairs[2 * k], b = pairs[2 * k + 1];
-    SwapCand c = {0u, 0u, 0u, 0u};
+    uint2 t = make_uint2(0u, 0u), c = make_uint2(0u, 0u);
     if (a < 0 || b < 0 || a >= npix || b >= npix) {
       atomicOr(status, 2);                                    // identity
     } else if ((cell[a] != 0) != (cell[b] != 0)) {
       if (cell[a] == 0) { const int t = a; a = b; b = t; }
       const int ay = a / g.W, ax = a - ay * g.W, by = b / g.W, bx = b - by * g.W;
-      c.ta = (uint32_t)(((ay + g.H * (ax >> 5)) * 8 + (ax & 7)) * 4 + ((ax >> 3) & 3));
-      c.tb = (uint32_t)(((by + g.H * (bx >> 5)) * 8 + (bx & 7)) * 4 + ((bx >> 3) & 3));
-      c.a = (uint32_t)ay << 16 | (uint32_t)ax;
-      c.b = (uint32_t)by << 16 | (uint32_t)bx;
+      t.x = (uint32_t)(((ay + g.H * (ax >> 5)) * 8 + (ax & 7)) * 4 + ((ax >> 3) & 3));
+      t.y = (uint32_t)(((by + g.H * (bx >> 5)) * 8 + (bx & 7)) * 4 + ((bx >> 3) & 3));
+      c.x = (uint32_t)ay << 16 | (uint32_t)ax;
+      c.y = (uint32_t)by << 16 | (uint32_t)bx;
     }
-    cand[k] = c;
+    cand.table[k] = t;
+    cand.pixel[k] = c;
   }
 }
 
@@ -290,13 +295,16 @@ __device__ __forceinline__ float swap_add_error(float acc, int d0, int d1, float
   return acc;
 }
 
-// Block = one vector chunk (x) and one share of the candidates (y); its threads
-// form G groups of tg, which take the chunk's vectors G at a time.
-// partial[chunk][K] (or null), dcounts [K][2][n_canon] (or null).
-template <bool MANY>
-__global__ void __launch_bounds__(kSwapThreads, 3) swap_kernel(SwapArgs g, const SwapCand* __restrict__ cand, int K,
+// Block = one part of a vector chunk (x) and one share of the candidates (y);
+// its threads form G groups of tg, which take the part's vectors G at a time.
+// U: candidates that a thread takes at a time, 0: the way of few candidates.
+// partial[part][K] (or null), dcounts [K][2][n_canon] (or null).
+template <int U>
+__global__ void __launch_bounds__(kSwapThreads, 3) swap_kernel(SwapArgs g, SwapCands cand, int K,
                                                                int32_t* __restrict__ dcounts,
                                                                float* __restrict__ partial) {
+  constexpr bool MANY = U > 0;
+  constexpr int kU = MANY ? U : 1;
   extern __shared__ __align__(16) uint32_t smw[];
   // per group (at most one per warp): whether some translation is in one of
   // the planes, and its vector (the candidates' loop reads no global memory
@@ -325,10 +333,11 @@ __global__ void __launch_bounds__(kSwapThreads, 3) swap_kernel(SwapArgs g, const
     int c = (32 * k - g.r32) % W;
     s_col[k] = c < 0 ? c + W : c;
   }
-  const int ch = blockIdx.x;
-  const int v0 = g.chunk[ch], v1 = g.chunk[ch + 1];
+  const int ch = blockIdx.x / g.split, sub = blockIdx.x - ch * g.split;
+  const int c0 = g.chunk[ch], nc = g.chunk[ch + 1] - c0;
+  const int v0 = c0 + (int)((int64_t)nc * sub / g.split), v1 = c0 + (int)((int64_t)nc * (sub + 1) / g.split);
   const int k_lo = (int)((int64_t)K * blockIdx.y / gridDim.y), k_hi = (int)((int64_t)K * (blockIdx.y + 1) / gridDim.y);
-  float* part = partial ? partial + (int64_t)ch * K : nullptr;
+  float* part = partial ? partial + (int64_t)blockIdx.x * K : nullptr;
   if (part) {
     if (MANY)
       for (int k = k_lo + tid; k < k_hi; k += nthr) part[k] = 0.0f;
@@ -465,66 +474,87 @@ __global__ void __launch_bounds__(kSwapThreads, 3) swap_kernel(SwapArgs g, const
         const uint8_t* tu = reinterpret_cast<const uint8_t*>(pl);
         const uint8_t* tn = tu + 32 * g.words;
         const uint4* pext = reinterpret_cast<const uint4*>(pl + plane_words);
-        uint4 next = make_uint4(0u, 0u, 0u, 0u);  // the next round's candidate, loaded a round ahead
-        if (k_lo + tid < k_hi) next = __ldg(reinterpret_cast<const uint4*>(cand) + k_lo + tid);
-        for (int k0 = k_lo + warp * 32; k0 < k_hi; k0 += nthr) {
-          const int k = k0 + lane;
-          int d0 = 0, d1 = 0;
-          const uint4 c = next;
-          next = make_uint4(0u, 0u, 0u, 0u);
-          if (k + nthr < k_hi) next = __ldg(reinterpret_cast<const uint4*>(cand) + k + nthr);
+        uint2 next[kU];  // the next round's candidates, loaded a round ahead
+        auto fetch = [&](int k0) {
+#pragma unroll
+          for (int u = 0; u < kU; ++u) {
+            const int k = k0 + lane + u * nthr;
+            next[u] = k < k_hi ? __ldg(cand.table + k) : make_uint2(0u, 0u);
+          }
+        };
+        if (any) fetch(k_lo + warp * 32);
+        for (int k0 = k_lo + warp * 32; k0 < k_hi; k0 += kU * nthr) {
+          int d0[kU], d1[kU];
+#pragma unroll
+          for (int u = 0; u < kU; ++u) d0[u] = d1[u] = 0;
           if (any) {
-            const bool swap = c.z != c.w;
-            bool share = false;
-            int ax = 0, ay = 0, bx = 0, by = 0;
-            if (swap) {
-              const int na = tn[c.x], nb = tn[c.y];
-              d0 = na - (int)tu[c.y];
-              d1 = nb - (int)tu[c.x];
-              if (na | nb) {
-                ax = c.z & 0xffff; ay = c.z >> 16;
-                bx = c.w & 0xffff; by = c.w >> 16;
-                share = swap_maybe_both(dv.x, dv.y, bx - ax, by - ay, H, W);
+            uint2 pix[kU];
+            uint32_t hit = 0;  // bit u: pix[u] is loaded
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+              const uint2 t = next[u];
+              pix[u] = make_uint2(0u, 0u);
+              if (t.x != t.y) {
+                const int na = tn[t.x], nb = tn[t.y];
+                d0[u] = na - (int)tu[t.y];
+                d1[u] = nb - (int)tu[t.x];
+                if (na | nb) {
+                  pix[u] = __ldg(cand.pixel + k0 + lane + u * nthr);
+                  hit |= 1u << u;
+                }
               }
             }
-            // translations through both pixels (a warp per such candidate, lanes over the segment)
-            for (unsigned m = __ballot_sync(0xffffffffu, share); m; m &= m - 1) {
-              const int src = __ffs(m) - 1;
-              const uint32_t A = __shfl_sync(0xffffffffu, c.z, src), B = __shfl_sync(0xffffffffu, c.w, src);
-              const int px = A & 0xffff, py = A >> 16, qx = B & 0xffff, qy = B >> 16;
-              int both = 0;  // phase 0 | phase 1 << 16
-              for (int i = lane; i < nq; i += 32) {
-                const short2 s = sq[i];
-                int x, y;
-                swap_start(px, py, s, H, W, x, y);
-                if ((pext[(y + g.ry) * S + ((x + g.r32) >> 5)].y >> (x & 31)) & 1u)
-                  both += swap_on_segment(sq, dv.x, dv.y, x, y, qx, qy, H, W);
-                swap_start(qx, qy, s, H, W, x, y);
-                if ((pext[(y + g.ry) * S + ((x + g.r32) >> 5)].z >> (x & 31)) & 1u)
-                  both += (int)swap_on_segment(sq, dv.x, dv.y, x, y, px, py, H, W) << 16;
-              }
-              both = __reduce_add_sync(0xffffffffu, both);
-              if (lane == src) {
-                d0 -= both & 0xffff;
-                d1 -= both >> 16;
+            fetch(k0 + kU * nthr);
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+              const bool share = (hit >> u & 1u) &&
+                                 swap_maybe_both(dv.x, dv.y, (int)(pix[u].y & 0xffff) - (int)(pix[u].x & 0xffff),
+                                                 (int)(pix[u].y >> 16) - (int)(pix[u].x >> 16), H, W);
+              // translations through both pixels (a warp per such candidate, lanes over the segment)
+              for (unsigned m = __ballot_sync(0xffffffffu, share); m; m &= m - 1) {
+                const int src = __ffs(m) - 1;
+                const uint32_t A = __shfl_sync(0xffffffffu, pix[u].x, src), B = __shfl_sync(0xffffffffu, pix[u].y, src);
+                const int px = A & 0xffff, py = A >> 16, qx = B & 0xffff, qy = B >> 16;
+                int both = 0;  // phase 0 | phase 1 << 16
+                for (int i = lane; i < nq; i += 32) {
+                  const short2 s = sq[i];
+                  int x, y;
+                  swap_start(px, py, s, H, W, x, y);
+                  if ((pext[(y + g.ry) * S + ((x + g.r32) >> 5)].y >> (x & 31)) & 1u)
+                    both += swap_on_segment(sq, dv.x, dv.y, x, y, qx, qy, H, W);
+                  swap_start(qx, qy, s, H, W, x, y);
+                  if ((pext[(y + g.ry) * S + ((x + g.r32) >> 5)].z >> (x & 31)) & 1u)
+                    both += (int)swap_on_segment(sq, dv.x, dv.y, x, y, px, py, H, W) << 16;
+                }
+                both = __reduce_add_sync(0xffffffffu, both);
+                if (lane == src) {
+                  d0[u] -= both & 0xffff;
+                  d1[u] -= both >> 16;
+                }
               }
             }
           }
-          if (k < k_hi) {
-            if (dcounts) {
+          float acc[kU];
+#pragma unroll
+          for (int u = 0; u < kU; ++u) {
+            const int k = k0 + lane + u * nthr;
+            acc[u] = part && (d0[u] | d1[u]) ? part[k] : 0.0f;
+            if (dcounts && k < k_hi) {
               int32_t* dk = dcounts + (int64_t)k * 2 * g.n_canon + vq;
-              dk[0] = d0;
-              dk[g.n_canon] = d1;
+              dk[0] = d0[u];
+              dk[g.n_canon] = d1[u];
             }
-            if (part && (d0 | d1)) part[k] = swap_add_error(part[k], d0, d1, dd0, dd1, g);
           }
+#pragma unroll
+          for (int u = 0; u < kU; ++u)
+            if (part && (d0[u] | d1[u])) part[k0 + lane + u * nthr] = swap_add_error(acc[u], d0[u], d1[u], dd0, dd1, g);
         }
       } else {
         for (int k = k_lo + warp; k < k_hi; k += nwarps) {
           int d0 = 0, d1 = 0;
-          const uint4 c = __ldg(reinterpret_cast<const uint4*>(cand) + k);
-          if (any && c.z != c.w) {
-            const int ax = c.z & 0xffff, ay = c.z >> 16, bx = c.w & 0xffff, by = c.w >> 16;
+          const uint2 c = __ldg(cand.pixel + k);
+          if (any && c.x != c.y) {
+            const int ax = c.x & 0xffff, ay = c.x >> 16, bx = c.y & 0xffff, by = c.y >> 16;
             int e0 = 0, e1 = 0;
             for (int i = lane; i < nq; i += 32) {
               const short2 s = sq[i];
@@ -559,15 +589,33 @@ __global__ void __launch_bounds__(kSwapThreads, 3) swap_kernel(SwapArgs g, const
 // ---------------------------------------------------------------------------
 // Host side
 
+static int swap_threads_per_vector(int words) {
+  return std::min(kSwapThreads, std::max(32, ((words + 1) / 2 + 31) / 32 * 32));
+}
+
+// Chunks hold equally many pixels, but long segments leave the walk early and
+// mostly have nothing for the candidates: whole chunks kept the SMs busy for
+// 64 % of the time (the short vectors' chunks ran on alone), and small windows
+// have fewer chunks than the SMs take blocks.  Parts in 1, 2, 4, 8, 16: 743,
+// 527, 496, 481, 476 us (4096 candidates, 128x128, window 64) and 104, 72, 66,
+// 76, 105 us (64 candidates, 50x50, full domain; four vectors side by side),
+// the sums over the parts 6, 4, 7, 11, 25 us of the first; so four, but a part
+// has vectors for all groups of its block.
+int swap_planes_split(const DeltaArgs& d) {
+  const int groups = kSwapThreads / swap_threads_per_vector(d.H * ((d.W + 31) / 32));
+  return (int)std::max<int64_t>(1, std::min<int64_t>(4, d.n_canon / std::max(1, d.n_chunks) / groups));
+}
+
 bool swap_planes_apply(const lpf_paths* p) { return std::max(p->host.rx, p->host.ry) + 1 <= kSwapMaxPixels; }
 
 int swap_planes_run(const uint8_t* img_dev, lpf_paths* paths, const int32_t* pairs_dev, int K, int32_t* dcounts_dev,
-                    float* partial_dev, const DeltaArgs& d, cudaStream_t s) {
+                    float* partial_dev, const DeltaArgs& d, int split, bool first, cudaStream_t s) {
   SwapArgs g{};
   g.H = d.H;
   g.W = d.W;
   g.rx = d.rx;
   g.ry = d.ry;
+  g.split = split;
   g.nw = (d.W + 31) / 32;
   g.r32 = ((d.rx + 31) / 32) * 32;
   g.S = (g.nw + ((g.r32 + d.rx) >> 5) + 1) | 1;  // odd: 32 rows in 32 banks
@@ -587,12 +635,17 @@ int swap_planes_run(const uint8_t* img_dev, lpf_paths* paths, const int32_t* pai
   g.inv_norm = d.inv_norm;
   // threads per vector: two words each, so that what a pixel step reads of
   // the segment serves two words; vectors side by side fill small blocks
-  g.tg = std::min(kSwapThreads, std::max(32, ((g.words + 1) / 2 + 31) / 32 * 32));
+  g.tg = swap_threads_per_vector(g.words);
   g.G = kSwapThreads / g.tg;
   const int max_smem = delta_max_smem();
-  // Sums for every pixel cost about H W / 32 (22 n + 130) instructions per
-  // vector, lookups about 28 n + 400 per candidate: equal near K = H W / 48.
-  bool many = (int64_t)K * 48 > (int64_t)g.H * g.W;
+  // Sums for every pixel cost the same for 1 and 256 candidates, lookups a
+  // warp's pass over the segment for each.  Lookups against sums in us:
+  // 64x64, window 32: 35, 45, 65 against 38 (16, 32, 64 candidates); 123x69,
+  // 17x30: 39, 57, 85 against 52; 128x128, 64: 223, 327, 541 against 354 (64,
+  // 128, 256); 250x200, 40: 198, 280 against 453 (128, 256).  Equal near
+  // H W / 250 while a block has fewer than two words per thread, near H W / 96
+  // beyond (the tables then leave room for three blocks on an SM or fewer).
+  bool many = (int64_t)K * (g.words < 2 * kSwapThreads ? 256 : 96) > (int64_t)g.H * g.W;
   if (many) {
     SwapArgs one = g;
     one.G = 1;
@@ -610,28 +663,34 @@ int swap_planes_run(const uint8_t* img_dev, lpf_paths* paths, const int32_t* pai
     paths->swap_cap = need;
   }
   uint32_t* sel = sel_words ? paths->d_swap + img_words : nullptr;
-  SwapCand* cand = reinterpret_cast<SwapCand*>(paths->d_swap + at_cand);
+  SwapCands cand;
+  cand.table = reinterpret_cast<uint2*>(paths->d_swap + at_cand);
+  cand.pixel = cand.table + K;
   g.img = paths->d_swap;
   g.sel = sel;
   const int n = (int)std::max<int64_t>({(int64_t)img_words, (int64_t)sel_words, (int64_t)K});
   swap_prep_kernel<<<std::min((n + 127) / 128, 4096), 128, 0, s>>>(img_dev, g, paths->d_swap, d.sel_ext, d.We, sel,
                                                                    pairs_dev, K, cand, paths->d_status,
                                                                    paths->checked);
-  if (paths->ev_start) cudaEventRecord(paths->ev_start, s);
-  // small windows have few chunks: shares of the candidates (at least one per
+  if (paths->ev_start && first) cudaEventRecord(paths->ev_start, s);
+  // small windows have few parts: shares of the candidates (at least one per
   // warp, or a block's threads' worth) fill the SMs' three blocks, each share
   // with its own walk (79x101, window 25x19, 28 candidates: 162 us without)
-  const int share = many ? kSwapThreads : kSwapWarps;
-  const dim3 grid(d.n_chunks, std::max(1, std::min(3 * delta_num_sms() / d.n_chunks, (K + share - 1) / share)));
-  if (many) swap_kernel<true><<<grid, g.G * g.tg, smem, s>>>(g, cand, K, dcounts_dev, partial_dev);
-  else swap_kernel<false><<<grid, g.G * g.tg, smem, s>>>(g, cand, K, dcounts_dev, partial_dev);
+  const int share = many ? kSwapThreads : kSwapWarps, parts = d.n_chunks * split;
+  const dim3 grid(parts, std::max(1, std::min(3 * delta_num_sms() / parts, (K + share - 1) / share)));
+  // several candidates at a time hide the latency of their loads (4096 of
+  // them: 929 us one by one, 815 by two, 746 by four, 817 by eight, before the
+  // parts), but cost where a thread has one at most (64: 110, 119, 123, 174)
+  const bool several = (K + (int)grid.y - 1) / (int)grid.y > g.G * g.tg;
+  auto kernel = !many ? swap_kernel<0> : several ? swap_kernel<kSwapUnroll> : swap_kernel<1>;
+  kernel<<<grid, g.G * g.tg, smem, s>>>(g, cand, K, dcounts_dev, partial_dev);
   if (paths->ev_stop) cudaEventRecord(paths->ev_stop, s);
   return LPF_OK;
 }
 
 int swap_planes_attributes(int optin, int* max_static) {
   cudaFuncAttributes fa;
-  for (const void* fn : {(const void*)swap_kernel<true>, (const void*)swap_kernel<false>}) {
+  for (const void* fn : {(const void*)swap_kernel<0>, (const void*)swap_kernel<1>, (const void*)swap_kernel<kSwapUnroll>}) {
     cudaError_t e = cudaFuncGetAttributes(&fa, fn);
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);

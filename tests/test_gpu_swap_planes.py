@@ -66,3 +66,21 @@ def test_sampled_translations(gpu_lib, H, W, rx, ry, copies):
                                       torch.from_numpy(np.tile(pairs, (copies, 1))).cuda())
     assert gpu_lib.lpf_paths_status(p) == 0
     assert all(np.array_equal(c, np.stack(ref)) for c in dc.cpu().numpy().reshape(copies, 5, 2, -1))
+
+
+def test_rounds_of_candidates(gpu_lib):
+    """More candidates than the sums of one round hold: every copy has the sums
+    and count changes of a short call."""
+    H = W = 128
+    r, k, copies = 64, 100, 1500
+    cell = synth.clustered_disks(H, W, 0.4, seed=5)
+    pairs = synth.swap_candidates(cell, k, seed=6).astype(np.int32)
+    p = gpu_lib.lpf_build_paths(r, r)
+    d, tp = torch.from_numpy(cell).cuda(), torch.from_numpy(pairs).cuda()
+    counts = gpu_lib.lpf_full(d, p)
+    target = (counts.double() / cell.size * 0.9).float()
+    dc, one = gpu_lib.lpf_delta_swap(d, p, tp, target=target, counts=counts, want_de=True)
+    assert np.array_equal(dc[:2].cpu().numpy(), oracle.delta_swap(cell, r, r, pairs[:2]))
+    _, de = gpu_lib.lpf_delta_swap(d, p, tp.repeat(copies, 1), target=target, counts=counts, want_de=True,
+                                   want_dcounts=False)
+    assert (de.reshape(copies, k) == one).all()
