@@ -453,12 +453,14 @@ int delta_swap_run(const uint8_t* img_dev, int32_t H, int32_t W, lpf_paths* path
     // Candidates in rounds whose sums per part fill at most kPartialFloats;
     // the walks' share of a round that long is small.
     const int split = whole_chunks ? 1 : swap_planes_split(g), rows = g.n_chunks * split;
-    const int round = de_dev ? std::max(1, std::min(K, kPartialFloats / rows)) : K;
-    if (de_dev && (rc = ensure_partial(paths, round, rows))) return rc;
-    for (int k0 = 0; k0 < K; k0 += round) {
-      const int n = std::min(round, K - k0);
-      rc = swap_planes_run(img_dev, paths, pairs_dev + 2 * (int64_t)k0, n,
-                           dcounts_dev ? dcounts_dev + (int64_t)k0 * 2 * g.n_canon : nullptr,
+    // (Room for them also without error changes: a later call that wants them,
+    // perhaps under stream capture, allocates nothing.)
+    const int fit = std::max(1, std::min(K, kPartialFloats / rows)), round = de_dev ? fit : K;
+    if ((rc = ensure_partial(paths, fit, rows))) return rc;
+    for (int64_t k0 = 0; k0 < K; k0 += round) {
+      const int n = (int)std::min<int64_t>(round, K - k0);
+      rc = swap_planes_run(img_dev, paths, pairs_dev + 2 * k0, n,
+                           dcounts_dev ? dcounts_dev + k0 * 2 * g.n_canon : nullptr,
                            de_dev ? paths->d_partial : nullptr, g, split, k0 == 0, s);
       if (rc) return rc;
       if (!de_dev) continue;
@@ -470,7 +472,7 @@ int delta_swap_run(const uint8_t* img_dev, int32_t H, int32_t W, lpf_paths* path
     }
   } else {
     // segments over 255 pixels: early-exit walks
-    if (de_dev && (rc = ensure_partial(paths, K, g.n_chunks))) return rc;
+    if ((rc = ensure_partial(paths, K, g.n_chunks))) return rc;
     float* partial = de_dev ? paths->d_partial : nullptr;
     const int blocks = (int)std::min<int64_t>((g.ext_bytes + 255) / 256, 4096);
     build_ext_kernel<<<blocks, 256, 0, s>>>(img_dev, H, W, g.rx, g.ry, g.We, g.He, g.ext_bytes, paths->d_ext,
