@@ -328,7 +328,7 @@ def extra_s2(lpf, reps: int = 20):
         lpf.s2_fft(d, 1, out)
     b.record()
     torch.cuda.synchronize()
-    return {"workload": "s2_fft 512x512, one phase, double-precision FFT", "ms_per_call": a.elapsed_time(b) / reps}
+    return {"workload": "s2_fft 512x512, one phase, exact integer transform", "ms_per_call": a.elapsed_time(b) / reps}
 
 
 def extra_proposer(lpf):

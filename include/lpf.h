@@ -338,10 +338,12 @@ int lpf_delta_swap_mc(const uint8_t *img_dev, int32_t H, int32_t W, lpf_paths *p
  * chi the indicator of the phase, which equals the direct periodic sum of
  * Eq. (S2dis) over (x1, y1) of chi(x1,y1) chi((x1+x)%W, (y1+y)%H) / (W*H).
  * img_dev: H*W uint8 (0/1); s2_dev: float [H][W] (row y = row offset,
- * column x = column offset).  Transforms in double precision (cuFFT), result
- * rounded to float32.  The first call for a size creates FFT plans and a
- * work area (cached per device and size; not for use inside stream capture
- * the first time).  H*W <= 2^26.  Errors: LPF_EINVAL, LPF_ECUDA, LPF_ENOMEM.
+ * column x = column offset).  The counts are computed exactly by number-
+ * theoretic transforms and divided in double precision, then rounded to float32; images whose transforms
+ * are longer than 4096 or hold more than 2^22 values go through double-
+ * precision FFTs (cuFFT), whose plans and work area the first call for a size
+ * creates (cached per device and size; not inside stream capture the first
+ * time).  H*W <= 2^26.  Errors: LPF_EINVAL, LPF_ECUDA, LPF_ENOMEM.
  */
 int s2_fft(const uint8_t *img_dev, int32_t H, int32_t W, int32_t phase, float *s2_dev,
            lpf_stream_t stream);
@@ -529,8 +531,9 @@ int lpf_sa_create_mc(uint8_t *cell_dev, int32_t H, int32_t W, lpf_paths *paths, 
  * after the run is done do nothing.
  * Lineal-path runs use one cooperative launch of a persistent kernel for up
  * to 4096 batches (or the proposer's refresh interval), whose resident
- * blocks keep the cell on chip and meet at a bounded grid barrier once per
- * batch.  S2 runs (and devices without cooperative launch) use one kernel
+ * blocks keep the cell on chip and exchange their partial sums once per
+ * batch, by messages (up to three candidates) or through a grid barrier, both
+ * with bounded waits.  S2 runs (and devices without cooperative launch) use one kernel
  * launch per batch, the first call with n_batches >= 16 (or >= the refresh
  * interval) capturing that many as a CUDA graph that is replayed afterwards.
  * Both give the same run.  Errors: LPF_EINVAL, LPF_ECUDA.
@@ -538,7 +541,7 @@ int lpf_sa_create_mc(uint8_t *cell_dev, int32_t H, int32_t W, lpf_paths *paths, 
 int lpf_sa_run(lpf_sa *sa, int32_t n_batches, lpf_stream_t stream);
 
 /* Synchronise `stream` and copy the run's counters to *out.  LPF_ETIMEOUT if
- * a bounded wait in a batch kernel gave up (staging copy or grid barrier)
+ * a bounded wait in a batch kernel gave up (staging copy, message or grid barrier)
  * since the last read: the library has then already made the state
  * consistent again -- counts recomputed from the cell, the error from the
  * counts, the run's counters those of the cell's last applied batch -- so
