@@ -312,8 +312,11 @@ int lpf_delta_swap(const uint8_t *img_dev, int32_t H, int32_t W, lpf_paths *path
  * after another in imgs_dev (uint8 [n_img][H][W]), e.g. the parallel cuts of
  * a volume: the ensemble average over cuts of Sec. 6.3 is counts / (n_img *
  * H * W).  counts_dev: int64 [2][n_vec_full] as in lpf_full.  The images are
- * evaluated side by side on `stream`, as many per pack and walk launch as the
- * handle's work area holds (64 MiB of packed rows, or one image).
+ * evaluated side by side on `stream`, as many per pack and walk launch as fit
+ * in 64 MiB of packed rows (at least one).  The handle keeps an area of that
+ * size or less for them beside lpf_full's; a call with more images or larger
+ * ones than before may allocate a larger one, and the smaller ones are kept
+ * with the handle (less than 192 MiB in all), so captured calls stay valid.
  * Errors: as lpf_full; n_img < 1 is LPF_EINVAL.
  */
 int lpf_full_ensemble(const uint8_t *imgs_dev, int32_t n_img, int32_t H, int32_t W, lpf_paths *paths,

@@ -480,6 +480,22 @@ int ensure_device(lpf_paths* p, size_t packed_words) {
   return LPF_OK;
 }
 
+// Room for the packed rows of several images.  An area that was too small is
+// kept until the handle goes: graphs that captured an ensemble still use it
+// (areas at least double up to kEnsembleWords: all of them together hold less
+// than 192 MiB).
+constexpr size_t kEnsembleWords = size_t(1) << 24;  // packed words (64 MiB)
+static int ensure_stack(lpf_paths* p, size_t words) {
+  if (words <= p->stack_cap) return LPF_OK;
+  const size_t cap = std::max(words, std::min(2 * p->stack_cap, kEnsembleWords));
+  uint32_t* area = nullptr;
+  if (cudaError_t e = cudaMalloc(&area, cap * 4)) return set_cuda_error(e);
+  if (p->d_stack) p->stack_old.push_back(p->d_stack);
+  p->d_stack = area;
+  p->stack_cap = cap;
+  return LPF_OK;
+}
+
 int bake(lpf_paths* p, const Program& prog0, const Geometry& g0, const Program* prog1, const Geometry* g1,
          Baked& b) {
   const int S1 = prog1 ? g1->S : -1, r32_1 = prog1 ? g1->r32 : -1;
@@ -730,8 +746,12 @@ static int run_full(const uint8_t* img, int H, int W, lpf_paths* p, int64_t* cou
     rc = stack_images(sd, n_img);
     if (rc) return rc;
   }
-  rc = ensure_device(p, sd.packed_words);
+  // (The rows of several images have an area of their own: d_packed stays where
+  // it is for the size it was made for, which captured calls rely on.)
+  rc = ensure_device(p, one.packed_words);
+  if (!rc && n_img > 1) rc = ensure_stack(p, sd.packed_words);
   if (rc) return rc;
+  uint32_t* const packed = n_img > 1 ? p->d_stack : p->d_packed;
   if ((rc = num_sms())) return rc;
   const Which which = standard ? Which::kPlain : tree_pieces(p, one, n_img);
   const Program& prog0 = side_program(p, which, 0);
@@ -748,7 +768,7 @@ static int run_full(const uint8_t* img, int H, int W, lpf_paths* p, int64_t* cou
   cudaError_t e = cudaSuccess;
   // pack the rows; zero the counts (unless accumulating) and the work
   // counters (not the status flags)
-  launch_pack(img, sd, p->d_packed, counts, accumulate ? 0 : 2 * n_full, p->d_status, p, s, n_img);
+  launch_pack(img, sd, packed, counts, accumulate ? 0 : 2 * n_full, p->d_status, p, s, n_img);
   const uint32_t* sel0 = nullptr;
   const uint32_t* sel1 = nullptr;
   if (sel) {
@@ -776,7 +796,7 @@ static int run_full(const uint8_t* img, int H, int W, lpf_paths* p, int64_t* cou
   p->nominal_pixels = prog0.n_pixel_words * one.g[0].nbg * tiles_of(one.g[0]);
   if (one.n == 2) p->nominal_pixels += prog1.n_pixel_words * one.g[1].nbg * tiles_of(one.g[1]);
   if (p->ev_start) cudaEventRecord(p->ev_start, s);
-  launch_walk(sd, b, p->d_packed, sel0, sel1, c, n_full, base, p->d_status, p, blocks, s);
+  launch_walk(sd, b, packed, sel0, sel1, c, n_full, base, p->d_status, p, blocks, s);
   if (p->ev_stop) cudaEventRecord(p->ev_stop, s);
   if (mirror && n_full > 1) {
     const int64_t n = 2 * (n_full - base - 1);
@@ -789,7 +809,6 @@ static int run_full(const uint8_t* img, int H, int W, lpf_paths* p, int64_t* cou
 // Summed counts of n images: as many of them per set of launches as the work
 // area and the unit counters hold (one by one, 64 images of 100x128 take 64
 // times three launches that each leave most of the GPU idle: 2.55 ms).
-constexpr size_t kEnsembleWords = size_t(1) << 24;  // packed words (64 MiB)
 static int run_ensemble(const uint8_t* imgs, int n, int H, int W, lpf_paths* p, int64_t* counts, cudaStream_t s) {
   int per = 1;
   if (p && p->host.dims == 2 && H >= 1 && W >= 1 && H <= 8192 && W <= 8192 && p->host.rx < W && p->host.ry < H) {
@@ -797,9 +816,12 @@ static int run_ensemble(const uint8_t* imgs, int n, int H, int W, lpf_paths* p, 
     for (const Tuned& t : p->tuned)
       if (t.H == H && t.W == W) { T = t.T; BB = t.BB; }
     Sides sd;
-    if (make_sides(p->host, H, W, T, BB, sd) == LPF_OK)
+    if (make_sides(p->host, H, W, T, BB, sd) == LPF_OK) {
+      size_t each = 0;  // packed words of an image among others (stack_images)
+      for (int q = 0; q < sd.n; ++q) each += (size_t)((sd.g[q].rows + 3) & ~3) * sd.g[q].S;
       per = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)n, kMaxBandGroups / sd.nbg, 65535,
-                                                         (int64_t)(kEnsembleWords / (sd.packed_words + 64))}));
+                                                         (int64_t)((kEnsembleWords - 16) / each)}));
+    }
   }
   for (int i = 0; i < n; i += per) {
     const int m = std::min(per, n - i);
@@ -1166,6 +1188,8 @@ void lpf_paths_free(lpf_paths* p) {
     cudaFree(p->plain.d_words);
     cudaFree(p->plain.d_piece);
     cudaFree(p->d_packed);
+    cudaFree(p->d_stack);
+    for (uint32_t* old : p->stack_old) cudaFree(old);
     cudaFree(p->d_status);
     cudaFree(p->delta.d_doff);
     cudaFree(p->delta.d_dptr);

@@ -107,6 +107,9 @@ struct lpf_paths {
   lpf::Baked tree, plain, fine;
   uint32_t* d_packed = nullptr;  // work area: packed image (one at a time)
   size_t packed_cap = 0;         // words
+  uint32_t* d_stack = nullptr;   // work area: packed images of an ensemble, side by side
+  size_t stack_cap = 0;          // words
+  std::vector<uint32_t*> stack_old;  // areas it grew out of
   int* d_status = nullptr;       // [0] status flags since the last check, [1] work counter,
                                  // [2..3] pixel words the walk warps ANDed (uint64)
   int64_t nominal_pixels = 0;    // the same without the zero-count skip, for the last walk
