@@ -317,6 +317,10 @@ int lpf_delta_swap(const uint8_t *img_dev, int32_t H, int32_t W, lpf_paths *path
  * size or less for them beside lpf_full's; a call with more images or larger
  * ones than before may allocate a larger one, and the smaller ones are kept
  * with the handle (less than 192 MiB in all), so captured calls stay valid.
+ * It may also upload the program in longer pieces than lpf_full's of that
+ * size.  Under stream capture it makes do with what an earlier lpf_full or
+ * lpf_full_ensemble of that size left on the device: those pieces, and as many
+ * images at a time as the area holds (as lpf_full does with an ensemble's).
  * Errors: as lpf_full; n_img < 1 is LPF_EINVAL.
  */
 int lpf_full_ensemble(const uint8_t *imgs_dev, int32_t n_img, int32_t H, int32_t W, lpf_paths *paths,

@@ -597,6 +597,13 @@ static Which tree_pieces(const lpf_paths* p, const Sides& sd, int n_img) {
   return units < 32 * (int64_t)g_num_sms ? Which::kFine : Which::kTree;
 }
 
+// Whether calls on s are being recorded into a graph (when nothing can be
+// allocated or uploaded).
+static bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(s, &st) == cudaSuccess && st != cudaStreamCaptureStatusNone;
+}
+
 // Bake one of the image's programs for the sides.
 static int bake_sides(lpf_paths* p, const Sides& sd, Which w) {
   return bake(p, side_program(p, w, 0), sd.g[0], sd.n == 2 ? &side_program(p, w, 1) : nullptr,
@@ -753,7 +760,13 @@ static int run_full(const uint8_t* img, int H, int W, lpf_paths* p, int64_t* cou
   if (rc) return rc;
   uint32_t* const packed = n_img > 1 ? p->d_stack : p->d_packed;
   if ((rc = num_sms())) return rc;
-  const Which which = standard ? Which::kPlain : tree_pieces(p, one, n_img);
+  Which which = standard ? Which::kPlain : tree_pieces(p, one, n_img);
+  if (!standard && !baked_for_sides(baked_program(p, which), one)) {
+    // A recorded ensemble walks the pieces an image of its size left on the
+    // device, a recorded image those of an ensemble, rather than fail.
+    const Which other = which == Which::kFine ? Which::kTree : Which::kFine;
+    if (baked_for_sides(baked_program(p, other), one) && capturing(s)) which = other;
+  }
   const Program& prog0 = side_program(p, which, 0);
   const Program& prog1 = side_program(p, which, 1);
   Baked& b = baked_program(p, which);
@@ -821,6 +834,8 @@ static int run_ensemble(const uint8_t* imgs, int n, int H, int W, lpf_paths* p, 
       for (int q = 0; q < sd.n; ++q) each += (size_t)((sd.g[q].rows + 3) & ~3) * sd.g[q].S;
       per = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)n, kMaxBandGroups / sd.nbg, 65535,
                                                          (int64_t)((kEnsembleWords - 16) / each)}));
+      const int64_t room = p->stack_cap > 16 ? (int64_t)((p->stack_cap - 16) / each) : 0;
+      if (per > room && per > 1 && capturing(s)) per = (int)std::max<int64_t>(1, room);  // (no new area then)
     }
   }
   for (int i = 0; i < n; i += per) {

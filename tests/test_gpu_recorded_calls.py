@@ -1,5 +1,7 @@
-"""Calls recorded into a CUDA graph stay valid while the same handle evaluates
-ensembles: their work areas do not move."""
+"""Calls recorded into a CUDA graph: they stay valid while the same handle
+evaluates ensembles (their work areas do not move), and after one plain
+evaluation of an image its ensembles can be recorded, and the other way
+round."""
 import numpy as np
 import pytest
 import torch
@@ -40,3 +42,28 @@ def test_recorded_evaluations_outlive_larger_ensembles(gpu_lib):
     np.testing.assert_array_equal(c1.cpu().numpy(), ref[id(first)])
     np.testing.assert_array_equal(c4.cpu().numpy(), ref[id(few)])
     assert (scratch == -1).all() and gpu_lib.lpf_paths_status(p) == 0
+
+
+def test_recorded_ensemble_after_a_plain_evaluation(gpu_lib):
+    H, W, rx, ry = 40, 61, 13, 9
+    imgs = _images(5, H, W, 7)
+    p = gpu_lib.lpf_build_paths(rx, ry)
+    d, c = torch.from_numpy(imgs).cuda(), torch.empty((2, p.n_full), dtype=torch.int64, device="cuda")
+    gpu_lib.lpf_full(d[0], p)
+    _graph(lambda: gpu_lib.lpf_full_ensemble(d, p, c)).replay()
+    np.testing.assert_array_equal(c.cpu().numpy(), sum(oracle.lpf_full(i, rx, ry) for i in imgs))
+    gpu_lib.lpf_full_ensemble(d[:3].contiguous(), p)  # now an area for three, still none for five
+    c.zero_()
+    _graph(lambda: gpu_lib.lpf_full_ensemble(d, p, c)).replay()
+    np.testing.assert_array_equal(c.cpu().numpy(), sum(oracle.lpf_full(i, rx, ry) for i in imgs))
+
+
+def test_recorded_evaluation_after_a_plain_ensemble(gpu_lib):
+    H, W, rx, ry = 40, 61, 30, 28
+    imgs = _images(200, H, W, 7)  # enough for the long pieces, which one image would not take
+    p = gpu_lib.lpf_build_paths(rx, ry)
+    d, c = torch.from_numpy(imgs).cuda(), torch.empty((2, p.n_full), dtype=torch.int64, device="cuda")
+    gpu_lib.lpf_full_ensemble(d, p)
+    _graph(lambda: gpu_lib.lpf_full(d[0], p, c)).replay()
+    np.testing.assert_array_equal(c.cpu().numpy(), oracle.lpf_full(imgs[0], rx, ry))
+    assert gpu_lib.lpf_paths_status(p) == 0
