@@ -21,8 +21,8 @@
 // phase and gains its new one: over all translations the two exchanged
 // pixels cancel, over a sample of translations they need not.
 //
-// Segments of up to 255 pixels are evaluated from bit planes (lpf_swap.cu);
-// the walks here serve longer ones.
+// Segments of up to 255 pixels are evaluated from bit planes (lpf_swap.cu)
+// where those fit in shared memory; the walks here serve the rest.
 //
 // Work split: blocks = (vector chunk) x (candidate stride); each block stages
 // the extended cell once (one bulk copy of a copy built per call in global
@@ -449,7 +449,7 @@ int delta_swap_run(const uint8_t* img_dev, int32_t H, int32_t W, lpf_paths* path
   g.phase_mask = phase_mask;
   g.sel_ext = sel_ext;
   if (inv_norm > 0.0f) g.inv_norm = inv_norm;
-  if (swap_planes_apply(paths)) {
+  if (swap_planes_apply(g)) {
     // Candidates in rounds whose sums per part fill at most kPartialFloats;
     // the walks' share of a round that long is small.
     const int split = whole_chunks ? 1 : swap_planes_split(g), rows = g.n_chunks * split;
@@ -471,7 +471,7 @@ int delta_swap_run(const uint8_t* img_dev, int32_t H, int32_t W, lpf_paths* path
         delta_reduce_kernel<<<blocks, 256, 0, s>>>(paths->d_partial, rows, n, de_dev + k0);
     }
   } else {
-    // segments over 255 pixels: early-exit walks
+    // early-exit walks over the extended cell
     if ((rc = ensure_partial(paths, K, g.n_chunks))) return rc;
     float* partial = de_dev ? paths->d_partial : nullptr;
     const int blocks = (int)std::min<int64_t>((g.ext_bytes + 255) / 256, 4096);

@@ -606,10 +606,8 @@ int swap_planes_split(const DeltaArgs& d) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(4, d.n_canon / std::max(1, d.n_chunks) / groups));
 }
 
-bool swap_planes_apply(const lpf_paths* p) { return std::max(p->host.rx, p->host.ry) + 1 <= kSwapMaxPixels; }
-
-int swap_planes_run(const uint8_t* img_dev, lpf_paths* paths, const int32_t* pairs_dev, int K, int32_t* dcounts_dev,
-                    float* partial_dev, const DeltaArgs& d, int split, bool first, cudaStream_t s) {
+// The kernel's arguments for this cell and window, but for the candidates' part.
+static SwapArgs swap_args(const DeltaArgs& d, int split) {
   SwapArgs g{};
   g.H = d.H;
   g.W = d.W;
@@ -637,6 +635,24 @@ int swap_planes_run(const uint8_t* img_dev, lpf_paths* paths, const int32_t* pai
   // the segment serves two words; vectors side by side fill small blocks
   g.tg = swap_threads_per_vector(g.words);
   g.G = kSwapThreads / g.tg;
+  return g;
+}
+
+// Segments of up to 255 pixels, of cells whose packed rows and one vector's
+// planes fit in shared memory.  Nearly all cells whose extended copy (a byte
+// per pixel) fits do: 32 columns take 16 bytes here.  But high cells of little
+// more than 32 columns pad them to two words (6000 rows of 33, window 1x1: 264
+// KB against 216 KB of the extended copy).
+bool swap_planes_apply(const DeltaArgs& d) {
+  if (std::max(d.rx, d.ry) + 1 > kSwapMaxPixels) return false;
+  SwapArgs g = swap_args(d, 1);
+  g.G = 1;
+  return swap_smem(g, false) <= (size_t)delta_max_smem();
+}
+
+int swap_planes_run(const uint8_t* img_dev, lpf_paths* paths, const int32_t* pairs_dev, int K, int32_t* dcounts_dev,
+                    float* partial_dev, const DeltaArgs& d, int split, bool first, cudaStream_t s) {
+  SwapArgs g = swap_args(d, split);
   const int max_smem = delta_max_smem();
   // Sums for every pixel cost the same for 1 and 256 candidates, lookups a
   // warp's pass over the segment for each.  Lookups against sums in us:
@@ -652,8 +668,7 @@ int swap_planes_run(const uint8_t* img_dev, lpf_paths* paths, const int32_t* pai
     if (swap_smem(one, true) > (size_t)max_smem) many = false;  // the tables of a large cell do not fit
   }
   while (g.G > 1 && swap_smem(g, many) > (size_t)max_smem / 3) --g.G;
-  const size_t smem = swap_smem(g, many);
-  if (smem > (size_t)max_smem) return LPF_EUNSUPPORTED;
+  const size_t smem = swap_smem(g, many);  // (at most max_smem: swap_planes_apply)
   const size_t img_words = (size_t)swap_img_words(g.H, g.ry, g.S), sel_words = d.sel_ext ? (size_t)g.words : 0;
   const size_t at_cand = (img_words + sel_words + 3) & ~size_t(3), need = at_cand + 4 * (size_t)K;
   cudaError_t e;

@@ -7,8 +7,9 @@ struct lpf_paths;
 
 namespace lpf {
 struct DeltaArgs;
-// Whether the handle's segments are short enough (255 pixels).
-bool swap_planes_apply(const lpf_paths* p);
+// Whether segments are short enough (255 pixels) and the planes fit in shared
+// memory.  d: geometry after delta_prepare.
+bool swap_planes_apply(const DeltaArgs& d);
 // Parts that a chunk's vectors are best cut into (by the cell and window alone,
 // so that sums do not depend on how many candidates a call has).
 int swap_planes_split(const DeltaArgs& d);
