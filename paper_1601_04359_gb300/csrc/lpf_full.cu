@@ -163,11 +163,16 @@ static int stack_images(Sides& s, int n) {
 // (z, b) stages rows z * slice_rows + 32 BB b onwards: its 32 BB
 // translation rows, ry above and below them, and the rz following slices.
 int make_geometry3(int D, int H, int W, int rx, int ry, int rz, int T, int BB, Geometry& g) {
-  if (T <= 0 && W > 64 && W <= 128 && H > 32 && ((H + 31) / 32) % 2 == 0) {
-    // two bands per tile (a window this size stages few bands either way)
-    T = 8;
-    if (BB <= 0) BB = 4;
-    if (((H + 31) / 32) % 4 != 0) BB = 2;
+  const int nbands = (H + 31) / 32;
+  if (T <= 0 && W > 64 && W <= 128 && nbands % 2 == 0) {
+    // Two bands per tile (a window this size stages few bands either way).  An
+    // odd number of pairs goes two bands per group, which are more groups than
+    // with four (2000x320x128: 10000 and 6000): not where they are too many.
+    const int bands = nbands % 4 == 0 ? 4 : 2;
+    if ((int64_t)D * (nbands / bands) <= kMaxBandGroups) {
+      T = 8;
+      BB = bands;
+    }
   }
   int rc = make_geometry(H, W, rx, ry, T, BB, g);
   if (rc && rc != LPF_EUNSUPPORTED) return rc;
