@@ -346,11 +346,14 @@ int lpf_delta_swap_mc(const uint8_t *img_dev, int32_t H, int32_t W, lpf_paths *p
  * Eq. (S2dis) over (x1, y1) of chi(x1,y1) chi((x1+x)%W, (y1+y)%H) / (W*H).
  * img_dev: H*W uint8 (0/1); s2_dev: float [H][W] (row y = row offset,
  * column x = column offset).  The counts are computed exactly by number-
- * theoretic transforms and divided in double precision, then rounded to float32; images whose transforms
- * are longer than 4096 or hold more than 2^22 values go through double-
- * precision FFTs (cuFFT), whose plans and work area the first call for a size
- * creates (cached per device and size; not inside stream capture the first
- * time).  H*W <= 2^26.  Errors: LPF_EINVAL, LPF_ECUDA, LPF_ENOMEM.
+ * theoretic transforms, divided in double precision and rounded to float32.
+ * Their work area (at most 25 MB) is the call's own; that of a call recorded
+ * into a CUDA graph is held as long as the graph.  Images whose transforms are
+ * longer than 4096 or hold more than 2^22 values go through double-precision
+ * FFTs (cuFFT), whose plans and work area the first call for a size creates
+ * (cached per device and size and shared by all calls of it, which therefore
+ * must not overlap, nor graphs that recorded them; not inside stream capture
+ * the first time).  H*W <= 2^26.  Errors: LPF_EINVAL, LPF_ECUDA, LPF_ENOMEM.
  */
 int s2_fft(const uint8_t *img_dev, int32_t H, int32_t W, int32_t phase, float *s2_dev,
            lpf_stream_t stream);

@@ -31,6 +31,7 @@
 #include <cufft.h>
 
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 #include <vector>
 
@@ -330,30 +331,78 @@ int ntt_log(int n) {
   return lg;
 }
 
-// A call recorded into a graph takes an area of its image size that stays
-// (shared by every graph of that size, as cuFFT's plans and buffers are): an
-// allocation in stream order would become a node of the graph, which then
-// could not be copied or instantiated twice.
+// A call recorded into a graph takes an area of its own, which the graph holds
+// (as a user object: so do its copies and the executables made from it, while
+// they run too): two recorded calls may run side by side, from two graphs or
+// on two branches of one.  An allocation in stream order would become a node of
+// the graph, which then could not be copied or instantiated twice; so the area
+// comes from the pool on a stream of the library's own and goes back there with
+// the first call after the last graph that held it.
 struct NttArea {
-  int dev, H, W;
-  uint32_t* area;
+  uint32_t* p = nullptr;
+  std::atomic<bool> idle{false};  // set by the runtime's thread, which must not call CUDA
 };
-std::vector<NttArea> g_ntt_areas;
+struct NttRecorded {
+  cudaStream_t stream = nullptr;
+  std::vector<NttArea*> areas;
+};
+NttRecorded g_ntt_recorded[64];
 
-int recorded_area(int dev, int H, int W, size_t bytes, uint32_t** out) {
-  std::lock_guard<std::mutex> lock(g_ntt_mu);
-  for (const NttArea& a : g_ntt_areas)
-    if (a.dev == dev && a.H == H && a.W == W) { *out = a.area; return LPF_OK; }
+// Areas that no graph holds any more back to the pool (g_ntt_mu held).
+void give_back_areas(NttRecorded& r) {
+  for (size_t i = 0; i < r.areas.size();) {
+    if (r.areas[i]->idle.load(std::memory_order_acquire)) {
+      cudaFreeAsync(r.areas[i]->p, r.stream);
+      delete r.areas[i];
+      r.areas[i] = r.areas.back();
+      r.areas.pop_back();
+    } else {
+      ++i;
+    }
+  }
+}
+
+cudaError_t new_recorded_area(NttRecorded& r, cudaMemPool_t pool, cudaGraph_t graph, size_t bytes, uint32_t** out) {
+  cudaError_t e = cudaSuccess;
+  if (!r.stream && (e = cudaStreamCreateWithFlags(&r.stream, cudaStreamNonBlocking)) != cudaSuccess) return e;
+  give_back_areas(r);
+  uint32_t* p = nullptr;
+  if ((e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&p), bytes, pool, r.stream)) != cudaSuccess) return e;
+  NttArea* area = new NttArea;
+  area->p = p;
+  cudaUserObject_t held = nullptr;
+  e = cudaStreamSynchronize(r.stream);  // (the graph's kernels run on other streams)
+  if (e == cudaSuccess)
+    e = cudaUserObjectCreate(&held, area, [](void* a) { static_cast<NttArea*>(a)->idle.store(true, std::memory_order_release); },
+                             1, cudaUserObjectNoDestructorSync);
+  if (e != cudaSuccess) {
+    cudaFreeAsync(p, r.stream);
+    delete area;
+    return e;
+  }
+  r.areas.push_back(area);
+  if ((e = cudaGraphRetainUserObject(graph, held, 1, cudaGraphUserObjectMove)) != cudaSuccess)
+    cudaUserObjectRelease(held, 1);  // (idle then)
+  *out = p;
+  return e;
+}
+
+int recorded_area(int dev, cudaStream_t s, size_t bytes, uint32_t** out) {
+  cudaMemPool_t pool;
+  if (int rc = ntt_pool(dev, &pool)) return rc;
+  cudaStreamCaptureStatus cap;
+  cudaGraph_t graph = nullptr;
+  cudaError_t e = cudaStreamGetCaptureInfo(s, &cap, nullptr, &graph);
+  if (e != cudaSuccess) return set_cuda_error(e);
+  if (cap != cudaStreamCaptureStatusActive) return set_cuda_error(cudaErrorStreamCaptureInvalidated);
   cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // (allocating is not part of what is recorded)
-  cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
-  if (e != cudaSuccess) return set_cuda_error(e);
-  uint32_t* area = nullptr;
-  e = cudaMalloc(reinterpret_cast<void**>(&area), bytes);
+  if ((e = cudaThreadExchangeStreamCaptureMode(&mode)) != cudaSuccess) return set_cuda_error(e);
+  {
+    std::lock_guard<std::mutex> lock(g_ntt_mu);
+    e = new_recorded_area(g_ntt_recorded[dev], pool, graph, bytes, out);
+  }
   (void)cudaThreadExchangeStreamCaptureMode(&mode);
-  if (e != cudaSuccess) return set_cuda_error(e);
-  g_ntt_areas.push_back({dev, H, W, area});
-  *out = area;
-  return LPF_OK;
+  return set_cuda_error(e);
 }
 
 int s2_ntt(int dev, const uint8_t* img, int H, int W, int phase, float* s2, cudaStream_t s) {
@@ -365,10 +414,14 @@ int s2_ntt(int dev, const uint8_t* img, int H, int W, int phase, float* s2, cuda
   const bool recorded = cap != cudaStreamCaptureStatusNone;
   uint32_t* A = nullptr;
   if (recorded) {
-    if (int rc = recorded_area(dev, H, W, bytes, &A)) return rc;
+    if (int rc = recorded_area(dev, s, bytes, &A)) return rc;
   } else {
     cudaMemPool_t pool;
     if (int rc = ntt_pool(dev, &pool)) return rc;
+    {
+      std::lock_guard<std::mutex> lock(g_ntt_mu);
+      give_back_areas(g_ntt_recorded[dev]);
+    }
     e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&A), bytes, pool, s);
     if (e != cudaSuccess) return set_cuda_error(e);
   }
