@@ -299,7 +299,12 @@ int lpf_full_standard(const uint8_t *img_dev, int32_t H, int32_t W, lpf_paths *p
  * periodically extended cell (W+2rx, padded to an odd number of 4-byte
  * words) x (H+2ry) bytes must fit in shared memory
  * (about 227 KB), else LPF_EUNSUPPORTED.  The first call for a cell width, or
- * with a larger K than before, allocates the handle's tables / work area.
+ * with a larger K than before, allocates the handle's tables / work area: 16
+ * bytes per candidate (an area outgrown is kept with the handle, so calls
+ * recorded for count changes alone stay valid), and partial sums of the error
+ * changes, whether the call wants them or not, at most 8 KB per candidate and,
+ * for windows up to 254, 512 MB in all (replaced when outgrown: calls recorded
+ * with error changes are then to be recorded again).
  * Errors: LPF_EINVAL, LPF_EUNSUPPORTED, LPF_ENOMEM, LPF_ECUDA.
  */
 int lpf_delta_swap(const uint8_t *img_dev, int32_t H, int32_t W, lpf_paths *paths,

@@ -1218,6 +1218,7 @@ void lpf_paths_free(lpf_paths* p) {
     cudaFree(p->delta.d_vec16);
     cudaFree(p->delta.d_shear);
     cudaFree(p->d_swap);
+    for (uint32_t* old : p->swap_old) cudaFree(old);
     cudaFree(p->d_partial);
     cudaFree(p->d_ext);
     cudaFree(p->d_sel);

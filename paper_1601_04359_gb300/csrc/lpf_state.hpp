@@ -124,6 +124,7 @@ struct lpf_paths {
   size_t sel_cap = 0;            // words
   uint32_t* d_swap = nullptr;    // work area of the bit-plane swap deltas: packed rows, selection, candidates
   size_t swap_cap = 0;           // words
+  std::vector<uint32_t*> swap_old;   // areas it grew out of
   int checked = 0;               // 1: kernels that read the image flag pixels other than 0 or 1
   int selftest = 0;              // 1: walks wait for bytes no copy delivers (failure-detection test)
 };

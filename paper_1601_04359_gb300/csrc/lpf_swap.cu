@@ -671,11 +671,17 @@ int swap_planes_run(const uint8_t* img_dev, lpf_paths* paths, const int32_t* pai
   const size_t smem = swap_smem(g, many);  // (at most max_smem: swap_planes_apply)
   const size_t img_words = (size_t)swap_img_words(g.H, g.ry, g.S), sel_words = d.sel_ext ? (size_t)g.words : 0;
   const size_t at_cand = (img_words + sel_words + 3) & ~size_t(3), need = at_cand + 4 * (size_t)K;
-  cudaError_t e;
+  // A larger area replaces the one there is, which is kept until the handle
+  // goes: graphs that recorded calls with count changes alone still use it, as
+  // they could while that area did not depend on K (areas at least double: the
+  // old ones together are smaller than the one in use).
   if (need > paths->swap_cap) {
-    if (paths->d_swap) { cudaDeviceSynchronize(); cudaFree(paths->d_swap); paths->d_swap = nullptr; paths->swap_cap = 0; }
-    if ((e = cudaMalloc(&paths->d_swap, need * 4)) != cudaSuccess) return set_cuda_error(e);
-    paths->swap_cap = need;
+    const size_t cap = std::max(need, 2 * paths->swap_cap);
+    uint32_t* area = nullptr;
+    if (cudaError_t e = cudaMalloc(&area, cap * 4)) return set_cuda_error(e);
+    if (paths->d_swap) paths->swap_old.push_back(paths->d_swap);
+    paths->d_swap = area;
+    paths->swap_cap = cap;
   }
   uint32_t* sel = sel_words ? paths->d_swap + img_words : nullptr;
   SwapCands cand;
