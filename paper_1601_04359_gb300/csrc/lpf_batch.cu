@@ -208,11 +208,12 @@ static inline int t_index(int T) { return T == 1 ? 0 : T == 2 ? 1 : T == 4 ? 2 :
 
 using BatchWalkFn = void (*)(const BatchDesc*, const BatchSlot*, int, int*, int, uint32_t, unsigned long long*);
 
-// gather: some image of the kernel has a window wide enough to re-deal masks.
+// gather: most of the kernel's work is in images that re-deal masks (four words
+// per thread or more: batch_build).
 static BatchWalkFn batch_walk_fn(int k, bool gather) {
   switch (k) {
     case 0: return batch_walk_kernel<1, false>;
-    case 1: return gather ? batch_walk_kernel<2, true> : batch_walk_kernel<2, false>;
+    case 1: return batch_walk_kernel<2, false>;
     case 2: return gather ? batch_walk_kernel<4, true> : batch_walk_kernel<4, false>;
     default: return gather ? batch_walk_kernel<8, true> : batch_walk_kernel<8, false>;
   }
@@ -431,6 +432,7 @@ static int batch_build(lpf_batch* bt, const uint8_t* const* imgs, const int32_t*
   }
   bt->smem = bt->max_band + (gather ? 8u * kBatchThreads : 0u);
   for (int k = 0; k < kBatchTs && gather; ++k) {
+    if (!bt->gather_T[k]) continue;
     cudaFuncAttributes fa;
     if ((e = cudaFuncGetAttributes(&fa, batch_walk_fn(k, true))) != cudaSuccess) return set_cuda_error(e);
     if ((int)bt->smem > optin - (int)fa.sharedSizeBytes) gather = false;
