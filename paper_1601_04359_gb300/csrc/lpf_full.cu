@@ -428,12 +428,15 @@ __global__ void __launch_bounds__(512, 2) walk_kernel(const __grid_constant__ Wa
     parity ^= 1u;
     __syncthreads();
     if (s_abort) break;
-    // One copy of the gathering walk serves both sides (two overflow the
-    // instruction cache: 270 instead of 205 us for the whole domain of
-    // 175x201); without it two copies, with the side's fields as constants,
-    // are the faster ones (18.4 and 18.9 us at 64x64, window 32).
+    // With four or eight words per thread one copy of the walk serves both
+    // sides: an SM whose blocks are on different sides runs two copies at once,
+    // which overflow the instruction cache (175x201, whole domain: 270 against
+    // 205 us; 16 images of 239x230, window 119, side by side: 6009 against 2806
+    // us, one of them at a time 242).  The shorter walks of one and two words
+    // per thread fit twice, and are faster with the side's fields as constants
+    // (18.4 and 18.9 us at 64x64, window 32).
     unsigned long long walked;
-    if (GATHER) walked = walk_band<T, R, GATHER>(sd, lbg, unit_ctr + bg, sm, deal, lane, prog, piece, counts, n_full, base);
+    if (T >= 4) walked = walk_band<T, R, GATHER>(sd, lbg, unit_ctr + bg, sm, deal, lane, prog, piece, counts, n_full, base);
     else if (side) walked = walk_band<T, R, GATHER>(ws.s[1], lbg, unit_ctr + bg, sm, deal, lane, prog, piece, counts, n_full, base);
     else walked = walk_band<T, R, GATHER>(ws.s[0], lbg, unit_ctr + bg, sm, deal, lane, prog, piece, counts, n_full, base);
     if (lbg >= sd.work_from) executed += walked;
