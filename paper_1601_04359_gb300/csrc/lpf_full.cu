@@ -375,6 +375,7 @@ __global__ void __launch_bounds__(512, 2) walk_kernel(const __grid_constant__ Wa
   extern __shared__ __align__(16) uint32_t sm[];
   __shared__ __align__(8) uint64_t bar;
   __shared__ int s_abort, s_next;
+  __shared__ WalkSide s_side;  // the band group's side (T >= 4)
   // per warp, behind the staged rows: masks being re-dealt (deal_at = 0: no room, never)
   uint2* deal = deal_at ? reinterpret_cast<uint2*>(reinterpret_cast<char*>(sm) + deal_at) + (threadIdx.x & ~31u) : nullptr;
   const int lane = threadIdx.x & 31;
@@ -422,6 +423,7 @@ __global__ void __launch_bounds__(512, 2) walk_kernel(const __grid_constant__ Wa
       const size_t row0 = (size_t)(lbg / sd.nbg_s) * sd.slice_rows + (size_t)(lbg % sd.nbg_s) * 32 * sd.BB;
       bulk_g2s(sm, sd.packed + row0 * sd.S, sd.band_bytes, &bar);
     }
+    if (T >= 4 && threadIdx.x == 0) s_side = sd;
     copy_pending = true;
     if (mbar_wait(&bar, parity, wait_rounds)) copy_pending = false;
     else s_abort = 1;
@@ -432,11 +434,12 @@ __global__ void __launch_bounds__(512, 2) walk_kernel(const __grid_constant__ Wa
     // sides: an SM whose blocks are on different sides runs two copies at once,
     // which overflow the instruction cache (175x201, whole domain: 270 against
     // 205 us; 16 images of 239x230, window 119, side by side: 6009 against 2806
-    // us, one of them at a time 242).  The shorter walks of one and two words
+    // us, one of them at a time 242); the side's fields are in shared memory
+    // (from the parameters by index: 128^3, window 16: 1987 -> 2016 us).  The shorter walks of one and two words
     // per thread fit twice, and are faster with the side's fields as constants
     // (18.4 and 18.9 us at 64x64, window 32).
     unsigned long long walked;
-    if (T >= 4) walked = walk_band<T, R, GATHER>(sd, lbg, unit_ctr + bg, sm, deal, lane, prog, piece, counts, n_full, base);
+    if (T >= 4) walked = walk_band<T, R, GATHER>(s_side, lbg, unit_ctr + bg, sm, deal, lane, prog, piece, counts, n_full, base);
     else if (side) walked = walk_band<T, R, GATHER>(ws.s[1], lbg, unit_ctr + bg, sm, deal, lane, prog, piece, counts, n_full, base);
     else walked = walk_band<T, R, GATHER>(ws.s[0], lbg, unit_ctr + bg, sm, deal, lane, prog, piece, counts, n_full, base);
     if (lbg >= sd.work_from) executed += walked;
