@@ -134,7 +134,8 @@ int make_sides(const Paths& paths, int H, int W, int T, int BB, Sides& s) {
   for (int q = 0; q < s.n; ++q)
     units += (int64_t)s.g[q].nbg * tiles_of(s.g[q]) *
              (int64_t)((q ? paths.tree_t : paths.tree).piece_begin.size() - 1);
-  s.gather = std::max(rx, ry) >= kGatherWindow && s.g[0].T >= 4 && units >= kGatherUnits;
+  // (rows that fold are at most 128 wide, both ways: their windows are smaller)
+  s.gather = std::max(rx, ry) >= kGatherWindow && s.g[0].T >= 4 && R == 1 && units >= kGatherUnits;
   if (s.nbg > kMaxBandGroups) return LPF_EUNSUPPORTED;
   return LPF_OK;
 }
@@ -624,14 +625,15 @@ static int bake_sides(lpf_paths* p, const Sides& sd, Which w) {
 using WalkFn = void (*)(const WalkSides, const uint4*, const uint32_t*, unsigned long long*, int64_t, int64_t, int*,
                         uint32_t, int, uint32_t, uint32_t);
 
+// (gather: images alone, see make_sides)
 static WalkFn walk_fn(int T, int R, bool gather) {
   switch (T) {
     case 1: return walk_kernel<1, 1, false>;
-    case 2: return gather ? walk_kernel<2, 1, true> : walk_kernel<2, 1, false>;
+    case 2: return walk_kernel<2, 1, false>;
     case 4: return gather ? walk_kernel<4, 1, true> : walk_kernel<4, 1, false>;
     default:
-      if (R == 4) return gather ? walk_kernel<8, 4, true> : walk_kernel<8, 4, false>;
-      if (R == 2) return gather ? walk_kernel<8, 2, true> : walk_kernel<8, 2, false>;
+      if (R == 4) return walk_kernel<8, 4, false>;
+      if (R == 2) return walk_kernel<8, 2, false>;
       return gather ? walk_kernel<8, 1, true> : walk_kernel<8, 1, false>;
   }
 }
@@ -939,7 +941,9 @@ static int run_full3(const uint8_t* vol, int D, int H, int W, lpf_paths* p, int6
   sd.packed_words = g.packed_words;
   sd.band_bytes = g.band_bytes;
   sd.nbg = g.nbg;
-  sd.gather = std::max(std::max(p->host.rx, p->host.ry), p->host.rz) >= kGatherWindow;
+  // (no re-dealing: volumes with windows of 128 and more along an axis are short
+  // along the others, and lost by it -- 3x160x50, window 2x130x1: 66 -> 87 us;
+  // 200x60x64, 3x3x128: 2080 -> 2330; 160^3, 3x130x2: 3944 -> 3972)
   // 16 warps per block whatever the band group's tile count: warps pull
   // units of any tile of the staged band group, and a volume's band group
   // (its slices with their rz halo) is large, so few blocks fit on an SM

@@ -1,7 +1,7 @@
 """The walks that re-deal few live masks over the lanes, on calls that take
 them: windows from 128 on with four or eight words per thread and enough units
-(images), windows from 120 on (batches), volumes with a window of 128 along any
-axis, also folded ones and those with two words per thread.  References: the
+(images), windows from 120 on (batches); and volumes with a window of 128 along
+an axis, in every shape of tile.  References: the
 oracle for the selections of translations and sampled vectors, and for
 whole tables the walk with one word per thread, which never re-deals."""
 import numpy as np
@@ -65,12 +65,12 @@ def test_batch_of_wide_and_narrow_windows(gpu_lib, T):
 
 
 @pytest.mark.parametrize("D,H,W,rx,ry,rz,shape", [
-    (3, 150, 20, 2, 130, 1, None),        # one word per thread (nothing to re-deal)
+    (3, 150, 20, 2, 130, 1, None),        # one word per thread
     (3, 160, 50, 2, 130, 1, None),        # two words
     (3, 150, 141, 128, 5, 1, None),       # four
     (2, 160, 229, 30, 130, 1, None),      # eight
-    (3, 192, 100, 2, 130, 1, None),       # two bands per tile, two per band group
-    (3, 256, 70, 2, 130, 1, None),        # two bands per tile, four per band group
+    (3, 192, 100, 2, 130, 1, None),       # three words
+    (3, 256, 70, 2, 130, 1, (8, 4)),      # two bands per tile
     (3, 256, 50, 2, 130, 1, (8, 4)),      # four bands per tile
     (131, 33, 60, 1, 1, 128, None),       # the window's long axis across the slices
 ])
