@@ -163,18 +163,7 @@ static int stack_images(Sides& s, int n) {
 // (y'' - ry) mod H of slice z' mod D, z' < D + rz; a block of band group
 // (z, b) stages rows z * slice_rows + 32 BB b onwards: its 32 BB
 // translation rows, ry above and below them, and the rz following slices.
-int make_geometry3(int D, int H, int W, int rx, int ry, int rz, int T, int BB, Geometry& g) {
-  const int nbands = (H + 31) / 32;
-  if (T <= 0 && W > 64 && W <= 128 && nbands % 2 == 0) {
-    // Two bands per tile (a window this size stages few bands either way).  An
-    // odd number of pairs goes two bands per group, which are more groups than
-    // with four (2000x320x128: 10000 and 6000): not where they are too many.
-    const int bands = nbands % 4 == 0 ? 4 : 2;
-    if ((int64_t)D * (nbands / bands) <= kMaxBandGroups) {
-      T = 8;
-      BB = bands;
-    }
-  }
+static int layout_volume(int D, int H, int W, int rx, int ry, int rz, int T, int BB, Geometry& g) {
   int rc = make_geometry(H, W, rx, ry, T, BB, g);
   if (rc && rc != LPF_EUNSUPPORTED) return rc;
   if (const int R = fold(g.T, W, H, g.BB); R > 1) {
@@ -196,6 +185,36 @@ int make_geometry3(int D, int H, int W, int rx, int ry, int rz, int T, int BB, G
   if (band > (size_t)kMaxSmem - 64 || g.nbg > kMaxBandGroups) return LPF_EUNSUPPORTED;
   if (((size_t)g.slice_rows * g.S) % 4 != 0 || ((size_t)32 * g.BB * g.S) % 4 != 0) return LPF_EUNSUPPORTED;
   return LPF_OK;
+}
+
+// Two bands per tile where rows are of three or four words: the decoding of
+// records then serves twice the translations, but there are half as many units
+// (tiles times pieces of the program) for the warps.  That pays from two thirds
+// of a unit per warp slot (152 SMs of 32) and one per warp of a block on, where
+// staging a band group is little beside its units: up to 1024 bytes per unit, or
+// 640 where an odd number of pairs of bands goes two bands per group, which
+// stage more than four together.  Measured over 70 volumes of 64 to 320 rows,
+// windows 3 to 40 (folded / plain, us): 128^3, 10: 462 / 621 (56832 units); 60 x
+// 128 x 128, 6: 69 / 81 (3960), 5: 73 / 59 (2040); 64 x 64 x 96, 6: 65 / 60
+// (2112); 100 x 128 x 70, 2 x 2 x 30: 76 / 68 (1041 bytes); odd pairs, 100 x 320
+// x 128: 10: 1030 / 2078 (439 bytes), 9: 781 / 872 (606), 8: 659 / 598 (815), 4:
+// 423 / 109 (4844).
+constexpr int64_t kFoldUnits = 2 * 32 * 152 / 3;
+constexpr int64_t kFoldUnitsGroup = 16;
+constexpr int64_t kFoldBytes = 1024, kFoldBytesOddPairs = 640;
+
+int make_geometry3(int D, int H, int W, int rx, int ry, int rz, int64_t n_pieces, int T, int BB, Geometry& g) {
+  const int nbands = (H + 31) / 32;
+  if (T <= 0 && W > 64 && W <= 128 && nbands % 2 == 0) {
+    const int bands = nbands % 4 == 0 ? 4 : 2;
+    const int rc = layout_volume(D, H, W, rx, ry, rz, 8, bands, g);
+    const int64_t per_group = tiles_of(g) * n_pieces;
+    const int64_t bytes = bands < std::min(4, nbands) ? kFoldBytesOddPairs : kFoldBytes;
+    if (rc == LPF_OK && per_group >= kFoldUnitsGroup && per_group * g.nbg >= kFoldUnits &&
+        (int64_t)g.band_bytes <= bytes * per_group)
+      return LPF_OK;
+  }
+  return layout_volume(D, H, W, rx, ry, rz, T, BB, g);
 }
 
 // ---------------------------------------------------------------------------
@@ -934,7 +953,8 @@ static int run_full3(const uint8_t* vol, int D, int H, int W, lpf_paths* p, int6
   for (const Tuned& t : p->tuned)
     if (t.H == H && t.W == W) { T = t.T; BB = t.BB; }
   Sides sd;  // one side
-  int rc = make_geometry3(D, H, W, p->host.rx, p->host.ry, p->host.rz, T, BB, sd.g[0]);
+  int rc = make_geometry3(D, H, W, p->host.rx, p->host.ry, p->host.rz, (int64_t)prog.piece_begin.size() - 1, T, BB,
+                          sd.g[0]);
   if (rc) return rc;
   const Geometry& g = sd.g[0];
   sd.n = 1;

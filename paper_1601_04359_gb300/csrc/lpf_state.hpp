@@ -64,7 +64,7 @@ struct Sides {
 };
 int make_sides(const Paths& paths, int H, int W, int T, int BB, Sides& s);
 // The same for a D x H x W volume and window (rx, ry, rz).
-int make_geometry3(int D, int H, int W, int rx, int ry, int rz, int T, int BB, Geometry& g);
+int make_geometry3(int D, int H, int W, int rx, int ry, int rz, int64_t n_pieces, int T, int BB, Geometry& g);
 
 // Walk-kernel launch shape chosen for one image size (by lpf_autotune_full).
 struct Tuned {
