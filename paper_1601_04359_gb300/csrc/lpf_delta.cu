@@ -327,10 +327,9 @@ int delta_prepare(lpf_paths* p, int H, int W) {
     // the swap-delta kernel and the annealing batch kernel stage the same
     // extended cell: allow both the opt-in maximum, and limit the cell by the
     // larger of their static shared memory
-    cudaFuncAttributes fa, fs, fp;
+    cudaFuncAttributes fa, fs;
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, delta_kernel);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fs, sa_batch_kernel_entry());
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fp, sa_persistent_kernel_entry());
     if (e == cudaSuccess) e = cudaFuncSetAttribute(delta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    optin - (int)fa.sharedSizeBytes);
     cudaFuncAttributes fz;
@@ -339,11 +338,17 @@ int delta_prepare(lpf_paths* p, int H, int W) {
                                                    optin - (int)fz.sharedSizeBytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(sa_batch_kernel_entry(), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    optin - (int)fs.sharedSizeBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(sa_persistent_kernel_entry(),
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   optin - (int)fp.sharedSizeBytes);
+    int max_static = 0;
+    for (bool lookup : {true, false}) {
+      cudaFuncAttributes fp;
+      if (e == cudaSuccess) e = cudaFuncGetAttributes(&fp, sa_persistent_kernel_entry(lookup));
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(sa_persistent_kernel_entry(lookup),
+                                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                     optin - (int)fp.sharedSizeBytes);
+      if (e == cudaSuccess) max_static = std::max(max_static, (int)fp.sharedSizeBytes);
+    }
     if (e != cudaSuccess) return set_cuda_error(e);
-    int max_static = (int)std::max(std::max(fa.sharedSizeBytes, fs.sharedSizeBytes), fp.sharedSizeBytes);
+    max_static = std::max(max_static, (int)std::max(fa.sharedSizeBytes, fs.sharedSizeBytes));
     if (int rc = swap_planes_attributes(optin, &max_static)) return rc;
     g_delta_max_smem = optin - max_static;
   }
@@ -353,13 +358,14 @@ int delta_prepare(lpf_paths* p, int H, int W) {
   if (rc) return rc;
   // one wave: SMs x resident blocks of the delta and annealing kernels for
   // this extended cell
-  // (the persistent annealer needs every chunk's block resident at once)
+  // (the persistent annealer needs every chunk's block resident at once; of its
+  // two kernels the one with lookups has more static shared memory)
   int occ_d = 0, occ_s = 0, occ_p = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_d, delta_kernel, kDeltaThreads, (size_t)ext);
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_s, sa_batch_kernel_entry(), kDeltaThreads,
                                                                          (size_t)ext);
   if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_p, sa_persistent_kernel_entry(), kDeltaThreads, (size_t)ext);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_p, sa_persistent_kernel_entry(true), kDeltaThreads, (size_t)ext);
   if (e != cudaSuccess) return set_cuda_error(e);
   const int occ = std::max(1, std::min(std::min(occ_d, occ_s), occ_p));
   // The tables stay as they are while the same cell width asks for the same
@@ -375,7 +381,7 @@ int delta_prepare(lpf_paths* p, int H, int W) {
     const size_t persist = persistent_smem_bytes(ext, p->delta.max_chunk_vecs, p->delta.max_chunk_entries);
     int occ2 = 0;
     if ((int64_t)persist <= g_delta_max_smem &&
-        (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ2, sa_persistent_kernel_entry(), kDeltaThreads,
+        (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ2, sa_persistent_kernel_entry(true), kDeltaThreads,
                                                            persist)) != cudaSuccess)
       return set_cuda_error(e);
     if (occ2 > 0 && occ2 < occ) {

@@ -333,6 +333,11 @@ static __device__ __noinline__ bool hear_messages(const unsigned long long* from
   return __all_sync(0xffffffffu, all);
 }
 
+// LOOKUP: count changes from the phase-0 counts g.z, which a run has or has not
+// from its start (as one kernel, either way carried the other's registers: the
+// walks of a 20x320 cell, window 300x9, took 93.8 us a batch, 72.5 alone; the
+// lookups at 128x128, window 64, 13.1 and 12.7).
+template <bool LOOKUP>
 __global__ void __launch_bounds__(kDeltaThreads, 3) sa_persistent_kernel(
     SaDev* __restrict__ st, uint8_t* __restrict__ cell, uint8_t* __restrict__ ext, DeltaArgs g,
     int32_t* __restrict__ pairs2, float* __restrict__ u2, int32_t* __restrict__ dcounts, float* __restrict__ partial2,
@@ -434,7 +439,7 @@ __global__ void __launch_bounds__(kDeltaThreads, 3) sa_persistent_kernel(
       u2[(size_t)(bi & 1) * k_max + k] = c.u;
     }
     *to = c;
-    if (!g.z && c.a != c.b) { delta_mark(sm, c.a, kMarkA, g); delta_mark(sm, c.b, kMarkB, g); }
+    if (!LOOKUP && c.a != c.b) { delta_mark(sm, c.a, kMarkA, g); delta_mark(sm, c.b, kMarkB, g); }
   };
   // The first candidate of every batch is drawn ahead by warp 1: after a
   // single-candidate batch both ways it can end, while the other blocks'
@@ -450,7 +455,7 @@ __global__ void __launch_bounds__(kDeltaThreads, 3) sa_persistent_kernel(
     const unsigned long long n0 = (unsigned long long)s_state.n_eval;
     const long long left = s_state.n_step - s_state.n_eval;
     const int Kv = (int)min((long long)Keff, max(0LL, left));
-    const bool fast = g.z && Keff <= kMsgCandidates;
+    const bool fast = LOOKUP && Keff <= kMsgCandidates;
     // (bar_extra > 0 only in lpf_sa_selftest_timeout: block bar_block, or
     // every block if bar_block < 0, waits for what never comes)
     const unsigned int extra = (bar_block < 0 || (int)blockIdx.x == bar_block) ? bar_extra : 0u;
@@ -474,7 +479,7 @@ __global__ void __launch_bounds__(kDeltaThreads, 3) sa_persistent_kernel(
       int32_t* dk = dcounts + (int64_t)k * 2 * g.n_canon;
       float acc = 0.0f;
       held_k = -1;
-      if (g.z) {
+      if (LOOKUP) {
         // count changes that stay in shared memory until the decision are not written out
         int32_t* out = held_ok && k == Keff - 1 ? nullptr : dk;
         if (a == b) {
@@ -632,7 +637,7 @@ __global__ void __launch_bounds__(kDeltaThreads, 3) sa_persistent_kernel(
       ct.d[mv + i] = 0;
     }
     // and the phase-0 counts follow the exchange
-    if (g.z && swap) {
+    if (LOOKUP && swap) {
       if (held_k == kstar) {
         delta_chunk_apply_held(g, last.q, v0, ct, held, held_zi, flagged ? s_maybe : nullptr);
       } else {
@@ -688,7 +693,10 @@ __global__ void build_ext_sa_kernel(const uint8_t* __restrict__ img, DeltaArgs g
 namespace lpf {
 
 const void* sa_batch_kernel_entry() { return reinterpret_cast<const void*>(&sa_batch_kernel); }
-const void* sa_persistent_kernel_entry() { return reinterpret_cast<const void*>(&sa_persistent_kernel); }
+const void* sa_persistent_kernel_entry(bool lookup) {
+  return lookup ? reinterpret_cast<const void*>(&sa_persistent_kernel<true>)
+                : reinterpret_cast<const void*>(&sa_persistent_kernel<false>);
+}
 
 constexpr int kPersistentBatches = 4096;  // batches per persistent launch (bounds one launch's duration)
 
@@ -706,7 +714,7 @@ static int launch_persistent(lpf_sa* sa, int nb, cudaStream_t s, unsigned int ba
   int k_max = sa->prm.k_max;
   void* args[] = {&sa->d_st, &sa->cell, &sa->d_ext, &sa->g, &sa->d_pairs, &sa->d_u, &sa->d_dc, &sa->d_partial,
                   &counts, &sa->d_status, &sa->d_bar, &msg, &nb, &k_max, &bar_extra, &bar_block};
-  e = cudaLaunchCooperativeKernel(sa_persistent_kernel_entry(), dim3(sa->g.n_chunks), dim3(kDeltaThreads), args,
+  e = cudaLaunchCooperativeKernel(sa_persistent_kernel_entry(sa->g.z != nullptr), dim3(sa->g.n_chunks), dim3(kDeltaThreads), args,
                                   persistent_smem(sa->g), s);
   return set_cuda_error(e);
 }
@@ -968,8 +976,8 @@ static int sa_create_lineal(uint8_t* cell_dev, int32_t H, int32_t W, lpf_paths* 
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const size_t smem = lpf::persistent_smem(sa->g);
     if (e == cudaSuccess && (int64_t)smem <= lpf::delta_max_smem())
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, lpf::sa_persistent_kernel_entry(), lpf::kDeltaThreads,
-                                                        smem);
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+          &occ, lpf::sa_persistent_kernel_entry(lpf::delta_z_bytes(paths, H, W) > 0), lpf::kDeltaThreads, smem);
     if (e != cudaSuccess) { lpf_sa_free(sa); return lpf::set_cuda_error(e); }
     // (the block-wide lookups number a chunk's vectors in 16 bits)
     sa->persistent = (coop && occ > 0 && sa->g.n_chunks <= occ * sms && sa->g.max_chunk_vecs <= 65535) ? 1 : 0;

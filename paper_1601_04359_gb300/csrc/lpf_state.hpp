@@ -167,7 +167,7 @@ void z_init_launch(const uint8_t* ext, const DeltaArgs& g, uint8_t* z, int* stat
 // The annealing batch kernel of the lineal-path objective (lpf_sa.cu), for
 // attribute and occupancy queries.
 const void* sa_batch_kernel_entry();
-const void* sa_persistent_kernel_entry();
+const void* sa_persistent_kernel_entry(bool lookup);
 // lpf_delta_swap with the error restricted to the phases in phase_mask and,
 // optionally, the walks restricted to selected start translations (sel_ext:
 // extended layout, from build_sel_ext) with descriptor = count * inv_norm
