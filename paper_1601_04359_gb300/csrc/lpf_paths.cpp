@@ -122,36 +122,37 @@ struct Walker {
 
 }  // namespace
 
-// Turn the event list into records.  At every record start the current node
-// and the live stack entries (levels 0..top-1, all ancestors of the next
-// node) are kept so that the list can be cut into independent pieces.
-static void emit_records(const std::vector<Event>& ev, Program& prog,
-                         std::vector<int64_t>& rec_word, std::vector<int64_t>& rec_pix,
-                         std::vector<int32_t>& rec_cur, std::vector<std::vector<int32_t>>& rec_stack,
-                         std::vector<uint8_t>& rec_restores) {
-  std::vector<uint32_t>& w = prog.words;
-  w.clear();
-  std::vector<int32_t> stack(kMaxStack, -1);
-  int top = 0;
-  int32_t cur = -1;
+// The records of a tree's depth-first event list.  Where a record starts, the
+// current node and the live stack entries (levels 0 .. top - 1, all ancestors of
+// the next node) are known, so that the list can be cut into independent pieces:
+// live is the push of the topmost entry, and the entry below it is that of
+// push_up.
+struct Records {
+  std::vector<int64_t> word, pix;  // of record r: word[r] .. word[r + 1], pixels before it
+  std::vector<int32_t> cur, live;
+  std::vector<int32_t> push_node, push_up;
+  Program full;
+};
+
+static void emit_records(const std::vector<Event>& ev, Records& rec) {
+  std::vector<uint32_t>& w = rec.full.words;
+  std::vector<int32_t> stack(kMaxStack, -1);  // pushes
+  int32_t cur = -1, live = -1;
   size_t i = 0;
   int64_t pix_total = 0;
   std::vector<uint32_t> pixels;
   while (i < ev.size()) {
-    rec_word.push_back((int64_t)w.size());
-    rec_pix.push_back(pix_total);
+    rec.word.push_back((int64_t)w.size());
+    rec.pix.push_back(pix_total);
     uint32_t hdr = 0;
-    bool restores = false;
     if (ev[i].kind == Event::kRestoreEv) {
       hdr |= kRestore | ((uint32_t)ev[i].a << kRlevelShift);
-      cur = stack[ev[i].a];
-      top = ev[i].a + 1;
-      restores = true;
+      live = stack[ev[i].a];
+      cur = rec.push_node[live];
       ++i;
     }
-    rec_cur.push_back(cur);
-    rec_restores.push_back(restores ? 1 : 0);
-    rec_stack.emplace_back(stack.begin(), stack.begin() + top);
+    rec.cur.push_back(cur);
+    rec.live.push_back(live);
     const size_t hdr_pos = w.size();
     w.push_back(0);  // header placeholder
     uint32_t npix = 0;
@@ -170,38 +171,30 @@ static void emit_records(const std::vector<Event>& ev, Program& prog,
       ++i;
     }
     if (i < ev.size() && ev[i].kind == Event::kPushEv) {
-      hdr |= kPush | ((uint32_t)ev[i].a << kPlevelShift);
-      stack[ev[i].a] = cur;
-      top = ev[i].a + 1;
+      const int32_t l = ev[i].a;
+      hdr |= kPush | ((uint32_t)l << kPlevelShift);
+      live = stack[l] = (int32_t)rec.push_node.size();
+      rec.push_node.push_back(cur);
+      rec.push_up.push_back(l > 0 ? stack[l - 1] : -1);
       ++i;
     }
     if (hdr & (kEmit | kPush)) w.push_back((uint32_t)level);  // skip word: the walk level until resolve_skips
     w.push_back(0u);                                            // pair count (formed when baked)
     hdr |= npix;
     w[hdr_pos] = hdr;
-    for (uint32_t q : pixels) w.push_back(q);
+    w.insert(w.end(), pixels.begin(), pixels.end());
     pix_total += npix;
   }
-  rec_word.push_back((int64_t)w.size());
-  rec_pix.push_back(pix_total);
+  rec.word.push_back((int64_t)w.size());
+  rec.pix.push_back(pix_total);
 }
 
-// The records of a tree's depth-first event list (emit_records), and its
-// program from them: cut
-// into n_pieces pieces of similar pixel count, each with a prologue that
-// rebuilds its starting state from the tree's root (no emits).
-struct Records {
-  std::vector<int64_t> word, pix;
-  std::vector<int32_t> cur;
-  std::vector<std::vector<int32_t>> stack;
-  std::vector<uint8_t> restores;
-  Program full;
-};
-
+// A tree's program from its records: cut into n_pieces pieces of similar pixel
+// count, each with a prologue that rebuilds its starting state from the tree's
+// root (no emits).
 static void make_tree_program(const Trie& t, const Records& rec, int max_level, int n_pieces, Program& tree) {
   const std::vector<int64_t>&rec_word = rec.word, &rec_pix = rec.pix;
   const std::vector<int32_t>& rec_cur = rec.cur;
-  const std::vector<std::vector<int32_t>>& rec_stack = rec.stack;
   const Program& full = rec.full;
   const int64_t nrec = (int64_t)rec_word.size() - 1;
   const int64_t total = rec_pix.back();
@@ -233,21 +226,25 @@ static void make_tree_program(const Trie& t, const Records& rec, int max_level, 
   tree.piece_pixels.clear();
   tree.stack_depth = max_level;
   tree.n_pixel_words = 0;
+  std::vector<int32_t> chain, live;
+  std::vector<uint32_t> run;
   for (size_t q = 0; q + 1 < cuts.size(); ++q) {
     const int64_t r0 = cuts[q], r1 = cuts[q + 1];
     tree.piece_begin.push_back((int64_t)tree.words.size());
     int64_t pix = 0;
     // prologue: walk root -> deepest node of the state, pushing stack entries
     {
-      const std::vector<int32_t>& live = rec_stack[r0];
+      live.clear();
+      for (int32_t x = rec.live[r0]; x >= 0; x = rec.push_up[x]) live.push_back(rec.push_node[x]);
+      std::reverse(live.begin(), live.end());
       // after a restore the state is the restored entry; otherwise the
       // current node (a descendant of every live entry)
       const int32_t target = rec_cur[r0];
-      std::vector<int32_t> chain;
+      chain.clear();
       for (int32_t x = target; x >= 0; x = t.parent[x]) chain.push_back(x);
       std::reverse(chain.begin(), chain.end());
       size_t li = 0;
-      std::vector<uint32_t> run;
+      run.clear();
       bool first = true;
       for (size_t ci = 0; ci < chain.size(); ++ci) {
         run.push_back((uint32_t)chain[ci]);
@@ -261,7 +258,7 @@ static void make_tree_program(const Trie& t, const Records& rec, int max_level, 
             ++li;
           }
           tree.words.push_back(0u);  // pair count
-          for (uint32_t n : run) tree.words.push_back(n);
+          tree.words.insert(tree.words.end(), run.begin(), run.end());
           pix += (int64_t)run.size();
           run.clear();
           first = false;
@@ -269,14 +266,10 @@ static void make_tree_program(const Trie& t, const Records& rec, int max_level, 
       }
     }
     // body: copy records r0..r1-1; the first record of piece 0 needs reset
-    for (int64_t r = r0; r < r1; ++r) {
-      const int64_t wb = rec_word[r], we = rec_word[r + 1];
-      uint32_t hdr = full.words[wb];
-      if (r == 0) hdr |= kReset;
-      tree.words.push_back(hdr);
-      for (int64_t j = wb + 1; j < we; ++j) tree.words.push_back(full.words[j]);
-      pix += rec_pix[r + 1] - rec_pix[r];
-    }
+    const size_t body = tree.words.size();
+    tree.words.insert(tree.words.end(), full.words.begin() + rec_word[r0], full.words.begin() + rec_word[r1]);
+    if (r0 == 0) tree.words[body] |= kReset;
+    pix += rec_pix[r1] - rec_pix[r0];
     tree.piece_pixels.push_back(pix);
     tree.n_pixel_words += pix;
   }
@@ -285,37 +278,32 @@ static void make_tree_program(const Trie& t, const Records& rec, int max_level, 
 
 // The plain program of one tree: the segment of every vector of orientation
 // o from scratch, in canonical order; its pixel words are the tree's nodes
-// along the segment (found by walking its oriented pixels down from root).
-static void make_plain_program(const Trie& t, const std::vector<int32_t>& cstart, const std::vector<int32_t>& clist,
-                               const std::vector<int16_t>& oseq, const std::vector<int64_t>& ptr,
-                               const std::vector<uint8_t>& orient, uint8_t o, int32_t root, int dims,
-                               Program& plain) {
+// along the segment, from the vector's node up.
+static void make_plain_program(const Trie& t, const std::vector<int64_t>& ptr, const std::vector<uint8_t>& orient,
+                               uint8_t o, Program& plain) {
   plain.words.clear();
   plain.stack_depth = 0;
   plain.n_pixel_words = 0;
-  std::vector<int32_t> chain;
   const int64_t n_canon = (int64_t)ptr.size() - 1;
+  std::vector<int32_t> node(n_canon, -1);
+  for (size_t n = 0; n < t.vec.size(); ++n)
+    if (t.vec[n] >= 0) node[t.vec[n]] = (int32_t)n;
+  int64_t n_words = 0;
+  for (int64_t c = 0; c < n_canon; ++c)
+    if (orient[c] == o) n_words += 4 + ptr[c + 1] - ptr[c];
+  plain.words.resize((size_t)n_words);
+  uint32_t* w = plain.words.data();
   for (int64_t c = 0; c < n_canon; ++c) {
     if (orient[c] != o) continue;
-    chain.clear();
-    int32_t n = root;
-    chain.push_back(n);
-    for (int64_t j = ptr[c] + 1; j < ptr[c + 1]; ++j) {
-      const int16_t x = oseq[dims * j], y = oseq[dims * j + 1], z = dims == 3 ? oseq[dims * j + 2] : 0;
-      int32_t found = -1;
-      for (int32_t k = cstart[n]; k < cstart[n + 1]; ++k) {
-        const int32_t ch = clist[k];
-        if (t.pix[3 * ch] == x && t.pix[3 * ch + 1] == y && t.pix[3 * ch + 2] == z) { found = ch; break; }
-      }
-      n = found;
-      chain.push_back(n);
-    }
-    plain.words.push_back(kReset | kEmit | (uint32_t)chain.size());
-    plain.words.push_back((uint32_t)c);
-    plain.words.push_back(0u);  // skip word (resolved to the next record)
-    plain.words.push_back(0u);  // pair count
-    for (int32_t x : chain) plain.words.push_back((uint32_t)x);
-    plain.n_pixel_words += (int64_t)chain.size();
+    const int64_t n = ptr[c + 1] - ptr[c];
+    w[0] = kReset | kEmit | (uint32_t)n;
+    w[1] = (uint32_t)c;
+    w[2] = 0u;  // skip word (resolved to the next record)
+    w[3] = 0u;  // pair count
+    w += 4 + n;
+    uint32_t* q = w;
+    for (int32_t x = node[c]; x >= 0; x = t.parent[x]) *--q = (uint32_t)x;
+    plain.n_pixel_words += n;
   }
 }
 
@@ -436,7 +424,7 @@ int build_paths_nd(int32_t rx, int32_t ry, int32_t rz, int dims, int n_pieces, P
     wk.node(root, 0);
     if (wk.max_level > kMaxStack) { err = "prefix-tree stack deeper than supported"; return -2; }
     Records rec;
-    emit_records(wk.ev, rec.full, rec.word, rec.pix, rec.cur, rec.stack, rec.restores);
+    emit_records(wk.ev, rec);
     make_tree_program(t, rec, wk.max_level, pieces_for(sub[root]), o ? p.tree_t : p.tree);
     if (dims == 2 && nn <= kFineNodes && std::max(rx, ry) <= kFineWindow) {
       const int64_t piece_nodes = std::max<int64_t>(32, (int64_t)std::max(rx, ry) + 1);
@@ -444,7 +432,7 @@ int build_paths_nd(int32_t rx, int32_t ry, int32_t rz, int dims, int n_pieces, P
                         o ? p.fine_t : p.fine);
     }
     // Plain program: every segment of the tree from scratch (Alg. 1 order).
-    make_plain_program(t, cstart, clist, oseq, p.ptr, orient, (uint8_t)o, root, dims, o ? p.plain_t : p.plain);
+    make_plain_program(t, p.ptr, orient, (uint8_t)o, o ? p.plain_t : p.plain);
     split_program(p, o ? p.plain_t : p.plain, pieces_for(sub[root]));
   }
   for (Program* prog : {&p.tree, &p.tree_t, &p.fine, &p.fine_t, &p.plain, &p.plain_t}) {
@@ -483,7 +471,8 @@ void align_program(Program& prog) {
     for (int k = record_extra_words(h); k > 0; --k) out.push_back(prog.words[i++]);
     while (out.size() % 4) out.push_back(0);
     const uint32_t n = h & kNpixMask;
-    for (uint32_t k = 0; k < n; ++k) out.push_back(prog.words[i++]);
+    out.insert(out.end(), prog.words.begin() + (std::ptrdiff_t)i, prog.words.begin() + (std::ptrdiff_t)(i + n));
+    i += n;
   }
   while (pi < prog.piece_begin.size()) new_begin[pi++] = (int64_t)out.size();
   prog.words.swap(out);
