@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(kNttThreads) s2_back_kernel(const uint32_t* __
   }
 }
 
-// The 1x1 image: S2(0) = chi (three launches and a work area took 13 us, this 5).
+// The 1x1 image: S2(0) = chi (three launches and a work area took 13 us, this 8).
 __global__ void s2_single_kernel(const uint8_t* __restrict__ img, int phase, float* __restrict__ s2) {
   *s2 = (*img != 0) == (phase != 0) ? 1.0f : 0.0f;
 }
