@@ -77,7 +77,7 @@ int layout_side(int H, int W, int rx, int ry, int T, int BB, Geometry& g, int up
 // Rows narrower than a thread's T = 8 words leave words without translations;
 // where BB bands can be folded R at a time, a tile takes R bands instead (the
 // decoding of records, most of the walk of short segments, then serves twice
-// the words: 128^3, window 16: 2.75 -> 1.98 ms).
+// the words: 128^3, window 16: 2.75 -> 1.99 ms).
 static int fold(int T, int W, int H, int BB) {
   if (T != 8) return 1;
   const int nw = (W + 31) / 32;

@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(kDeltaThreads, 3) sa_batch_kernel(
 // What bounds it: a batch is a chain of latencies -- the lookups, the messages'
 // way, the decision, its consequences -- and of the instructions of 48 warps
 // per SM in the lookups and updates.  Measured at 128x128, window 64 (a batch
-// of one): 14.0 -> 11.9 us by taking off that chain what another warp can do
+// of one): 16.3 -> 12.7 us (11.8 on another box) by taking off that chain what another warp can do
 // while the messages are on their way (the next candidate and the schedule's
 // next step for both outcomes, which vectors may hold both pixels), one word
 // instead of four per vector in the lookups, and no marks for lookups.

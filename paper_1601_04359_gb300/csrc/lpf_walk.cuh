@@ -25,7 +25,7 @@
 // own word of the staged rows, so its loads meet in a bank now and then (45e6
 // of 271e6 wavefronts), which the ALU time saved pays for (1.08e9 -> 0.70e9
 // ALU instructions).  Restoring a mask that was pushed before the re-deal ends
-// the gathered walk.  Measured: 512x512 ellipses, window 256: 2.32 -> 1.96 ms
+// the gathered walk.  Measured, kernel alone: 512x512 ellipses, window 256: 2.46 -> 2.08 ms
 // (issue slots 72 % busy: the decoding of records, 18 pixels each, is what is
 // left); 175x201 squares, whole domain: 239 -> 191 us.
 #pragma once
@@ -272,7 +272,7 @@ static __device__ __noinline__ uint2 gathered_walk(const uint4* __restrict__ pro
 // Groups of program below which a re-deal does not pay (it costs about 100
 // instructions, a group saves about 30; 6, 12 and 24 measured the same).
 constexpr uint32_t kGatherGroups = 12;
-constexpr int kMaxLive = 32;  // one mask per lane (16: 2.18 instead of 1.97 ms at 512x512, window 256)
+constexpr int kMaxLive = 32;  // one mask per lane (16: 11 % slower at 512x512, window 256)
 // Windows from which tiles empty out enough to re-deal (kernels of their own:
 // their code costs a launch 4 us and a walk that never re-deals 3 to 6 %); at
 // window 128 a third of the walk is gathered.  Images walked one at a time
@@ -280,7 +280,7 @@ constexpr int kMaxLive = 32;  // one mask per lane (16: 2.18 instead of 1.97 ms 
 // took 88 instead of 73 us) and two units per warp slot (112x93, whole
 // domain: 93 instead of 87 us); at window 119 (239x230) it is a loss of 2 %,
 // at 143 (210x286) a gain of a third; batches, whose images share a kernel, pay
-// from windows of 120 (96 and less: 3 to 5 % slower).
+// from windows of 120 (96 and less: 3 to 5 % slower).  Volumes do not re-deal.
 constexpr int kGatherWindow = 128;
 constexpr int kGatherWindowBatch = 120;
 
